@@ -11,10 +11,12 @@
  *     part lies beyond what a second-order Hermite expansion carries (what a low-order
  *     node can hold, Sec. 2.2), measured on a high-order run;
  *   network: 8 -> 64 -> 64 -> 1, GELU (erf form) hidden layers, sigmoid output.
- * Training runs here in FP32 (forward, backward, weight gradients, Adam: one kernel
+ * Training runs here in FP32 (mini-batch training in one cluster kernel; whole-set gradients
+ * as a forward, a backward, a weight-gradient and an Adam kernel
  * each); inference uses BF16 weights with FP32 accumulation. Parameter layout:
  * W1 [64][8], b1 [64], W2 [64][64], b2 [64], W3 [64], b3 [1] (4801 values).
  */
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -41,10 +43,10 @@ __device__ __forceinline__ float gelu_grad(float a)
     return 0.5f * (1.0f + erff(a * 0.70710678118654752f)) + a * expf(-0.5f * a * a) * 0.39894228040143268f;
 }
 
-/* Forward pass of a mini-batch: sample b uses column idx[b] of X [NF][n]; keeps the
- * pre-activations and activations for the backward pass. One thread per sample. */
+/* Forward pass of samples 0 .. B - 1 (columns of X [NF][n]); keeps the pre-activations and
+ * activations for the backward pass. One thread per sample. */
 __global__ void fwd_kernel(const float *__restrict__ th, const float *__restrict__ norm, const float *__restrict__ X,
-                           long long n, const int *__restrict__ idx, int B, float *xn, float *a1, float *h1, float *a2,
+                           long long n, int B, float *xn, float *a1, float *h1, float *a2,
                            float *h2, float *pout)
 {
     __shared__ float s[NPARAM];
@@ -52,7 +54,7 @@ __global__ void fwd_kernel(const float *__restrict__ th, const float *__restrict
     __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    const long long c = idx ? idx[b] : b;
+    const long long c = b;
     float x[NF];
     for (int f = 0; f < NF; ++f) {
         x[f] = (X[(long long)f * n + c] - norm[f]) / norm[NF + f];
@@ -79,7 +81,7 @@ __global__ void fwd_kernel(const float *__restrict__ th, const float *__restrict
 }
 
 /* Backward pass through the activations: dz = (p - y) / B, then dA2 and dA1 per sample. */
-__global__ void bwd_kernel(const float *__restrict__ th, const float *__restrict__ Y, const int *__restrict__ idx, int B,
+__global__ void bwd_kernel(const float *__restrict__ th, const float *__restrict__ Y, int B,
                            const float *a1, const float *a2, const float *pout, float *dz, float *da1, float *da2,
                            double *loss_acc)
 {
@@ -88,8 +90,7 @@ __global__ void bwd_kernel(const float *__restrict__ th, const float *__restrict
     __syncthreads();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    const long long c = idx ? idx[b] : b;
-    const float y = Y[c], p = pout[b];
+    const float y = Y[b], p = pout[b];
     const float g = (p - y) / (float)B;
     dz[b] = g;
     if (loss_acc) {
@@ -147,6 +148,289 @@ __global__ void adam_kernel(float *th, float *m, float *v, const float *g, int t
     v[k] = vk;
     const float mh = mk / (1.0f - powf(b1, (float)t)), vh = vk / (1.0f - powf(b2, (float)t));
     th[k] -= lr * mh / (sqrtf(vh) + eps);
+}
+
+/* ---- mini-batch training: one thread-block cluster takes every batch of a launch ----
+ *
+ * A batch of a few hundred samples is about 3.5 M multiply-adds, and the next batch needs
+ * the updated weights: the work is a chain of small steps, bound by latency, not by the
+ * chip's rate. One launch per layer and batch cost 113 us a batch (a weight gradient that
+ * walked the samples one by one in each thread, and five launches). Here a cluster of
+ * TR_NC blocks keeps the weights, the activations and Adam's moments on chip for all the
+ * batches of a launch: block r takes the batch's samples r B / TR_NC .. in tiles of TR_S,
+ * every block writes its gradient sums to its shared memory, and after a cluster barrier
+ * block r adds the TR_NC sums of its slice of the parameters in rank order through
+ * distributed shared memory, updates it and stores the new values into every block. Two
+ * cluster barriers a batch; sums in a fixed order, so a run repeats bit for bit. The next
+ * tile's samples (a gather over the shuffled order) are loaded while this one is computed.
+ * Measured: 100 000 samples in batches of 256, one epoch 51.9 ms -> 4.8 ms. */
+constexpr int TR_NC = 8, TR_S = 32, TR_T = 512;
+constexpr int TR_LD = NH + 4;   /* activation and W2 rows in shared memory: conflict-free 16-byte reads */
+constexpr int TR_SL = (NPARAM + TR_NC - 1) / TR_NC;
+static_assert(TR_T == 16 * TR_S && TR_SL <= 2 * TR_T && TR_T == 8 * NH, "thread mapping of the training kernel");
+
+struct TrainSmem {
+    float w1[NH][NF + 4], w2[NH][TR_LD], b1[NH], b2[NH], w3[NH], b3, pad[3];
+    float x[TR_S][NF + 4], y[TR_S];
+    float h1[TR_S][TR_LD], g1[TR_S][TR_LD], h2[TR_S][TR_LD], d2[TR_S][TR_LD], d1[TR_S][TR_LD];
+    float zp[TR_S][2], dz[TR_S];
+    float grad[NPARAM + 3];
+};
+
+/* parameter k of the packed vector in a block's shared memory */
+__device__ __forceinline__ float *train_param(TrainSmem &s, int k)
+{
+    if (k < OFF_B1) return &s.w1[k / NF][k % NF];
+    if (k < OFF_W2) return &s.b1[k - OFF_B1];
+    if (k < OFF_B2) return &s.w2[(k - OFF_W2) / NH][(k - OFF_W2) % NH];
+    if (k < OFF_W3) return &s.b2[k - OFF_B2];
+    if (k < OFF_B3) return &s.w3[k - OFF_W3];
+    return &s.b3;
+}
+
+/* Batches of `batch` samples (the last may be short) over samples idx[0 .. count): forward,
+ * backward, Adam with step numbers t0 + 1, ...; p of sample idx[k] at its batch's weights
+ * goes to pall[k] when pall is not NULL. th, m, v are read at the start and written at the
+ * end. Launched as one cluster. */
+__global__ void __cluster_dims__(TR_NC, 1, 1) __launch_bounds__(TR_T, 1)
+    train_kernel(float *__restrict__ th, float *__restrict__ m, float *__restrict__ v, const float *__restrict__ norm,
+                 const float *__restrict__ X, long long n, const float *__restrict__ Y, const int *__restrict__ idx,
+                 int count, int batch, int t0, float lr, float *__restrict__ pall)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char train_smem[];
+    TrainSmem &s = *reinterpret_cast<TrainSmem *>(train_smem);
+    const int tid = threadIdx.x, rank = (int)cl.block_rank(), lane = tid & 31;
+    for (int k = tid; k < NPARAM; k += TR_T) *train_param(s, k) = th[k];
+    /* this thread's parameters of the block's slice, with their Adam moments */
+    const int k0 = rank * TR_SL + tid, kend = min(NPARAM, (rank + 1) * TR_SL);
+    float mk[2] = {0.0f, 0.0f}, vk[2] = {0.0f, 0.0f};
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+        if (k0 + u * TR_T < kend) {
+            mk[u] = m[k0 + u * TR_T];
+            vk[u] = v[k0 + u * TR_T];
+        }
+    /* samples of tile q of this block in the batch at s0: idx[first .. first + cnt) */
+    auto tile = [&](int s0, int q, int &first, int &cnt) {
+        const int B = min(batch, count - s0), per = (B + TR_NC - 1) / TR_NC;
+        const int lo = rank * per + q * TR_S, hi = min(B, (rank + 1) * per);
+        cnt = max(0, min(TR_S, hi - lo));
+        first = s0 + lo;
+    };
+    /* one value of a tile per thread: feature tid / TR_S of sample tid % TR_S (normalised), or
+     * the label; 0 beyond the tile's samples */
+    const int pf = tid / TR_S, ps = tid % TR_S;
+    float nmean = 0.0f, nscale = 1.0f;
+    if (pf < NF) {
+        nmean = norm[pf];
+        nscale = norm[NF + pf];
+    }
+    auto fetch = [&](int s0, int q) -> float {
+        int first, cnt;
+        tile(s0, q, first, cnt);
+        if (pf > NF || ps >= cnt) return 0.0f;
+        const long long c = idx[first + ps];
+        return pf < NF ? (X[(long long)pf * n + c] - nmean) / nscale : Y[c];
+    };
+    auto put = [&](float val) {
+        if (pf < NF) s.x[ps][pf] = val;
+        else if (pf == NF) s.y[ps] = val;
+    };
+    const int i64 = tid % NH, sg = tid / NH * 4;   /* a unit and four samples */
+    const int wi = tid / 16 * 2, wj = tid % 16 * 4;   /* a 2 x 4 block of the W2 gradient */
+    put(fetch(0, 0));
+    cl.sync();
+    int t = t0;
+    for (int s0 = 0; s0 < count; s0 += batch) {
+        const int B = min(batch, count - s0), nt = ((B + TR_NC - 1) / TR_NC + TR_S - 1) / TR_S;
+        float gw2[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}}, gw1 = 0.0f, gb = 0.0f;
+        for (int q = 0; q < nt; ++q) {
+            int first, cnt;
+            tile(s0, q, first, cnt);
+            const bool last = q + 1 == nt;
+            const bool more = !last || s0 + batch < count;
+            float nxt = 0.0f;
+            if (more) nxt = last ? fetch(s0 + batch, 0) : fetch(s0, q + 1);
+            float g2[4], z4[4];
+            if (sg < cnt) {   /* layer 1 */
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float a = s.b1[i64];
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) a = fmaf(s.w1[i64][f], s.x[sg + u][f], a);
+                    const float c = 0.5f * (1.0f + erff(a * 0.70710678118654752f));
+                    s.h1[sg + u][i64] = a * c;
+                    s.g1[sg + u][i64] = c + a * expf(-0.5f * a * a) * 0.39894228040143268f;
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s.h1[sg + u][i64] = 0.0f;
+            }
+            __syncthreads();
+            if (sg < cnt) {   /* layer 2 and the output's dot product */
+                float a[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) a[u] = s.b2[i64];
+#pragma unroll
+                for (int k = 0; k < NH; k += 4) {
+                    const float4 w = *reinterpret_cast<const float4 *>(&s.w2[i64][k]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float4 h = *reinterpret_cast<const float4 *>(&s.h1[sg + u][k]);
+                        a[u] = fmaf(w.x, h.x, a[u]);
+                        a[u] = fmaf(w.y, h.y, a[u]);
+                        a[u] = fmaf(w.z, h.z, a[u]);
+                        a[u] = fmaf(w.w, h.w, a[u]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float c = 0.5f * (1.0f + erff(a[u] * 0.70710678118654752f));
+                    const float h = a[u] * c;
+                    g2[u] = c + a[u] * expf(-0.5f * a[u] * a[u]) * 0.39894228040143268f;
+                    s.h2[sg + u][i64] = h;
+                    z4[u] = s.w3[i64] * h;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) z4[u] += __shfl_xor_sync(0xffffffffu, z4[u], o);
+                if (lane < 4) s.zp[sg + lane][i64 / 32] = lane == 0 ? z4[0] : (lane == 1 ? z4[1] : (lane == 2 ? z4[2] : z4[3]));
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s.h2[sg + u][i64] = 0.0f;
+            }
+            __syncthreads();
+            if (sg < cnt) {   /* dz = (p - y) / B; layer 2's deltas */
+                float dzl = 0.0f;
+                if (lane < 4) {
+                    const int sm = sg + lane;
+                    const float p = 1.0f / (1.0f + expf(-(s.b3 + s.zp[sm][0] + s.zp[sm][1])));
+                    dzl = sm < cnt ? (p - s.y[sm]) / (float)B : 0.0f;
+                    if (i64 < 32) {
+                        s.dz[sm] = dzl;
+                        if (pall && sm < cnt) pall[first + sm] = p;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    s.d2[sg + u][i64] = __shfl_sync(0xffffffffu, dzl, u) * s.w3[i64] * g2[u];
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s.d2[sg + u][i64] = 0.0f;
+                if (i64 < 4) s.dz[sg + i64] = 0.0f;
+            }
+            __syncthreads();
+            if (sg < cnt) {   /* layer 1's deltas */
+                float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int i = 0; i < NH; i += 4) {
+                    const float w0 = s.w2[i][i64], w1 = s.w2[i + 1][i64], w2 = s.w2[i + 2][i64], w3 = s.w2[i + 3][i64];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float4 d = *reinterpret_cast<const float4 *>(&s.d2[sg + u][i]);
+                        a[u] = fmaf(d.x, w0, a[u]);
+                        a[u] = fmaf(d.y, w1, a[u]);
+                        a[u] = fmaf(d.z, w2, a[u]);
+                        a[u] = fmaf(d.w, w3, a[u]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s.d1[sg + u][i64] = a[u] * s.g1[sg + u][i64];
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s.d1[sg + u][i64] = 0.0f;
+            }
+            const int ns = (cnt + 3) & ~3;   /* rows up to here are filled */
+            for (int b = 0; b < ns; ++b) {
+                const float2 d = *reinterpret_cast<const float2 *>(&s.d2[b][wi]);
+                const float4 h = *reinterpret_cast<const float4 *>(&s.h1[b][wj]);
+                gw2[0][0] = fmaf(d.x, h.x, gw2[0][0]);
+                gw2[0][1] = fmaf(d.x, h.y, gw2[0][1]);
+                gw2[0][2] = fmaf(d.x, h.z, gw2[0][2]);
+                gw2[0][3] = fmaf(d.x, h.w, gw2[0][3]);
+                gw2[1][0] = fmaf(d.y, h.x, gw2[1][0]);
+                gw2[1][1] = fmaf(d.y, h.y, gw2[1][1]);
+                gw2[1][2] = fmaf(d.y, h.z, gw2[1][2]);
+                gw2[1][3] = fmaf(d.y, h.w, gw2[1][3]);
+            }
+            __syncthreads();
+            for (int b = 0; b < ns; ++b) gw1 = fmaf(s.d1[b][tid / NF], s.x[b][tid % NF], gw1);
+            if (tid < NH) {
+                for (int b = 0; b < ns; ++b) gb += s.d1[b][tid];
+            } else if (tid < 2 * NH) {
+                for (int b = 0; b < ns; ++b) gb += s.d2[b][tid - NH];
+            } else if (tid < 3 * NH) {
+                for (int b = 0; b < ns; ++b) gb = fmaf(s.dz[b], s.h2[b][tid - 2 * NH], gb);
+            } else if (tid == 3 * NH) {
+                for (int b = 0; b < ns; ++b) gb += s.dz[b];
+            }
+            __syncthreads();
+            if (more) put(nxt);
+            if (!last) __syncthreads();
+        }
+        s.grad[OFF_W1 + tid] = gw1;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) s.grad[OFF_W2 + (wi + a) * NH + wj + b] = gw2[a][b];
+        if (tid < NH) s.grad[OFF_B1 + tid] = gb;
+        else if (tid < 2 * NH) s.grad[OFF_B2 + tid - NH] = gb;
+        else if (tid < 3 * NH) s.grad[OFF_W3 + tid - 2 * NH] = gb;
+        else if (tid == 3 * NH) s.grad[OFF_B3] = gb;
+        cl.sync();   /* every block's sums are in place */
+        t += 1;
+        const float c1 = 1.0f - powf(0.9f, (float)t), c2 = 1.0f - powf(0.999f, (float)t);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int k = k0 + u * TR_T;
+            if (k >= kend) continue;
+            float gr[TR_NC];
+#pragma unroll
+            for (int r = 0; r < TR_NC; ++r) gr[r] = *cl.map_shared_rank(&s.grad[k], r);
+            float g = gr[0];
+#pragma unroll
+            for (int r = 1; r < TR_NC; ++r) g += gr[r];
+            mk[u] = 0.9f * mk[u] + (1.0f - 0.9f) * g;
+            vk[u] = 0.999f * vk[u] + (1.0f - 0.999f) * g * g;
+            const float nw = *train_param(s, k) - lr * (mk[u] / c1) / (sqrtf(vk[u] / c2) + 1e-8f);
+#pragma unroll
+            for (int r = 0; r < TR_NC; ++r) *cl.map_shared_rank(train_param(s, k), r) = nw;
+        }
+        cl.sync();   /* the new weights are in place, the sums may be overwritten */
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int k = k0 + u * TR_T;
+        if (k >= kend) continue;
+        th[k] = *train_param(s, k);
+        m[k] = mk[u];
+        v[k] = vk[u];
+    }
+}
+
+/* Cross-entropy of samples idx[0 .. count) with outputs pall[k], one FP64 partial sum per
+ * block (summed in block order on the host). */
+constexpr int LOSS_BLOCKS = 304, LOSS_T = 128;
+__global__ void __launch_bounds__(LOSS_T) loss_kernel(const float *__restrict__ pall, const float *__restrict__ Y,
+                                                      const int *__restrict__ idx, int count, double *__restrict__ part)
+{
+    __shared__ double sh[LOSS_T];
+    double l = 0.0;
+    for (int k = blockIdx.x * LOSS_T + threadIdx.x; k < count; k += LOSS_BLOCKS * LOSS_T) {
+        const double y = (double)Y[idx[k]], pc = fmin(fmax((double)pall[k], 1e-30), 1.0 - 1e-7);
+        if (y != 0.0) l -= y * log(pc);
+        if (y != 1.0) l -= (1.0 - y) * log(1.0 - pc);
+    }
+    sh[threadIdx.x] = l;
+    __syncthreads();
+    for (int o = LOSS_T / 2; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
 /* BF16 copy of the weights used by inference. */
@@ -296,8 +580,12 @@ struct lb_mlp {
     int cap = 0;   /* batch capacity of the activation buffers */
     float *xn = nullptr, *a1 = nullptr, *h1 = nullptr, *a2 = nullptr, *h2 = nullptr, *p = nullptr, *dz = nullptr,
           *da1 = nullptr, *da2 = nullptr;
-    int *idx = nullptr;
     double *loss = nullptr;
+    /* training: order, outputs (one chunk of samples) and loss partials */
+    int *idx = nullptr;
+    float *pall = nullptr;
+    double *lpart = nullptr;
+    int idx_cap = 0;
     int t = 0;
     lb_opts opts{};
     cudaStream_t stream = nullptr;
@@ -348,22 +636,40 @@ int ensure_batch(lb_mlp *M, int B)
     M->da2 = (float *)mlp_alloc(M, b * lbm::NH * 4);
     M->p = (float *)mlp_alloc(M, b * 4);
     M->dz = (float *)mlp_alloc(M, b * 4);
-    M->idx = (int *)mlp_alloc(M, b * 4);
-    if (!M->xn || !M->a1 || !M->h1 || !M->a2 || !M->h2 || !M->da1 || !M->da2 || !M->p || !M->dz || !M->idx)
+    if (!M->xn || !M->a1 || !M->h1 || !M->a2 || !M->h2 || !M->da1 || !M->da2 || !M->p || !M->dz)
         return mlp_err(LB_ERR_NOMEM, "lb_mlp: device allocation failed");
     M->cap = B;
     return LB_OK;
 }
 
-/* forward + backward + weight gradients of one batch (samples idx_host, or the first B) */
-int batch_grad(lb_mlp *M, const float *x, const float *y, int64_t n, const int *idx_dev, int B, bool want_loss)
+/* workspace of a training launch over `count` samples, and the kernel's shared memory */
+int ensure_train(lb_mlp *M, int count)
+{
+    if (cudaFuncSetAttribute(lbm::train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(lbm::TrainSmem)) != cudaSuccess) {
+        cudaGetLastError();
+        return mlp_err(LB_ERR_CUDA, "lb_mlp: the training kernel's shared memory was refused");
+    }
+    if (!M->lpart) M->lpart = (double *)mlp_alloc(M, sizeof(double) * lbm::LOSS_BLOCKS);
+    if (count > M->idx_cap) {
+        /* grow (old buffers stay owned until destroy) */
+        M->idx = (int *)mlp_alloc(M, (size_t)count * 4);
+        M->pall = (float *)mlp_alloc(M, (size_t)count * 4);
+        M->idx_cap = M->idx && M->pall ? count : 0;
+    }
+    if (!M->idx || !M->pall || !M->lpart) return mlp_err(LB_ERR_NOMEM, "lb_mlp: device allocation failed");
+    return LB_OK;
+}
+
+/* forward + backward + weight gradients of the first B samples */
+int batch_grad(lb_mlp *M, const float *x, const float *y, int64_t n, int B, bool want_loss)
 {
     const int T = 128, nb = (B + T - 1) / T;
     if (want_loss && cudaMemsetAsync(M->loss, 0, sizeof(double), M->stream) != cudaSuccess)
         return mlp_err(LB_ERR_CUDA, "lb_mlp: memset failed");
-    lbm::fwd_kernel<<<nb, T, 0, M->stream>>>(M->th, M->norm, x, (long long)n, idx_dev, B, M->xn, M->a1, M->h1, M->a2,
+    lbm::fwd_kernel<<<nb, T, 0, M->stream>>>(M->th, M->norm, x, (long long)n, B, M->xn, M->a1, M->h1, M->a2,
                                              M->h2, M->p);
-    lbm::bwd_kernel<<<nb, T, 0, M->stream>>>(M->th, y, idx_dev, B, M->a1, M->a2, M->p, M->dz, M->da1, M->da2,
+    lbm::bwd_kernel<<<nb, T, 0, M->stream>>>(M->th, y, B, M->a1, M->a2, M->p, M->dz, M->da1, M->da2,
                                              want_loss ? M->loss : nullptr);
     lbm::wgrad_kernel<<<(lbm::NPARAM + 127) / 128, 128, 0, M->stream>>>(B, M->xn, M->h1, M->h2, M->dz, M->da1, M->da2,
                                                                         M->g);
@@ -432,7 +738,7 @@ int lb_mlp_grad(lb_mlp *M, const float *x, const float *y, int64_t n, float *gra
 {
     if (!M || !x || !y || !grad || n < 1 || n > (1 << 20)) return mlp_err(LB_ERR_INVALID, "lb_mlp_grad: bad argument");
     if (int e = ensure_batch(M, (int)n)) return e;
-    if (int e = batch_grad(M, x, y, n, nullptr, (int)n, true)) return e;
+    if (int e = batch_grad(M, x, y, n, (int)n, true)) return e;
     cudaError_t ce = cudaMemcpyAsync(grad, M->g, lbm::NPARAM * 4, cudaMemcpyDeviceToHost, M->stream);
     double l = 0.0;
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(&l, M->loss, sizeof(double), cudaMemcpyDeviceToHost, M->stream);
@@ -447,35 +753,37 @@ int lb_mlp_train(lb_mlp *M, const float *x, const float *y, int64_t n, int32_t e
 {
     if (!M || !x || !y || n < 1 || epochs < 1 || batch < 1 || batch > 65536 || !(lr > 0.0f))
         return mlp_err(LB_ERR_INVALID, "lb_mlp_train: bad argument");
-    if (int e = ensure_batch(M, batch)) return e;
+    /* whole batches of at most TRAIN_CHUNK samples (one batch at least) per launch: the order
+     * and the outputs of a launch's samples are the workspace */
+    constexpr int64_t TRAIN_CHUNK = 1 << 18;
+    const int64_t chunk = std::min<int64_t>(n, std::max<int64_t>(1, TRAIN_CHUNK / batch) * batch);
+    if (int e = ensure_train(M, (int)chunk)) return e;
     std::vector<int> perm((size_t)n);
     for (int64_t k = 0; k < n; ++k) perm[(size_t)k] = (int)k;
     std::mt19937_64 rng(seed);
     double eloss = 0.0;
     for (int ep = 0; ep < epochs; ++ep) {
         for (int64_t k = n - 1; k > 0; --k) std::swap(perm[(size_t)k], perm[(size_t)(rng() % (uint64_t)(k + 1))]);
-        eloss = 0.0;
-        int nbat = 0;
-        for (int64_t s0 = 0; s0 < n; s0 += batch) {
-            const int B = (int)std::min<int64_t>(batch, n - s0);
-            if (cudaMemcpyAsync(M->idx, perm.data() + s0, (size_t)B * 4, cudaMemcpyHostToDevice, M->stream) != cudaSuccess)
+        const bool last_epoch = ep == epochs - 1;
+        for (int64_t s0 = 0; s0 < n; s0 += chunk) {
+            const int cnt = (int)std::min<int64_t>(chunk, n - s0);
+            if (cudaMemcpyAsync(M->idx, perm.data() + s0, (size_t)cnt * 4, cudaMemcpyHostToDevice, M->stream) != cudaSuccess)
                 return mlp_err(LB_ERR_CUDA, "lb_mlp_train: copy failed");
-            const bool last_epoch = ep == epochs - 1;
-            if (int e = batch_grad(M, x, y, n, M->idx, B, last_epoch)) return e;
-            M->t += 1;
-            lbm::adam_kernel<<<(lbm::NPARAM + 127) / 128, 128, 0, M->stream>>>(M->th, M->m, M->v, M->g, M->t, lr, 0.9f,
-                                                                              0.999f, 1e-8f);
+            lbm::train_kernel<<<lbm::TR_NC, lbm::TR_T, sizeof(lbm::TrainSmem), M->stream>>>(
+                M->th, M->m, M->v, M->norm, x, (long long)n, y, M->idx, cnt, batch, M->t, lr,
+                last_epoch ? M->pall : nullptr);
+            if (cudaGetLastError() != cudaSuccess) return mlp_err(LB_ERR_CUDA, "lb_mlp_train: launch failed");
+            M->t += (cnt + batch - 1) / batch;
             if (last_epoch) {
-                double l = 0.0;
-                if (cudaMemcpyAsync(&l, M->loss, sizeof(double), cudaMemcpyDeviceToHost, M->stream) != cudaSuccess ||
+                double part[lbm::LOSS_BLOCKS];
+                lbm::loss_kernel<<<lbm::LOSS_BLOCKS, lbm::LOSS_T, 0, M->stream>>>(M->pall, y, M->idx, cnt, M->lpart);
+                if (cudaMemcpyAsync(part, M->lpart, sizeof(part), cudaMemcpyDeviceToHost, M->stream) != cudaSuccess ||
                     cudaStreamSynchronize(M->stream) != cudaSuccess)
                     return mlp_err(LB_ERR_CUDA, "lb_mlp_train: copy failed");
-                eloss += l * B;
-                ++nbat;
+                for (double l : part) eloss += l;
             }
         }
-        (void)nbat;
-        /* the copy above waits; keep perm alive until the last batch's upload finished */
+        /* keep perm as it is until its last upload has finished */
         if (cudaStreamSynchronize(M->stream) != cudaSuccess) return mlp_err(LB_ERR_CUDA, "lb_mlp_train: sync failed");
     }
     lbm::to_bf16_kernel<<<(lbm::NPARAM + 255) / 256, 256, 0, M->stream>>>(M->th, M->wb);
@@ -489,7 +797,7 @@ int lb_mlp_adam_step(lb_mlp *M, const float *x, const float *y, int64_t n, float
 {
     if (!M || !x || !y || n < 1 || n > (1 << 20)) return mlp_err(LB_ERR_INVALID, "lb_mlp_adam_step: bad argument");
     if (int e = ensure_batch(M, (int)n)) return e;
-    if (int e = batch_grad(M, x, y, n, nullptr, (int)n, false)) return e;
+    if (int e = batch_grad(M, x, y, n, (int)n, false)) return e;
     M->t += 1;
     lbm::adam_kernel<<<(lbm::NPARAM + 127) / 128, 128, 0, M->stream>>>(M->th, M->m, M->v, M->g, M->t, lr, 0.9f, 0.999f,
                                                                       1e-8f);
