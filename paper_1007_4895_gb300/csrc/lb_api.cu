@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -128,6 +129,15 @@ struct lb_ctx {
     int2 *d_rdesc = nullptr;
     uint32_t *d_rctr = nullptr;
     std::unique_ptr<lbk::RingTab> rtab;
+    /* resident steps (lb_resident.cuh): several steps per launch, the state in shared memory */
+    bool res_on = false, res_pair = false;
+    lbk::ResPlan rplan;
+    void *d_rplan = nullptr, *d_rpar = nullptr;
+    uint32_t *d_roff = nullptr;
+    lbk::RingTab *d_rtab = nullptr;
+    size_t rplan_cap = 0;
+    std::tuple<int, int, int, int, int, uint64_t> res_key{};
+    bool res_variant = false;       /* the layout in use stands in for the resident steps */
     uint32_t dcol_hash = 0;         /* FNV-1a of those deltas (0: one reference density) */
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     /* learned placement */
@@ -743,15 +753,220 @@ bool variant_available(const lb_ctx *c, int v)
     return v >= 0 && v < LB_NUM_VARIANTS;
 }
 
+/* ------------------------------------------------------- resident steps -- */
+
+/* Lattices the resident steps take: the TVD scheme with mode-B views, periodic x, every
+ * row in one set across x, one reference density; the layout not forced. */
+bool resident_candidate(const lb_ctx *c)
+{
+    if (c->opts.variant >= 0 || c->opts.scheme != LB_SCHEME_TVD || c->opts.iface != LB_IFACE_HERMITE || c->d_dcol)
+        return false;
+    if (c->walls[2].kind != LB_WALL_PERIODIC || c->ny > 0xfff0 || c->nx > 0x7fff) return false;
+    for (int j = 0; j < c->ny; ++j)
+        for (int tx = 1; tx < c->ntx; ++tx)
+            if ((c->tmap[(size_t)j * c->ntx + tx] ^ c->tmap[(size_t)j * c->ntx]) & LB_TILE_HIGH) return false;
+    return true;
+}
+
+lbk::ResLattice resident_lattice(const lb_ctx *c, uint64_t group)
+{
+    lbk::ResLattice l;
+    l.W = c->nx;
+    l.ny = c->ny;
+    l.q[0] = c->q[0];
+    l.q[1] = c->q[1];
+    l.periodic_y = c->walls[0].kind == LB_WALL_PERIODIC;
+    l.wall[0] = c->walls[0].kind == LB_WALL_DIFFUSE;
+    l.wall[1] = c->walls[1].kind == LB_WALL_DIFFUSE;
+    l.flags = c->tmap.data();
+    l.ntx = c->ntx;
+    l.group = group;
+    return l;
+}
+
+/* equal for lattices whose population constants are equal bit for bit (without the force
+ * and the row step, which a block takes per lattice) */
+uint64_t resident_group(const lb_ctx *c, bool pair)
+{
+    uint64_t h = 1469598103934665603ull;
+    auto mix = [&](const void *p, size_t n) {
+        for (size_t k = 0; k < n; ++k) h = (h ^ static_cast<const unsigned char *>(p)[k]) * 1099511628211ull;
+    };
+    if (pair) {
+        for (int s = 0; s < 2; ++s)
+            for (int a = 0; a < c->q[s]; ++a) {
+                lbk::RingPop r = c->rtab->pop[s][a];
+                r.gxi2 = make_float2(0.0f, 0.0f);
+                r.ystep = 0;
+                mix(&r, sizeof(r));
+            }
+    } else {
+        SetConst<double> k;
+        for (int s = 0; s < 2; ++s) {
+            std::memset(&k, 0, sizeof(k));
+            fill_set(c, s, k);
+            mix(&k, sizeof(k));
+        }
+    }
+    return h ? h : 1u;
+}
+
+/* device copies of a plan (grown as needed), of the two launch parameter sets and of the
+ * constants */
+template <typename R>
+int resident_upload_t(lb_ctx *c)
+{
+    const size_t pb = (c->rplan.blob.size() + 255) / 256 * 256, ob = c->rplan.off.size() * sizeof(uint32_t);
+    if (pb + ob > c->rplan_cap) {
+        const size_t cap = std::max(pb + ob, 2 * c->rplan_cap);
+        void *d = own(c, cap);
+        if (!d) return fail(LB_ERR_NOMEM, "device allocation failed");
+        c->d_rplan = d;
+        c->rplan_cap = cap;
+    }
+    c->d_roff = reinterpret_cast<uint32_t *>(static_cast<char *>(c->d_rplan) + pb);
+    if (!c->d_rpar) {
+        void *d = own(c, 2 * sizeof(StepParams<R>));
+        if (!d) return fail(LB_ERR_NOMEM, "device allocation failed");
+        c->d_rpar = d;
+    }
+    StepParams<R> p[2] = {make_params<R>(c, 0, 1, c->t + c->dt), make_params<R>(c, 1, 0, c->t + c->dt)};
+    cudaError_t e = cudaMemcpyAsync(c->d_rpar, p, sizeof(p), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->d_rplan, c->rplan.blob.data(), c->rplan.blob.size(), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_roff, c->rplan.off.data(), ob, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && c->res_pair) {
+        if (!c->d_rtab) {
+            c->d_rtab = static_cast<lbk::RingTab *>(own(c, sizeof(lbk::RingTab)));
+            if (!c->d_rtab) return fail(LB_ERR_NOMEM, "device allocation failed");
+        }
+        e = cudaMemcpyAsync(c->d_rtab, c->rtab.get(), sizeof(lbk::RingTab), cudaMemcpyHostToDevice, c->stream);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    return cuda_check(c, e, "resident plan upload");
+}
+int resident_upload(lb_ctx *c) { return use_f64(c) ? resident_upload_t<double>(c) : resident_upload_t<float>(c); }
+
+/* n <= RES_OSC steps with oscillating walls, any n with steady ones; advance = 0: the
+ * level is left as it is */
+template <typename R>
+int resident_steps_t(lb_ctx *c, int n, int advance)
+{
+    lbk::ResOsc<R> osc;
+    osc.n = 0;
+    if (c->walls[0].omega > 0.0 || c->walls[1].omega > 0.0) {
+        osc.n = n;
+        double t = c->t;
+        for (int k = 0; k < n; ++k) {
+            t += c->dt;
+            const StepParams<R> p = make_params<R>(c, 0, 1, t);
+            for (int w = 0; w < 2; ++w) {
+                osc.v[k][w][0] = p.uw_x[w];
+                osc.v[k][w][1] = p.uw_y[w];
+                for (int s = 0; s < 2; ++s) {
+                    osc.v[k][w][2 + s] = p.kdiff[s][w];
+                    osc.v[k][w][4 + s] = p.kout[s][w];
+                }
+            }
+        }
+    }
+    const bool force = c->opts.gx != 0.0 || c->opts.gy != 0.0;
+    if (lbk::launch_resident(c->store, c->res_pair, force, c->rplan, c->d_rplan, c->d_roff, c->d_rpar, c->d_rtab, n, c->cur,
+                             (uint32_t)c->step, advance, c->d_squeue, &osc, 1, c->stream) != 0) {
+        cudaGetLastError();
+        c->status = LB_ERR_CUDA;
+        return fail(LB_ERR_CUDA, "resident steps: launch failed");
+    }
+    return launch_check(c, "resident steps");
+}
+int resident_steps(lb_ctx *c, int n, int advance)
+{
+    return use_f64(c) ? resident_steps_t<double>(c, n, advance) : resident_steps_t<float>(c, n, advance);
+}
+
+std::mutex g_tune_mu;   /* the tuners' caches */
+std::map<std::tuple<int, int, int, int, int, uint64_t>, int> g_res_tune;   /* cluster size, 0: layouts */
+
+/* Chooses the cluster size of the resident steps by timing (or takes the cached choice)
+ * and leaves the plan on the device; res_on stays false when nothing fits. Returns the
+ * time of a step in ms (0: taken from the cache). */
+int setup_resident(lb_ctx *c, float *step_ms)
+{
+    c->res_on = false;
+    *step_ms = 0.0f;
+    if (!resident_candidate(c)) return LB_OK;
+    c->res_pair = c->store == LB_STORE_F32 || c->store == LB_STORE_F32_DEV;
+    if (c->res_pair && !c->rtab) return LB_OK;
+    const int sr = (c->opts.rounding == LB_ROUND_STOCHASTIC &&
+                    (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV)) ? 1 : 0;
+    uint64_t hsh = 1469598103934665603ull;
+    for (uint8_t b : c->tmap) hsh = (hsh ^ b) * 1099511628211ull;
+    hsh = (hsh ^ (uint64_t)(sr + 2 * (c->opts.gx != 0.0 || c->opts.gy != 0.0) + 4 * (c->walls[0].kind == LB_WALL_PERIODIC))) *
+          1099511628211ull;
+    const std::tuple<int, int, int, int, int, uint64_t> key{c->store, c->nx, c->ny, c->q[0], c->q[1], hsh};
+    c->res_key = key;
+    int known = -1;
+    {
+        std::lock_guard<std::mutex> g(g_tune_mu);
+        auto it = g_res_tune.find(key);
+        if (it != g_res_tune.end()) known = it->second;
+    }
+    if (known == 0) return LB_OK;
+    const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
+    if (known > 0) {
+        if (!lbk::res_plan_build(one, c->store, c->res_pair, known, 1, sr, c->rplan)) return LB_OK;
+        if (int e = resident_upload(c)) return e;
+        c->res_on = true;
+        return LB_OK;
+    }
+    cudaEvent_t e0, e1;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+        cudaGetLastError();
+        return LB_OK;
+    }
+    constexpr int STEPS = 24;
+    float best = 1e30f;
+    int best_c = 0;
+    for (int cl : {1, 2, 4, 8, 16}) {
+        if (!lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, c->rplan) || resident_upload(c) != LB_OK) continue;
+        float ms = 1e30f;
+        for (int rep = 0; rep < 2; ++rep) {
+            cudaEventRecord(e0, c->stream);
+            if (resident_steps(c, STEPS, 0) != LB_OK) {
+                c->status = LB_OK;   /* this size cannot be launched here */
+                break;
+            }
+            cudaEventRecord(e1, c->stream);
+            float t = 0.0f;
+            if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess) ms = std::min(ms, t);
+        }
+        if (ms < 0.97f * best) {
+            best = ms;
+            best_c = cl;
+        }
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    if (int e = launch_check(c, "resident tuning")) return e;
+    if (best_c == 0 || !lbk::res_plan_build(one, c->store, c->res_pair, best_c, 1, sr, c->rplan)) return LB_OK;
+    if (int e = resident_upload(c)) return e;
+    {
+        std::lock_guard<std::mutex> g(g_tune_mu);
+        g_res_tune[key] = best_c;
+    }
+    c->res_on = true;
+    *step_ms = best / STEPS;
+    return LB_OK;
+}
+
 /* Autotuner: times every step-kernel layout on this lattice (reading the current level,
  * writing the other one, which the next step overwrites) and keeps the fastest. Results
  * are cached per (storage, grid, sets, interface mode, map) for the process. */
 using TuneKey = std::tuple<int, int, int, int, int, int, uint64_t>;
-std::mutex g_tune_mu;
 std::map<TuneKey, int> g_tune;
 
 template <typename R>
-int autotune_t(lb_ctx *c)
+int autotune_t(lb_ctx *c, float *step_ms)
 {
     uint64_t hsh = 1469598103934665603ull;
     for (uint8_t b : c->tmap) hsh = (hsh ^ b) * 1099511628211ull;
@@ -800,18 +1015,48 @@ int autotune_t(lb_ctx *c)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (cudaGetLastError() != cudaSuccess) return 0;
+    *step_ms = best_ms / 5.0f;
     std::lock_guard<std::mutex> g(g_tune_mu);
     g_tune[key] = best;
     return best;
 }
 
-int choose_variant(lb_ctx *c)
+int choose_variant(lb_ctx *c, float *step_ms)
 {
     if (c->opts.scheme == LB_SCHEME_STREAM) return 0;   /* one kernel */
     if (c->opts.variant >= 0) return variant_available(c, c->opts.variant) ? c->opts.variant : 0;
-    return use_f64(c) ? autotune_t<double>(c) : autotune_t<float>(c);
+    return use_f64(c) ? autotune_t<double>(c, step_ms) : autotune_t<float>(c, step_ms);
 }
 
+
+/* The resident steps or a layout: the resident steps outright for lattices whose whole work
+ * is a few thousand warp x population units (a step of the layouts is then one launch and
+ * one chain of populations, 25 us and more, against 2 to 6 us), else whichever a step
+ * times faster. */
+constexpr double RES_ALWAYS = 4000.0;
+int choose_steps(lb_ctx *c)
+{
+    float res_ms = 0.0f;
+    c->res_variant = false;
+    if (int e = setup_resident(c, &res_ms)) return e;
+    if (c->res_on && (res_ms == 0.0f || c->rplan.cost * c->rplan.cluster <= RES_ALWAYS)) {
+        c->variant = c->res_pair ? 9 : 0;   /* the layout with the same bits */
+        c->res_variant = true;
+        return LB_OK;
+    }
+    float lay_ms = 0.0f;
+    c->variant = choose_variant(c, &lay_ms);
+    if (c->res_on && lay_ms > 0.0f && lay_ms < res_ms) {
+        c->res_on = false;
+        std::lock_guard<std::mutex> g(g_tune_mu);
+        for (auto &kv : g_res_tune)   /* this lattice takes the layouts from now on */
+            if (kv.first == c->res_key) kv.second = 0;
+    } else if (c->res_on) {
+        c->variant = c->res_pair ? 9 : 0;
+        c->res_variant = true;
+    }
+    return LB_OK;
+}
 
 int ensure_learned_buffers(lb_ctx *c)
 {
@@ -885,10 +1130,43 @@ int learned_update(lb_ctx *c)
     return set_region_map_impl(c, cell.data());
 }
 
+/* what follows a step: the periodic reduction and the learned map's update */
+template <typename R>
+int after_step(lb_ctx *c)
+{
+    if (c->opts.reduce_every > 0 && c->step % c->opts.reduce_every == 0) {
+        StepParams<R> q = make_params<R>(c, c->cur, c->cur, c->t);
+        lbk::launch_reduce<R>(c->store, q, static_cast<R *>(c->d_uprev), c->d_part, c->d_counter, c->d_out,
+                              c->red_blocks, c->stream);
+        if (int e = launch_check(c, "reduce")) return e;
+        if (int e = cuda_check(c, cudaMemcpyAsync(c->h_out, c->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost,
+                                                  c->stream), "reduce copy"))
+            return e;
+        cudaEventRecord(c->red_event, c->stream);
+        c->red_pending = true;
+    }
+    if (c->mlp && c->mlp_every > 0 && c->step % c->mlp_every == 0) return learned_update(c);
+    return LB_OK;
+}
+
 template <typename R>
 int step_t(lb_ctx *c, int64_t n)
 {
     for (int64_t k = 0; k < n; ++k) {
+        if (c->res_on) {
+            /* as many steps as the next reduction, map update or wall table allows, in one launch */
+            int64_t m = std::min<int64_t>(n - k, 1 << 20);
+            if (c->opts.reduce_every > 0) m = std::min<int64_t>(m, c->opts.reduce_every - c->step % c->opts.reduce_every);
+            if (c->mlp && c->mlp_every > 0) m = std::min<int64_t>(m, c->mlp_every - c->step % c->mlp_every);
+            if (c->walls[0].omega > 0.0 || c->walls[1].omega > 0.0) m = std::min<int64_t>(m, lbk::RES_OSC);
+            if (int e = resident_steps_t<R>(c, (int)m, 1)) return e;
+            c->cur ^= (int)(m & 1);
+            for (int64_t i = 0; i < m; ++i) c->t += c->dt;
+            c->step += m;
+            k += m - 1;
+            if (int e = after_step<R>(c)) return e;
+            continue;
+        }
         const double t_new = c->t + c->dt;
         StepParams<R> p = make_params<R>(c, c->cur, c->cur ^ 1, t_new);
         if (c->opts.scheme == LB_SCHEME_STREAM) {
@@ -902,19 +1180,7 @@ int step_t(lb_ctx *c, int64_t n)
         c->cur ^= 1;
         c->t = t_new;
         c->step += 1;
-        if (c->opts.reduce_every > 0 && c->step % c->opts.reduce_every == 0) {
-            StepParams<R> q = make_params<R>(c, c->cur, c->cur, c->t);
-            lbk::launch_reduce<R>(c->store, q, static_cast<R *>(c->d_uprev), c->d_part, c->d_counter, c->d_out,
-                                  c->red_blocks, c->stream);
-            if (int e = launch_check(c, "reduce")) return e;
-            if (int e = cuda_check(c, cudaMemcpyAsync(c->h_out, c->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost,
-                                                      c->stream), "reduce copy"))
-                return e;
-            cudaEventRecord(c->red_event, c->stream);
-            c->red_pending = true;
-        }
-        if (c->mlp && c->mlp_every > 0 && c->step % c->mlp_every == 0)
-            if (int e = learned_update(c)) return e;
+        if (int e = after_step<R>(c)) return e;
     }
     return LB_OK;
 }
@@ -1256,7 +1522,11 @@ int lb_create(const lb_grid *grid, const uint8_t *region_map, const int32_t sets
         *out = nullptr;
         return e;
     }
-    c->variant = choose_variant(c);
+    if (int e2 = choose_steps(c)) {
+        lb_destroy(c);
+        *out = nullptr;
+        return e2;
+    }
     if (int e2 = launch_check(c, "autotune")) {
         lb_destroy(c);
         *out = nullptr;
@@ -1433,6 +1703,35 @@ int lb_learned_map_now(lb_ctx *c)
 }  // extern "C"
 
 namespace {
+/* After a map change: the resident plan of the new map with the cluster size in use, or a
+ * layout where the new map has none (timed on this map; every layout reads the level that
+ * finalize_level completes next). */
+int replan(lb_ctx *c)
+{
+    if (!c->res_variant) return LB_OK;
+    const int sr = (c->opts.rounding == LB_ROUND_STOCHASTIC &&
+                    (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV)) ? 1 : 0;
+    c->res_on = false;
+    if (resident_candidate(c)) {
+        const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
+        const int now = c->rplan.cluster;
+        for (int cl : {now, 1, 2, 4, 8, 16})
+            if (lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, c->rplan)) {
+                if (int e = resident_upload(c)) return e;
+                c->res_on = true;
+                return LB_OK;
+            }
+    }
+    /* a later map may take the resident steps again: the flag stays */
+    float ms = 0.0f;
+    const int keep = c->variant;
+    c->variant = -1;   /* the level is completed for every layout */
+    if (int e = finalize_level(c, c->cur)) return e;
+    c->variant = choose_variant(c, &ms);
+    if (c->variant < 0) c->variant = keep;
+    return LB_OK;
+}
+
 int set_region_map_impl(lb_ctx *c, const uint8_t *map)
 {
     std::vector<uint8_t> tm;
@@ -1457,6 +1756,7 @@ int set_region_map_impl(lb_ctx *c, const uint8_t *map)
     c->tmap = tm;
     c->iface_rows = rows;
     if (int e = upload_tiles(c)) return e;
+    if (int e = replan(c)) return e;
     if (int e = finalize_level(c, c->cur)) return e;
     return cuda_check(c, cudaStreamSynchronize(c->stream), "remap sync");
 }
@@ -1599,6 +1899,7 @@ int lb_load(lb_ctx *c, const char *path)
     for (int j = 0; j < c->ny; ++j)
         if (c->tmap[(size_t)j * c->ntx] & LB_TILE_IFACE) c->iface_rows.push_back(j);
     if (int e = upload_tiles(c)) return e;
+    if (int e = replan(c)) return e;
     if (int e = lb_state_load(c, buf.data(), bytes)) return e;
     if (int e = cuda_check(c, cudaStreamSynchronize(c->stream), "load sync")) return e;   /* buf goes away */
     c->step = hd.step;
@@ -1667,6 +1968,11 @@ struct lb_batch {
     lbk::RingTab *d_tabs = nullptr;
     uint32_t *d_items = nullptr;
     int2 *d_ranges = nullptr;
+    /* on the resident steps: bundles of lattices, one block each */
+    bool resident = false, res_pair = false;
+    lbk::ResPlan plan;
+    unsigned char *d_plan = nullptr;
+    uint32_t *d_off = nullptr;
     int status = LB_OK;
     std::vector<void *> owned;
 };
@@ -1819,8 +2125,54 @@ int batch_ring_setup(lb_batch *b)
     return LB_OK;
 }
 
+/* The resident steps for the whole batch: true when every lattice fits a block. */
+int batch_resident_setup(lb_batch *b, int nsm)
+{
+    std::vector<lbk::ResLattice> L;
+    for (const lb_ctx *c : b->inst) {
+        for (int j = 0; j < c->ny; ++j)
+            for (int tx = 1; tx < c->ntx; ++tx)
+                if ((c->tmap[(size_t)j * c->ntx + tx] ^ c->tmap[(size_t)j * c->ntx]) & LB_TILE_HIGH) return LB_OK;
+        if (c->ny > 0xfff0 || c->nx > 0x7fff || (b->res_pair && !c->rtab)) return LB_OK;
+        L.push_back(resident_lattice(c, resident_group(c, b->res_pair)));
+    }
+    if (!lbk::res_plan_build(L, b->store, b->res_pair, 1, nsm, 0, b->plan)) return LB_OK;
+    b->d_plan = static_cast<unsigned char *>(batch_alloc(b, b->plan.blob.size()));
+    b->d_off = static_cast<uint32_t *>(batch_alloc(b, b->plan.off.size() * sizeof(uint32_t)));
+    if (!b->d_plan || !b->d_off) return fail(LB_ERR_NOMEM, "device allocation failed");
+    cudaError_t e = cudaMemcpyAsync(b->d_plan, b->plan.blob.data(), b->plan.blob.size(), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_off, b->plan.off.data(), b->plan.off.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, b->stream);
+    std::vector<lbk::RingTab> tabs(b->res_pair ? b->n : 0);
+    if (b->res_pair) {
+        for (int i = 0; i < b->n; ++i) tabs[i] = *b->inst[i]->rtab;
+        b->d_tabs = static_cast<lbk::RingTab *>(batch_alloc(b, sizeof(lbk::RingTab) * b->n));
+        if (!b->d_tabs) return fail(LB_ERR_NOMEM, "device allocation failed");
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->d_tabs, tabs.data(), sizeof(lbk::RingTab) * b->n, cudaMemcpyHostToDevice, b->stream);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return fail(LB_ERR_CUDA, "batch plan upload failed");
+    b->resident = true;
+    for (lb_ctx *c : b->inst) c->ring_batch = false;   /* no carried moments to keep */
+    b->threads = 512;
+    b->grid = std::min(b->plan.parts, std::max(1, nsm));
+    return LB_OK;
+}
+
 int batch_launch(lb_batch *b, int64_t nsteps, int advance, cudaStream_t st)
 {
+    if (b->resident) {
+        const lbk::ResOsc<double> none{};   /* steady walls: only the count is read */
+        static_assert(offsetof(lbk::ResOsc<double>, n) == 0 && offsetof(lbk::ResOsc<float>, n) == 0, "the count comes first");
+        if (lbk::launch_resident(b->store, b->res_pair, b->force, b->plan, b->d_plan, b->d_off, b->d_params, b->d_tabs,
+                                 (int)nsteps, b->phase, 0u, advance, b->d_queue, &none, b->grid, st) != 0) {
+            cudaGetLastError();
+            b->status = LB_ERR_CUDA;
+            return fail(LB_ERR_CUDA, "batch launch failed");
+        }
+        return LB_OK;
+    }
     if (cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned int), st) != cudaSuccess)
         return fail(LB_ERR_CUDA, "batch queue reset failed");
     const int r = b->ring ? lbk::launch_ring_batch(b->store, b->q1, static_cast<const StepParams<float> *>(b->d_params),
@@ -1936,13 +2288,18 @@ int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps,
     if (!e && cudaMemcpyAsync(b->d_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
         e = fail(LB_ERR_CUDA, "batch order upload failed");
     if (!e) e = b->store == LB_STORE_F64 ? batch_upload_params<double>(b) : batch_upload_params<float>(b);
-    if (!e && b->ring) e = batch_ring_setup(b);
-    /* block size of the one-quad kernel: time each candidate without moving the state */
     int dev = 0, nsm = 0;
-    if (!e && !b->ring &&
+    if (!e &&
         (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
         e = fail(LB_ERR_CUDA, "device query failed");
-    if (!e && !b->ring) {
+    /* the resident steps where every lattice fits a block's shared memory (the bits of the
+     * other two kernels): layout 9's arithmetic for the ring batch's lattices, layout 0's
+     * for FP64 */
+    b->res_pair = b->ring;
+    if (!e && (b->ring || b->store == LB_STORE_F64)) e = batch_resident_setup(b, nsm);
+    if (!e && b->ring && !b->resident) e = batch_ring_setup(b);
+    /* block size of the one-quad kernel: time each candidate without moving the state */
+    if (!e && !b->ring && !b->resident) {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -2005,7 +2362,7 @@ int lb_batch_step_each(lb_batch *b, int64_t nsteps)
             if (int e = lb_step(c, 1)) return e;
     b->phase ^= (int)(nsteps & 1);
     /* layout 9 carries no moments: the ring batch's are summed again */
-    if (b->ring && nsteps > 0)
+    if (b->ring && !b->resident && nsteps > 0)
         for (lb_ctx *c : b->inst) {
             lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), nullptr, 0, c->stream);
             if (int e = launch_check(c, "carried moments")) return e;

@@ -21,6 +21,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 #include <vector_types.h>
 
@@ -195,6 +196,65 @@ int launch_ring_batch(int store, int q1, const StepParams<float> *params, const 
 /* Layout 10 (sets of 9 and of 16 or 36 populations), at most nblocks blocks */
 void launch_ring_units(int store, const StepParams<float> &p, const RingTab &tab, const RowQueues &rq, int nblocks,
                        void *stream);
+
+/* Resident steps (lb_resident.cuh): small lattices advanced n steps in one launch with the
+ * state in shared memory. A plan holds, per part (a bundle of lattices for one block, or
+ * one block's rows of a lattice on a cluster), the tables below; host-built by
+ * res_plan_build, from the rows' sets. */
+constexpr uint16_t RES_NONE = 0xffffu;
+enum : uint16_t { RES_SHADOW = 4u, RES_PUSH = 8u };   /* ResRow::flags; 1 / 2: bottom / top diffuse wall */
+struct alignas(8) ResRow {
+    uint16_t own, m2, m1, p1, p2;   /* row slots of the row and of rows j - 2 .. j + 2 in its set */
+    uint16_t view;                  /* its slot in the other set (shadow rows) */
+    uint16_t lat, flags;
+    uint16_t wallord, shord, j, pad;
+};
+struct ResGRow {
+    int lat, j;   /* the row's place in the lattices' planes */
+};
+struct ResRank {
+    uint32_t off_plane[2];
+    int nslot[2];
+};
+constexpr int RES_MAX_CLUSTER = 16;
+struct alignas(16) ResHead {
+    int q[2], K[2], nh[2];          /* populations, spare planes, wall-bound populations per set */
+    int nrow[2], nslot[2], nunit[2], G[2], nsh[2];   /* own rows, slots, units, population groups, shadow rows */
+    int rounds, nlat, W, pitch, xoff, nhmax, sr, table_bytes;
+    uint32_t upr_magic;
+    uint32_t off_rows, off_push, off_shlist, off_ids, off_grow, off_lat, off_pop, off_state, off_herm, off_wall, off_plane[2];
+    ResRank rank[RES_MAX_CLUSTER];
+};
+constexpr int RES_OSC = 64;
+template <typename R>
+struct ResOsc {   /* wall values of up to RES_OSC steps: u_x, u_y, kdiff of both sets, kout of both */
+    int n;
+    R v[RES_OSC][2][6];
+};
+/* One lattice as the plan needs it */
+struct ResLattice {
+    int W, ny, q[2];
+    bool periodic_y, wall[2];
+    const uint8_t *flags;           /* tile flags of the rows (every tile of a row has the row's set) */
+    int ntx;
+    uint64_t group;                 /* lattices of one bundle share it (equal population constants) */
+};
+struct ResPlan {
+    std::vector<unsigned char> blob;
+    std::vector<uint32_t> off;      /* [parts + 1] */
+    int parts = 0, cluster = 1;
+    size_t smem = 0;
+    double cost = 0.0;              /* work of the largest part, warp x population units */
+};
+/* cluster = 1: bundles for at most `blocks` resident blocks (any number of parts); else
+ * one lattice over `cluster` blocks. False when it does not fit. */
+bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int cluster, int blocks, int sr, ResPlan &out);
+/* Launch; params [lattice][2] and tabs [lattice] as for launch_ring_batch, plan and offsets
+ * in device memory, osc: ResOsc of the arithmetic type (n = 0: steady walls). Returns 0 or
+ * -1. */
+int launch_resident(int store, bool pair, bool force, const ResPlan &plan, const void *d_plan, const uint32_t *d_off,
+                    const void *params, const RingTab *tabs, int nsteps, int base, uint32_t step0, int advance,
+                    unsigned int *queue, const void *osc, int blocks, void *stream);
 
 /* The quad of nodes x0 .. x0+3 of row j needs none of the boundary work of the step
  * (wall overwrite, ghost-row or ghost-column copies, pressure column, mode-B shadow or

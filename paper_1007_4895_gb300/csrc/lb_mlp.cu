@@ -12,8 +12,8 @@
  *     node can hold, Sec. 2.2), measured on a high-order run;
  *   network: 8 -> 64 -> 64 -> 1, GELU (erf form) hidden layers, sigmoid output.
  * Training runs here in FP32 (mini-batch training in one cluster kernel; whole-set gradients
- * as a forward, a backward, a weight-gradient and an Adam kernel
- * each); inference uses BF16 weights with FP32 accumulation. Parameter layout:
+ * as a forward, a backward, a weight-gradient and an Adam kernel each);
+ * inference uses BF16 weights with FP32 accumulation. Parameter layout:
  * W1 [64][8], b1 [64], W2 [64][64], b2 [64], W3 [64], b3 [1] (4801 values).
  */
 #include <cooperative_groups.h>
