@@ -219,9 +219,10 @@ struct ResRank {
 constexpr int RES_MAX_CLUSTER = 16;
 struct alignas(16) ResHead {
     int q[2], K[2], nh[2];          /* populations, spare planes, wall-bound populations per set */
-    int nrow[2], nslot[2], nunit[2], G[2], nsh[2];   /* own rows, slots, units, population groups, shadow rows */
+    int nrow[2], nslot[2], nunit[2], nsh[2], nwall[2];   /* own rows, slots, units, shadow and wall rows */
+    int n[2], kr[2], rpg[2];        /* abscissae of the rule; abscissa rows per round and per item */
     int rounds, nlat, W, pitch, xoff, nhmax, sr, table_bytes;
-    uint32_t upr_magic;
+    uint32_t upr_magic, unit_magic[2];
     uint32_t off_rows, off_push, off_shlist, off_ids, off_grow, off_lat, off_pop, off_state, off_herm, off_wall, off_plane[2];
     ResRank rank[RES_MAX_CLUSTER];
 };

@@ -50,7 +50,8 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
     const bool images = z.V > 1 && f.W % z.V != 0;
     h.xoff = images ? 4 : 0;
     h.pitch = images ? 4 * upr + 8 : upr * z.V;
-    h.upr_magic = upr > 1 ? (uint32_t)(((1ull << 32) + upr - 1) / upr) : 0u;
+    auto magic = [](int n) { return n > 1 ? (uint32_t)(((1ull << 32) + n - 1) / n) : 0u; };   /* exact to 2^16 */
+    h.upr_magic = magic(upr);
     auto flag = [&](int lat, int j) { return L[lat].flags[(size_t)j * L[lat].ntx]; };
     auto set_of = [&](int lat, int j) { return (int)(flag(lat, j) & LB_TILE_HIGH); };
     auto owned = [&](int lat, int j) {
@@ -62,12 +63,14 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
         int lat, j, key;
     };
     std::vector<Own> own[2];
+    h.nwall[0] = h.nwall[1] = 0;
     for (size_t k = 0; k < p.own.size(); ++k) {
         const Piece &o = p.own[k];
         p.ids.push_back(o.lat);
         for (int j = o.j0; j < o.j1; ++j) {
             const bool wall = (j == 0 && L[o.lat].wall[0]) || (j == L[o.lat].ny - 1 && L[o.lat].wall[1]);
             /* the rows with the longest chains first: walls, then shadow rows */
+            h.nwall[set_of(o.lat, j)] += wall;
             own[set_of(o.lat, j)].push_back({o.lat, j, wall ? 0 : ((flag(o.lat, j) & LB_TILE_SHADOW) ? 1 : 2)});
         }
     }
@@ -79,6 +82,8 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
         }
         h.nrow[s] = (int)own[s].size();
         h.nunit[s] = h.nrow[s] * upr;
+        h.unit_magic[s] = magic(h.nunit[s]);
+        if (h.nunit[s] * 6 > 0xffff) return false;   /* items of a round */
     }
     auto lat_index = [&](int lat) {
         for (size_t k = 0; k < p.ids.size(); ++k)
@@ -136,6 +141,7 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
         if (h.nslot[s] > 60000) return false;
         h.q[s] = f.q[s];
         const int n1 = f.q[s] == 9 ? 3 : (f.q[s] == 16 ? 4 : 6);
+        h.n[s] = n1;
         h.nh[s] = n1 * (n1 / 2);
     }
     h.nhmax = std::max(h.nh[0], h.nh[1]);
@@ -149,7 +155,10 @@ size_t place_part(Part &p, const Sizes &z, int rounds, size_t pop_bytes, size_t 
 {
     ResHead &h = p.h;
     h.rounds = rounds;
-    for (int s = 0; s < 2; ++s) h.K[s] = (h.q[s] + rounds - 1) / rounds;
+    for (int s = 0; s < 2; ++s) {   /* whole abscissa rows, so that a row's planes are adjacent */
+        h.kr[s] = (h.n[s] + rounds - 1) / rounds;
+        h.K[s] = h.kr[s] * h.n[s];
+    }
     const int upr = (h.W + z.V - 1) / z.V;
     size_t o = up16(sizeof(ResHead));
     h.off_rows = (uint32_t)o;
@@ -180,34 +189,29 @@ size_t place_part(Part &p, const Sizes &z, int rounds, size_t pop_bytes, size_t 
     return o;
 }
 
-/* population groups per set that give the shortest round on the block's warps: a unit
- * costs its populations plus about a third of one for its set-up */
+/* abscissa rows per item that give the shortest round on the block's warps: an item costs
+ * its populations plus about half of one for its set-up */
 void split_part(Part &p)
 {
     ResHead &h = p.h;
     const int NW = 16;
-    const int nc[2] = {(h.nunit[0] + 31) / 32, (h.nunit[1] + 31) / 32};
     double best = 1e30;
-    for (int g1 = 1; g1 <= h.K[1]; ++g1) {
-        const int per1 = (h.K[1] + g1 - 1) / g1;
-        if ((h.K[1] + per1 - 1) / per1 != g1) continue;
-        for (int g0 = 1; g0 <= h.K[0]; ++g0) {
-            const int per0 = (h.K[0] + g0 - 1) / g0;
-            if ((h.K[0] + per0 - 1) / per0 != g0) continue;
+    h.rpg[0] = h.rpg[1] = 1;
+    for (int g1 = 1; g1 <= h.kr[1]; ++g1)
+        for (int g0 = 1; g0 <= h.kr[0]; ++g0) {
             double t[NW] = {};
-            const int u1 = nc[1] * g1, u0 = nc[0] * g0;
-            for (int u = 0; u < u1 + u0; ++u) t[u % NW] += 0.35 + (u < u1 ? per1 : per0);
+            const int u1 = (h.nunit[1] * ((h.kr[1] + g1 - 1) / g1) + 31) / 32, u0 = (h.nunit[0] * ((h.kr[0] + g0 - 1) / g0) + 31) / 32;
+            for (int u = 0; u < u1 + u0; ++u) t[u % NW] += 0.5 + (u < u1 ? g1 * h.n[1] : g0 * h.n[0]);
             double mx = 0.0, sum = 0.0;
             for (double v : t) mx = std::max(mx, v), sum += v;
             const double c = mx + 0.02 * sum;
             if (c < best) {
                 best = c;
-                h.G[0] = g0;
-                h.G[1] = g1;
+                h.rpg[0] = g0;
+                h.rpg[1] = g1;
             }
         }
-    }
-    p.cost = (double)nc[1] * h.q[1] + (double)nc[0] * h.q[0];
+    p.cost = (double)(h.nunit[1] * h.q[1] + h.nunit[0] * h.q[0]) / 32.0;
 }
 
 }  // namespace
@@ -215,7 +219,7 @@ void split_part(Part &p)
 bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int cluster, int blocks, int sr, ResPlan &out)
 {
     const Sizes z{pair ? 4 : 1, store == 0 ? 8 : (store <= 2 ? 4 : 2), store == 0 ? 8 : 4, store == 2, pair};
-    const size_t pop_bytes = pair ? sizeof(RingTab) : 2 * LB_QMAX * 16 * (size_t)z.rsize;
+    const size_t pop_bytes = (L[0].q[0] + L[0].q[1]) * (pair ? sizeof(RingPop) : 16 * (size_t)z.rsize);
     const size_t lat_bytes = 24 * (size_t)z.rsize;
     std::vector<Part> parts;
     if (cluster > 1) {
@@ -253,7 +257,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
             p.own.push_back({(int)i, 0, L[i].ny});
             if (!layout_part(L, p, z, false)) return false;
             bool fits = false;
-            for (int r : {1, 2, 3, 4, 6, 9, 12}) {
+            for (int r : {1, 2, 3, 6}) {
                 if (place_part(p, z, r, pop_bytes, lat_bytes) <= RES_SMEM) {
                     fits = true;
                     break;
@@ -332,7 +336,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
     }
     /* one number of rounds for the blocks of a cluster (a round ends with a barrier of
      * all of them); each bundle the fewest that fit */
-    for (int r : {1, 2, 3, 4, 6, 9, 12}) {
+    for (int r : {1, 2, 3, 6}) {
         bool all = true;
         for (Part &p : parts) {
             if (cluster == 1 && p.h.rounds > 0 && p.smem <= RES_SMEM) continue;

@@ -85,6 +85,23 @@ __device__ __forceinline__ void res_st(T *p, const T (&v)[V])
     else stn<V>(p, v);
 }
 
+/* Everything lives in one dynamic allocation; every function below takes its address from
+ * this symbol, so that all accesses are shared-memory loads and stores. */
+extern __shared__ __align__(16) unsigned char res_smem[];
+
+__device__ __forceinline__ const ResHead &res_head() { return *reinterpret_cast<const ResHead *>(res_smem); }
+
+/* minmod (the median of a, b and 0) on the bit patterns of FP64 values: the FP64 units are
+ * the bound of these steps, the integer units are idle. The value is minmod_n's. */
+__device__ __forceinline__ double res_minmod(double a, double b)
+{
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const unsigned long long ma = (unsigned long long)ia & 0x7fffffffffffffffull, mb = (unsigned long long)ib & 0x7fffffffffffffffull;
+    const long long m = ma < mb ? ia : ib;
+    return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m);
+}
+__device__ __forceinline__ float res_minmod(float a, float b) { return minmod_n(a, b, neg_part(a), neg_part(b)); }
+
 template <int ST, bool PAIR, bool FORCE, bool CL>
 struct Resident {
     using T = typename Store<ST>::T;
@@ -95,157 +112,191 @@ struct Resident {
     /* a deviation survives encode and decode unchanged: the wall sums can read the planes */
     static constexpr bool EXACT = ST == 2;
 
-    const ResHead &h;
-    unsigned char *sm;
-    const ResRow *rows;
-    const ResLat<R> *lats;
-    const Pop *pops;   /* [2][LB_QMAX] */
-    int warp, lane, W, upr, pitch, xoff;
-    uint32_t rowb;
-
-    __device__ __forceinline__ Resident(const ResHead &hh, unsigned char *s)
-        : h(hh), sm(s), rows(reinterpret_cast<const ResRow *>(s + hh.off_rows)),
-          lats(reinterpret_cast<const ResLat<R> *>(s + hh.off_lat)), pops(reinterpret_cast<const Pop *>(s + hh.off_pop)),
-          warp(threadIdx.x / 32), lane(threadIdx.x & 31), W(hh.W), upr((hh.W + V - 1) / V), pitch(hh.pitch),
-          xoff(hh.xoff), rowb(hh.pitch * sizeof(T))
+    static __device__ __forceinline__ const ResRow *rows() { return reinterpret_cast<const ResRow *>(res_smem + res_head().off_rows); }
+    static __device__ __forceinline__ const ResLat<R> *lats() { return reinterpret_cast<const ResLat<R> *>(res_smem + res_head().off_lat); }
+    static __device__ __forceinline__ const Pop *pops(int s) { return reinterpret_cast<const Pop *>(res_smem + res_head().off_pop) + (s ? res_head().q[0] : 0); }
+    static __device__ __forceinline__ T *at(uint32_t off) { return reinterpret_cast<T *>(res_smem + off); }
+    static __device__ __forceinline__ int upr_of(int W) { return (W + V - 1) / V; }
+    static __device__ __forceinline__ int div(int e, int n, uint32_t magic) { return n == 1 ? e : (int)__umulhi((uint32_t)e, magic); }
+    /* physical plane of population a of set s */
+    static __device__ __forceinline__ int phys(const ResHead &h, int s, int a, int phase)
     {
-    }
-    __device__ __forceinline__ int phys(int s, int a, int phase) const
-    {
-        const int M = h.q[s] + h.K[s];
-        int k = a + phase;
+        const int M = h.q[s] + h.K[s], k = a + phase;
         return k >= M ? k - M : k;
     }
-    __device__ __forceinline__ T *plane(int s, int ph) const
+    /* byte offset of row slot `slot` of physical plane ph */
+    static __device__ __forceinline__ uint32_t place(const ResHead &h, int s, int ph, int slot)
     {
-        return reinterpret_cast<T *>(sm + h.off_plane[s] + (uint32_t)ph * h.nslot[s] * rowb);
+        return h.off_plane[s] + ((uint32_t)(ph * h.nslot[s] + slot) * (uint32_t)h.pitch + (uint32_t)h.xoff) * (uint32_t)sizeof(T);
     }
-    /* unit e of set s: row and first column */
-    __device__ __forceinline__ void locate(int e, int &r, int &x0) const
+    /* a unit of a row (rowp: its column 0), with the row's periodic images beside it where
+     * the width is not a whole number of quads */
+    static __device__ __forceinline__ void put(T *rowp, int x0, int W, bool images, const T (&e)[V])
     {
-        r = upr == 1 ? e : (int)__umulhi((uint32_t)e, h.upr_magic);
-        x0 = (e - r * upr) * V;
-    }
-    __device__ __forceinline__ R *state(int s) const
-    {
-        return reinterpret_cast<R *>(sm + h.off_state) + (s ? 5 * V * h.nunit[0] : 0);
-    }
-    /* the row's periodic images beside it (only rows whose width is not a whole number of
-     * quads keep any), then the copies in other blocks */
-    __device__ __forceinline__ void put(T *pl, int slot, int x0, const T (&e)[V]) const
-    {
-        T *row = pl + slot * pitch + xoff;
-        if (V == 1 || xoff == 0 || x0 + V <= W) {
-            res_st<V>(row + x0, e);
-        } else {
-#pragma unroll
-            for (int k = 0; k < V; ++k)
-                if (x0 + k < W) row[x0 + k] = e[k];
+        if (V == 1 || !images) {
+            res_st<V>(rowp + x0, e);
+            return;
         }
-        if (V > 1 && xoff != 0) {
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-                const int x = x0 + k;
-                if (x < 2) row[x + W] = e[k];
-                if (x >= W - 2 && x < W) row[x - W] = e[k];
-            }
+        for (int k = 0; k < V; ++k) {
+            const int x = x0 + k;
+            if (x < W) rowp[x] = e[k];
+            if (x < 2) rowp[x + W] = e[k];
+            if (x >= W - 2 && x < W) rowp[x - W] = e[k];
         }
     }
-    __device__ __forceinline__ void push(int s, int ph, const uint16_t *to, int x0, const T (&e)[V]) const
+    /* the same unit into the blocks that read the row */
+    static __device__ __forceinline__ void push(const ResHead &h, int s, int ph, int rowi, int view, int x0, const T (&e)[V])
     {
-        namespace cg = cooperative_groups;
         if constexpr (CL) {
+            namespace cg = cooperative_groups;
+            const uint16_t *to = reinterpret_cast<const uint16_t *>(res_smem + h.off_push) + 8 * rowi + 4 * view;
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
                 const int rk = to[2 * t];
                 if (rk == RES_NONE) continue;
                 const ResRank &k = h.rank[rk];
-                T *local = reinterpret_cast<T *>(sm + k.off_plane[s] + (uint32_t)ph * k.nslot[s] * rowb);
-                put(cg::this_cluster().map_shared_rank(local, rk), to[2 * t + 1], x0, e);
+                T *local = at(k.off_plane[s] + ((uint32_t)(ph * k.nslot[s] + to[2 * t + 1]) * (uint32_t)h.pitch + (uint32_t)h.xoff) * (uint32_t)sizeof(T));
+                put(cg::this_cluster().map_shared_rank(local, rk), x0, h.W, V > 1 && h.xoff != 0, e);
             }
         }
     }
-    __device__ __forceinline__ const uint16_t *pushes(int row, int view) const
-    {
-        return reinterpret_cast<const uint16_t *>(sm + h.off_push) + 8 * row + 4 * view;
-    }
     static __device__ __forceinline__ R dec(T v, R winv, R rho0) { return decode<ST>(v, winv, rho0); }
 
-    /* ---- 1. moments and collision coefficients (and the wall fill of wall rows) ---- */
-    template <bool FILL>
-    __device__ void moments(const int (&phase)[2])
+    /* ---- wall rows (Sec. 3.2): one (unit, gas-bound population) per thread. rho_W from the
+     * wall-bound populations as updated, before they were rounded to storage (every thread
+     * of a unit forms the same sum, in population order), then f = rho_W S(u_W). ---- */
+    static __device__ __forceinline__ void walls(const int (&phase)[2])
     {
-        const int nc[2] = {(h.nunit[0] + 31) / 32, (h.nunit[1] + 31) / 32};
-        for (int u = warp; u < nc[0] + nc[1]; u += RES_WARPS) {
-            const int s = u < nc[1] ? 1 : 0;
-            const int e = (s ? u : u - nc[1]) * 32 + lane;
-            const bool on = e < h.nunit[s];
-            int r, x0;
-            locate(on ? e : 0, r, x0);
-            const int rowi = (s ? h.nrow[0] : 0) + r;
-            const ResRow rr = rows[rowi];
-            const ResLat<R> &L = lats[rr.lat];
-            const Pop *tp = pops + s * LB_QMAX;
+        const ResHead &h = res_head();
+        const int W = h.W, upr = upr_of(W);
+        const int n0 = h.nwall[0] * upr, n1 = h.nwall[1] * upr;
+        const int t0 = n0 * h.nh[0], total = t0 + n1 * h.nh[1];
+        for (int it = threadIdx.x; it < total; it += RES_THREADS) {
+            const int s = it < t0 ? 0 : 1, k0 = s ? it - t0 : it, n = s ? n1 : n0;
+            const int i = k0 / n, un = k0 - i * n;
+            const int r = div(un, upr, h.upr_magic), x0 = (un - r * upr) * V;   /* the wall rows come first */
+            const int rowi = (s ? h.nrow[0] : 0) + r, Q = h.q[s], nh = h.nh[s];
+            const ResRow rr = rows()[rowi];
+            const ResLat<R> &L = lats()[rr.lat];
+            const int w = (rr.flags & 2) ? 1 : 0;
+            const R nsgn = w == 0 ? R(1) : R(-1), rho0 = L.rho0;
+            const int ab = w == 0 ? 0 : Q - nh, a = (w == 0 ? Q - nh : 0) + i;   /* wall-bound half, this population */
+            const Pop *tp = pops(s);
+            R num[V];
+#pragma unroll
+            for (int k = 0; k < V; ++k) num[k] = R(0);
+            const R *wb = reinterpret_cast<const R *>(res_smem + h.off_wall) + ((rr.wallord * h.nhmax) * upr + x0 / V) * V;
+            const uint32_t pstride = (uint32_t)(h.nslot[s] * h.pitch) * (uint32_t)sizeof(T);
+            uint32_t po = place(h, s, phys(h, s, ab, phase[s]), rr.own) + x0 * (uint32_t)sizeof(T);
+            const uint32_t pend = h.off_plane[s] + (uint32_t)(Q + h.K[s]) * pstride, plen = (uint32_t)(Q + h.K[s]) * pstride;
+#pragma unroll 6
+            for (int b = 0; b < nh; ++b) {
+                const Pop &p = tp[ab + b];
+                const R xn = PO::cy(p) * nsgn;
+                R d[V];
+                if constexpr (EXACT) {
+                    T raw[V];
+                    res_ld<V>(at(po), raw);
+#pragma unroll
+                    for (int k = 0; k < V; ++k) d[k] = dec(raw[k], PO::winv(p), rho0);
+                    po += pstride;
+                    if (po >= pend) po -= plen;
+                } else {
+                    res_ld<V>(wb + b * upr * V, d);
+                }
+#pragma unroll
+                for (int k = 0; k < V; ++k) num[k] = fma(-xn * PO::w(p), d[k], num[k]);
+            }
+            const R uwx = L.uw_x[w], uwy = L.uw_y[w];
+            const R usw = uwx * uwx + uwy * uwy;
+            const R kd = L.kdiff[s][w], kout = L.kout[s][w];
+            const Pop &p = tp[a];
+            const R ew = PO::cx(p) * uwx + PO::cy(p) * uwy;
+            const R sm1 = ew + R(0.5) * (ew * ew - usw);    /* S / w - 1 */
+            T e[V];
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                const R rwd = fma(rho0, kd, num[k]) / kout;   /* rho_W - rho0 */
+                e[k] = encode<ST>(fma(rwd + rho0, sm1, rwd), PO::w(p), rho0);
+            }
+            const int ph = phys(h, s, a, phase[s]);
+            put(at(place(h, s, ph, rr.own)), x0, W, V > 1 && h.xoff != 0, e);
+            if (CL && (rr.flags & RES_PUSH)) push(h, s, ph, rowi, 0, x0, e);
+        }
+    }
+
+    /* ---- moments in population order, and each node's collision coefficients ---- */
+    static __device__ __forceinline__ void moments(const int (&phase)[2])
+    {
+        const ResHead &h = res_head();
+        const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+        const int W = h.W, upr = upr_of(W), nc1 = (h.nunit[1] + 31) / 32, nc0 = (h.nunit[0] + 31) / 32;
+        for (int u = warp; u < nc0 + nc1; u += RES_WARPS) {
+            const int s = u < nc1 ? 1 : 0, nu = h.nunit[s];
+            const int e = (s ? u : u - nc1) * 32 + lane;
+            const bool on = e < nu;
+            const int r = div(on ? e : 0, upr, h.upr_magic), x0 = ((on ? e : 0) - r * upr) * V;
+            const ResRow rr = rows()[(s ? h.nrow[0] : 0) + r];
+            const ResLat<R> &L = lats()[rr.lat];
+            const Pop *tp = pops(s);
             const int Q = h.q[s];
             const R rho0 = L.rho0;
-            const int off = rr.own * pitch + xoff + x0;
-            const bool wall = on && (rr.flags & 3);
-            if (FILL && wall) wall_fill(s, rr, rowi, x0, phase[s], L);
-            R rd[V], jx[V], jy[V], hh[3][V];
+            const uint32_t pstride = (uint32_t)(h.nslot[s] * h.pitch) * (uint32_t)sizeof(T);
+            const uint32_t plen = (uint32_t)(Q + h.K[s]) * pstride, pend = h.off_plane[s] + plen;
+            uint32_t po = place(h, s, phase[s], rr.own) + x0 * (uint32_t)sizeof(T);
+            R rd[V], jx[V], jy[V];
 #pragma unroll
-            for (int k = 0; k < V; ++k) rd[k] = jx[k] = jy[k] = hh[0][k] = hh[1][k] = hh[2][k] = R(0);
+            for (int k = 0; k < V; ++k) rd[k] = jx[k] = jy[k] = R(0);
             const bool sh = on && (rr.flags & RES_SHADOW);
-            const int M = Q + h.K[s];
-            int ph = phase[s];
-            if (__any_sync(0xffffffffu, sh)) {
-#pragma unroll 4
-                for (int a = 0; a < Q; ++a) {
-                    T raw[V];
-                    res_ld<V>(plane(s, ph) + off, raw);
-                    ph = ph + 1 == M ? 0 : ph + 1;
-                    const Pop &p = tp[a];
+            R hh[3][V];
 #pragma unroll
-                    for (int k = 0; k < V; ++k) {
-                        const R d = dec(raw[k], PO::winv(p), rho0);
-                        rd[k] = fma(PO::w(p), d, rd[k]);
-                        jx[k] = fma(PO::wcx(p), d, jx[k]);
-                        jy[k] = fma(PO::wcy(p), d, jy[k]);
-                        hh[0][k] = fma(R(p.wxx), d, hh[0][k]);
-                        hh[1][k] = fma(R(p.wxy), d, hh[1][k]);
-                        hh[2][k] = fma(R(p.wyy), d, hh[2][k]);
-                    }
-                }
-            } else {
-#pragma unroll 6
-                for (int a = 0; a < Q; ++a) {
-                    T raw[V];
-                    res_ld<V>(plane(s, ph) + off, raw);
-                    ph = ph + 1 == M ? 0 : ph + 1;
-                    const Pop &p = tp[a];
-                    if constexpr (PAIR) {
+            for (int k = 0; k < V; ++k) hh[0][k] = hh[1][k] = hh[2][k] = R(0);
+            auto sums = [&](const Pop &p, const T (&raw)[V], auto herm) {
+                if constexpr (PAIR) {
 #pragma unroll
-                        for (int k = 0; k < V; k += 2) {
-                            const float2 d = make_float2(dec(raw[k], p.winv2.x, rho0), dec(raw[k + 1], p.winv2.x, rho0));
-                            const float2 a0 = fma2(p.w2, d, make_float2(rd[k], rd[k + 1]));
-                            const float2 a1 = fma2(p.wcx2, d, make_float2(jx[k], jx[k + 1]));
-                            const float2 a2 = fma2(p.wcy2, d, make_float2(jy[k], jy[k + 1]));
-                            rd[k] = a0.x, rd[k + 1] = a0.y;
-                            jx[k] = a1.x, jx[k + 1] = a1.y;
-                            jy[k] = a2.x, jy[k + 1] = a2.y;
+                    for (int k = 0; k < V; k += 2) {
+                        const float2 d = make_float2(dec(raw[k], p.winv2.x, rho0), dec(raw[k + 1], p.winv2.x, rho0));
+                        const float2 a0 = fma2(p.w2, d, make_float2(rd[k], rd[k + 1]));
+                        const float2 a1 = fma2(p.wcx2, d, make_float2(jx[k], jx[k + 1]));
+                        const float2 a2 = fma2(p.wcy2, d, make_float2(jy[k], jy[k + 1]));
+                        rd[k] = a0.x, rd[k + 1] = a0.y;
+                        jx[k] = a1.x, jx[k + 1] = a1.y;
+                        jy[k] = a2.x, jy[k + 1] = a2.y;
+                        if constexpr (decltype(herm)::value) {
+                            hh[0][k] = fma(p.wxx, d.x, hh[0][k]), hh[0][k + 1] = fma(p.wxx, d.y, hh[0][k + 1]);
+                            hh[1][k] = fma(p.wxy, d.x, hh[1][k]), hh[1][k + 1] = fma(p.wxy, d.y, hh[1][k + 1]);
+                            hh[2][k] = fma(p.wyy, d.x, hh[2][k]), hh[2][k + 1] = fma(p.wyy, d.y, hh[2][k + 1]);
                         }
-                    } else {
-                        const R d = dec(raw[0], PO::winv(p), rho0);
-                        rd[0] = fma(PO::w(p), d, rd[0]);
-                        jx[0] = fma(PO::wcx(p), d, jx[0]);
-                        jy[0] = fma(PO::wcy(p), d, jy[0]);
+                    }
+                } else {
+                    const R d = dec(raw[0], p.winv, rho0);
+                    rd[0] = fma(p.w, d, rd[0]);
+                    jx[0] = fma(p.wcx, d, jx[0]);
+                    jy[0] = fma(p.wcy, d, jy[0]);
+                    if constexpr (decltype(herm)::value) {
+                        hh[0][0] = fma(p.wxx, d, hh[0][0]);
+                        hh[1][0] = fma(p.wxy, d, hh[1][0]);
+                        hh[2][0] = fma(p.wyy, d, hh[2][0]);
                     }
                 }
-            }
+            };
+            auto all = [&](auto herm) {
+#pragma unroll 3
+                for (int a = 0; a < Q; ++a) {
+                    T raw[V];
+                    res_ld<V>(at(po), raw);
+                    po += pstride;
+                    if (po >= pend) po -= plen;
+                    sums(tp[a], raw, herm);
+                }
+            };
+            if (__any_sync(0xffffffffu, sh)) all(std::true_type{});
+            else all(std::false_type{});
             if (!on) continue;
-            /* velocity, relaxation frequency, and (PAIR) the constant part of the folded
-             * collision, as pair_node_state forms them, or the density deviation */
-            R *st = state(s) + V * e;
-            const int n = V * h.nunit[s];
+            /* velocity, relaxation frequency, density and (PAIR) the constant part of the
+             * folded collision, as pair_node_state forms them, or the density deviation */
+            R *st = reinterpret_cast<R *>(res_smem + h.off_state) + (s ? 5 * V * h.nunit[0] : 0) + V * e;
             R out[5][V];
 #pragma unroll
             for (int k = 0; k < V; ++k) {
@@ -267,9 +318,9 @@ struct Resident {
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 5; ++i) res_st<V>(st + i * n, out[i]);
+            for (int i = 0; i < 5; ++i) res_st<V>(st + i * V * nu, out[i]);
             if (sh) {
-                R *hs = reinterpret_cast<R *>(sm + h.off_herm) + ((size_t)rr.shord * upr + x0 / V) * 6 * V;
+                R *hs = reinterpret_cast<R *>(res_smem + h.off_herm) + (rr.shord * upr + x0 / V) * 6 * V;
                 res_st<V>(hs, rd);
                 res_st<V>(hs + V, jx);
                 res_st<V>(hs + 2 * V, jy);
@@ -280,77 +331,26 @@ struct Resident {
         }
     }
 
-    /* wall row: rho_W from the wall-bound populations as updated (before they were rounded
-     * to storage), then the gas-bound ones f = rho_W S(u_W) */
-    __device__ __noinline__ void wall_fill(int s, const ResRow &rr, int rowi, int x0, int phase, const ResLat<R> &L)
+    /* ---- views of shadow rows in the other set, one (unit, population) per thread ---- */
+    static __device__ __forceinline__ void views(const int (&phase)[2])
     {
-        const int w = (rr.flags & 2) ? 1 : 0, Q = h.q[s], nh = h.nh[s];
-        const R nsgn = w == 0 ? R(1) : R(-1), rho0 = L.rho0;
-        const Pop *tp = pops + s * LB_QMAX;
-        const int off = rr.own * pitch + xoff + x0;
-        const int ab = w == 0 ? 0 : Q - nh, ag = w == 0 ? Q - nh : 0;   /* wall-bound, gas-bound halves */
-        const R *wb = reinterpret_cast<const R *>(sm + h.off_wall) + ((size_t)rr.wallord * h.nhmax * upr + x0 / V) * V;
-        R num[V];
-#pragma unroll
-        for (int k = 0; k < V; ++k) num[k] = R(0);
-#pragma unroll 6
-        for (int i = 0; i < nh; ++i) {
-            const Pop &p = tp[ab + i];
-            const R xn = PO::cy(p) * nsgn;
-            R d[V];
-            if constexpr (EXACT) {
-                T raw[V];
-                res_ld<V>(plane(s, phys(s, ab + i, phase)) + off, raw);
-#pragma unroll
-                for (int k = 0; k < V; ++k) d[k] = dec(raw[k], PO::winv(p), rho0);
-            } else {
-                res_ld<V>(wb + (size_t)i * upr * V, d);
-            }
-#pragma unroll
-            for (int k = 0; k < V; ++k) num[k] = fma(-xn * PO::w(p), d[k], num[k]);
-        }
-        const R uwx = L.uw_x[w], uwy = L.uw_y[w];
-        const R usw = uwx * uwx + uwy * uwy;
-        const R kd = L.kdiff[s][w], kout = L.kout[s][w];
-        R rwd[V];
-#pragma unroll
-        for (int k = 0; k < V; ++k) rwd[k] = fma(rho0, kd, num[k]) / kout;   /* rho_W - rho0 */
-        const uint16_t *to = pushes(rowi, 0);
-#pragma unroll 2
-        for (int i = 0; i < nh; ++i) {
-            const int a = ag + i;
-            const Pop &p = tp[a];
-            const R ew = PO::cx(p) * uwx + PO::cy(p) * uwy;
-            const R sm1 = ew + R(0.5) * (ew * ew - usw);    /* S / w - 1 */
-            T e[V];
-#pragma unroll
-            for (int k = 0; k < V; ++k) e[k] = encode<ST>(fma(rwd[k] + rho0, sm1, rwd[k]), PO::w(p), rho0);
-            const int ph = phys(s, a, phase);
-            put(plane(s, ph), rr.own, x0, e);
-            if (CL && (rr.flags & RES_PUSH)) push(s, ph, to, x0, e);
-        }
-    }
-
-    /* ---- 2. views of shadow rows in the other set, one (unit, population) per thread ---- */
-    __device__ void views(const int (&phase)[2])
-    {
-        const uint16_t *list = reinterpret_cast<const uint16_t *>(sm + h.off_shlist);
-        const int q1 = h.q[1], q0 = h.q[0];
-        const int n1 = h.nsh[1] * upr, n0 = h.nsh[0] * upr;   /* shadow units per own set */
-        const int total = n0 * q1 + n1 * q0;
+        const ResHead &h = res_head();
+        const uint16_t *list = reinterpret_cast<const uint16_t *>(res_smem + h.off_shlist);
+        const int W = h.W, upr = upr_of(W), n1 = h.nsh[1] * upr, n0 = h.nsh[0] * upr;   /* shadow units per own set */
+        const int t0 = n0 * h.q[1], total = t0 + n1 * h.q[0];
         for (int i = threadIdx.x; i < total; i += RES_THREADS) {
-            const int s = i < n0 * q1 ? 0 : 1;   /* the rows' own set */
-            const int t = 1 - s, k0 = s == 0 ? i : i - n0 * q1, n = s == 0 ? n0 : n1;
+            const int s = i < t0 ? 0 : 1;   /* the rows' own set */
+            const int t = 1 - s, k0 = s == 0 ? i : i - t0, n = s == 0 ? n0 : n1;
             const int b = k0 / n, un = k0 - b * n;
-            const int ord = (s == 0 ? 0 : h.nsh[0]) + un / upr, x0 = (un % upr) * V;
+            const int o = div(un, upr, h.upr_magic), x0 = (un - o * upr) * V, ord = (s == 0 ? 0 : h.nsh[0]) + o;
             const int rowi = list[ord];
-            const ResRow rr = rows[rowi];
-            const R rho0 = lats[rr.lat].rho0;
-            const R *hs = reinterpret_cast<const R *>(sm + h.off_herm) + ((size_t)ord * upr + x0 / V) * 6 * V;
+            const ResRow rr = rows()[rowi];
+            const R rho0 = lats()[rr.lat].rho0;
+            const R *hs = reinterpret_cast<const R *>(res_smem + h.off_herm) + (ord * upr + x0 / V) * 6 * V;
             R c[6][V];
 #pragma unroll
             for (int m = 0; m < 6; ++m) res_ld<V>(hs + m * V, c[m]);
-            const Pop &p = pops[t * LB_QMAX + b];
+            const Pop &p = pops(t)[b];
             T e[V];
 #pragma unroll
             for (int k = 0; k < V; ++k) {   /* hermite_rebuild, term by term */
@@ -361,180 +361,281 @@ struct Resident {
                 v = fma(c[5][k], R(p.hyy), v);
                 e[k] = encode<ST>(v, PO::w(p), rho0);
             }
-            const int ph = phys(t, b, phase[t]);
-            if (rr.view != RES_NONE) put(plane(t, ph), rr.view, x0, e);
-            if (CL && (rr.flags & RES_PUSH)) push(t, ph, pushes(rowi, 1), x0, e);
+            const int ph = phys(h, t, b, phase[t]);
+            if (rr.view != RES_NONE) put(at(place(h, t, ph, rr.view)), x0, W, V > 1 && h.xoff != 0, e);
+            if (CL && (rr.flags & RES_PUSH)) push(h, t, ph, rowi, 1, x0, e);
         }
     }
 
-    /* ---- 3. one round of the update: populations [a0, a1) of set s for 32 units ---- */
-    __device__ __forceinline__ void update(int s, int chunk, int a0, int a1, int phase, uint32_t step_key, bool sr)
+    /* ---- one round of the update of set s: abscissa rows iy [lo, hi) of the product rule,
+     * an item being a unit x rpg of those rows (n populations each, so that the sign of
+     * xi_x is the same in every lane); warps take 32 items at a time, starting at u0 ---- */
+    static __device__ __forceinline__ void update(int s, int lo, int hi, int phase, int u0, uint32_t step_key, bool sr)
     {
-        const int e = chunk * 32 + lane;
-        if (e >= h.nunit[s]) return;
-        int r, x0;
-        locate(e, r, x0);
-        const int rowi = (s ? h.nrow[0] : 0) + r;
-        const ResRow rr = rows[rowi];
-        const ResLat<R> &L = lats[rr.lat];
-        const Pop *tp = pops + s * LB_QMAX;
-        const R rho0 = L.rho0;
-        const int n = V * h.nunit[s];
-        R stt[5][V];
-        {
-            const R *st = state(s) + V * e;
+        const ResHead &h = res_head();
+        const int lane = threadIdx.x & 31, nu = h.nunit[s], rpg = h.rpg[s], n = h.n[s];
+        const int items = nu * ((hi - lo + rpg - 1) / rpg), nunits = (items + 31) / 32;
+        const int W = h.W, upr = upr_of(W), r0 = s ? h.nrow[0] : 0;
+        const bool images = V > 1 && h.xoff != 0;
+        const uint32_t pitchb = (uint32_t)h.pitch * (uint32_t)sizeof(T), pstride = (uint32_t)h.nslot[s] * pitchb;
+        const uint32_t umagic = h.unit_magic[s], upmagic = h.upr_magic;
+        const uint32_t base = h.off_plane[s] + (uint32_t)h.xoff * (uint32_t)sizeof(T);
+        const int M = h.q[s] + h.K[s], K = h.K[s];
+        const R *stb = reinterpret_cast<const R *>(res_smem + h.off_state) + (s ? 5 * V * h.nunit[0] : 0);
+        const Pop *tp = pops(s);
+        for (int u = u0; u < nunits; u += RES_WARPS) {
+            const int item = u * 32 + lane;
+            if (item >= items) continue;
+            const int g = div(item, nu, umagic), e = item - g * nu;
+            const int r = div(e, upr, upmagic), x0 = (e - r * upr) * V;
+            const ResRow rr = rows()[r0 + r];
+            const ResLat<R> &L = lats()[rr.lat];
+            const R rho0 = L.rho0;
+            R stt[5][V];
 #pragma unroll
-            for (int i = 0; i < 5; ++i) res_ld<V>(st + i * n, stt[i]);
-        }
-        const int xb = xoff + x0;
-        const int oo = rr.own * pitch + xb;
-        const int om2 = rr.m2 * pitch + xb, om1 = rr.m1 * pitch + xb, op1 = rr.p1 * pitch + xb, op2 = rr.p2 * pitch + xb;
-        /* x neighbours: the row's other end where the width is a whole number of units, the
-         * images beside the row else */
-        int ox[4];
-        if constexpr (PAIR) {
-            ox[0] = oo + ((xoff == 0 && x0 == 0) ? W - 2 : -2);
-            ox[1] = oo + ((xoff == 0 && x0 + 4 == W) ? 4 - W : 4);
-            ox[2] = ox[3] = 0;
-        } else {
-            const int ro = oo - x0;
-            ox[0] = ro + (x0 >= 2 ? x0 - 2 : x0 - 2 + W);
-            ox[1] = ro + (x0 >= 1 ? x0 - 1 : x0 - 1 + W);
-            ox[2] = ro + (x0 + 1 < W ? x0 + 1 : x0 + 1 - W);
-            ox[3] = ro + (x0 + 2 < W ? x0 + 2 : x0 + 2 - W);
-        }
-        const int wall = rr.flags & 3;
-        const R wsgn = wall == 1 ? R(1) : (wall == 2 ? R(-1) : R(0));
-        const int M = h.q[s] + h.K[s];
-        int ph = phys(s, a0, phase);
-        int pn = ph - h.K[s];
-        if (pn < 0) pn += M;
-        const uint32_t pstride = (uint32_t)h.nslot[s] * rowb;
-        if constexpr (PAIR) {
-            PairNode nd;
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int k = 2 * hh;
-                nd.ux[hh] = make_float2(stt[0][k], stt[0][k + 1]);
-                nd.uy[hh] = make_float2(stt[1][k], stt[1][k + 1]);
-                nd.nom[hh] = make_float2(-stt[2][k], -stt[2][k + 1]);
-                nd.P[hh] = make_float2(stt[2][k] * stt[3][k], stt[2][k + 1] * stt[3][k + 1]);
-                nd.B[hh] = make_float2(stt[4][k], stt[4][k + 1]);
-                if constexpr (FORCE) nd.dr[hh] = make_float2(L.dt * stt[3][k], L.dt * stt[3][k + 1]);
+            for (int i = 0; i < 5; ++i) res_ld<V>(stb + i * V * nu + V * e, stt[i]);
+            R gx = R(0), gy = R(0), dtl = R(0);
+            if constexpr (FORCE) {
+                gx = L.gx;
+                gy = L.gy;
+                dtl = L.dt;
             }
-            const float2 nrho02 = f2(-rho0);
-            auto dec2 = [&](float2 raw, float2 winv2) -> float2 {
-                if constexpr (ST == 1) return fma2(raw, winv2, nrho02);
-                else return raw;
-            };
-#pragma unroll 1
-            for (int a = a0; a < a1; ++a) {
-                const RingPop &rp = tp[a];
-                const T *pl = reinterpret_cast<const T *>(sm + h.off_plane[s] + (uint32_t)ph * pstride);
-                T own[4], yv[3][4], hl[2], hr[2];
-                const float cy = rp.cy2.x, cx = rp.cx2.x;
-                ldn<4>(pl + oo, own);
-                if (cy > 0.0f) {
-                    ldn<4>(pl + om2, yv[0]);
-                    ldn<4>(pl + om1, yv[1]);
-                    ldn<4>(pl + op1, yv[2]);
-                } else if (cy < 0.0f) {
-                    ldn<4>(pl + op2, yv[0]);
-                    ldn<4>(pl + op1, yv[1]);
-                    ldn<4>(pl + om1, yv[2]);
-                }
-                if (cx != 0.0f) {
-                    ld2(pl + ox[0], hl);
-                    ld2(pl + ox[1], hr);
-                }
-                float2 v[2], c[2];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) v[hh] = dec2(make_float2(to_r(own[2 * hh]), to_r(own[2 * hh + 1])), rp.winv2);
-                PairC pc;
-                PairC2 pc2;
-                pc.cx2 = rp.cx2;
-                pc.cy2 = rp.cy2;
-                pc.ncx2 = rp.ncx2;
-                pc.nacy2 = rp.nacy2;
-                pc.ky2 = rp.ky2;
-                pc.crx = -rp.ncx2.x;
-                pc.kx = rp.kx;
-                pc.ystep = cy != 0.0f;
-                if constexpr (FORCE) pc2.gxi2 = f2(xi_dot(cx, cy, L.gx, L.gy));
-                auto xh = [&](int i) -> float { return dec(i < 2 ? hl[i] : hr[i - 2], rp.winv2.x, rho0); };
-                auto yw = [&](int hh, int i) -> float2 {
-                    return dec2(make_float2(to_r(yv[i][2 * hh]), to_r(yv[i][2 * hh + 1])), rp.winv2);
+            /* byte offsets, relative to a plane, of the unit and of its y neighbours; the x
+             * neighbours relative to the unit: the row's other end where the width is a
+             * whole number of units, the images beside the row else */
+            const uint32_t xb = (uint32_t)x0 * (uint32_t)sizeof(T);
+            const uint32_t oo = rr.own * pitchb + xb;
+            const uint32_t m2 = rr.m2 * pitchb + xb, m1 = rr.m1 * pitchb + xb, p1 = rr.p1 * pitchb + xb, p2 = rr.p2 * pitchb + xb;
+            int ox[4] = {0, 0, 0, 0};
+            if constexpr (PAIR) {
+                ox[0] = (!images && x0 == 0) ? W - 2 : -2;
+                ox[1] = (!images && x0 + 4 == W) ? 4 - W : 4;
+            } else {
+                ox[0] = x0 >= 2 ? -2 : W - 2;
+                ox[1] = x0 >= 1 ? -1 : W - 1;
+                ox[2] = x0 + 1 < W ? 1 : 1 - W;
+                ox[3] = x0 + 2 < W ? 2 : 2 - W;
+            }
+            const bool special = (rr.flags & (3 | RES_PUSH)) != 0;
+            const R wsgn = (rr.flags & 1) ? R(1) : ((rr.flags & 2) ? R(-1) : R(0));
+            const int iy1 = min(hi, lo + (g + 1) * rpg);
+            for (int iy = lo + g * rpg; iy < iy1; ++iy) {
+                const int a0 = iy * n;
+                int ph = a0 + phase;
+                ph = ph >= M ? ph - M : ph;
+                int pn = ph - K;
+                pn = pn < 0 ? pn + M : pn;
+                const uint32_t pa = base + (uint32_t)ph * pstride, pw = base + (uint32_t)pn * pstride;
+                const Pop *ta = tp + a0;
+                const R cy = PO::cy(*ta);
+                /* the window rows j - 2s, j - s, j + s, s = sign(xi_y) */
+                const bool up = cy > R(0);
+                const uint32_t w0 = up ? m2 : p2, w1 = up ? m1 : p1, w3 = up ? p1 : m1;
+                /* what follows a population's update on wall rows (the unrounded wall-bound
+                 * value is kept) and on rows other blocks read */
+                auto finish = [&](int a, const R (&dn)[V], const T (&ev)[V], uint32_t dst) {
+                    put(at(dst - xb), x0, W, images, ev);
+                    if (special) {
+                        if (!EXACT && cy * wsgn < R(0)) {
+                            const int i = (rr.flags & 2) ? a - (h.q[s] - h.nh[s]) : a;
+                            res_st<V>(reinterpret_cast<R *>(res_smem + h.off_wall) + ((rr.wallord * h.nhmax + i) * upr + x0 / V) * V, dn);
+                        }
+                        if (CL && (rr.flags & RES_PUSH)) {
+                            int k = a + phase - K;   /* physical plane written */
+                            k = k < 0 ? k + M : (k >= M ? k - M : k);
+                            push(h, s, k, r0 + r, 0, x0, ev);
+                        }
+                    }
                 };
-                pair_increment<FORCE>(pc, pc2, nd, v, xh, yw, c);
-                float2 dn[2];
+                if constexpr (PAIR) {
+                    const RingPop &pr = *ta;
+                    const float2 cy2 = pr.cy2, nacy2 = pr.nacy2, ky2 = pr.ky2;
+                    const bool hy = nacy2.x != 0.0f;
+                    float2 ux[2], uy[2], om[2], P[2], B[2], dr[2];
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) dn[hh] = add2(v[hh], c[hh]);
-                T ev[4];
-                if constexpr (ST == 1) {
-                    const float2 e0 = mul2(rp.w2, add2(f2(rho0), dn[0])), e1 = mul2(rp.w2, add2(f2(rho0), dn[1]));
-                    ev[0] = e0.x, ev[1] = e0.y, ev[2] = e1.x, ev[3] = e1.y;
+                    for (int k = 0; k < 2; ++k) {
+                        ux[k] = make_float2(stt[0][2 * k], stt[0][2 * k + 1]);
+                        uy[k] = make_float2(stt[1][2 * k], stt[1][2 * k + 1]);
+                        om[k] = make_float2(-stt[2][2 * k], -stt[2][2 * k + 1]);
+                        P[k] = make_float2(stt[2][2 * k] * stt[3][2 * k], stt[2][2 * k + 1] * stt[3][2 * k + 1]);
+                        B[k] = make_float2(stt[4][2 * k], stt[4][2 * k + 1]);
+                        if constexpr (FORCE) dr[k] = make_float2(dtl * stt[3][2 * k], dtl * stt[3][2 * k + 1]);
+                    }
+                    const float2 nrho02 = f2(-rho0);
+                    auto pop = [&](int ix, auto sxc) {
+                        constexpr int SX = decltype(sxc)::value;
+                        const RingPop &px = tp[ix];   /* the abscissa's constants: the same in every lane */
+                        const uint32_t src = pa + (uint32_t)ix * pstride;
+                        float2 w2 = f2(1.0f), winv2 = f2(1.0f);
+                        if constexpr (ST == 1) {
+                            w2 = ta[ix].w2;
+                            winv2 = ta[ix].winv2;
+                        }
+                        auto dec2 = [&](T a, T b) -> float2 {
+                            const float2 raw = make_float2(to_r(a), to_r(b));
+                            if constexpr (ST == 1) return fma2(raw, winv2, nrho02);
+                            else return raw;
+                        };
+                        T own[4];
+                        ldn<4>(at(src + oo), own);
+                        float2 v[2], c[2];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) v[k] = dec2(own[2 * k], own[2 * k + 1]);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            float2 eu;
+                            if constexpr (SX == 0) eu = mul2(cy2, uy[k]);
+                            else eu = fma2(cy2, uy[k], mul2(px.cx2, ux[k]));
+                            const float2 t = fma2(mul2(f2(0.5f), eu), eu, eu);
+                            c[k] = fma2(om[k], v[k], fma2(P[k], t, B[k]));
+                            if constexpr (FORCE) {
+                                const float2 gxi2 = f2(xi_dot(px.cx2.x, cy2.x, gx, gy));
+                                c[k] = fma2(dr[k], fma2(gxi2, eu, gxi2), c[k]);
+                            }
+                        }
+                        if constexpr (SX != 0) {
+                            T hl[2], hr[2];
+                            ld2(at(src + oo) + ox[0], hl);
+                            ld2(at(src + oo) + ox[1], hr);
+                            const float2 hl2 = dec2(hl[0], hl[1]), hr2 = dec2(hr[0], hr[1]);
+                            const float kx = px.kx;
+                            float D[4];
+                            float d[6], nn[6], m[5];
+                            if constexpr (SX > 0) {
+                                d[0] = hl2.y - hl2.x;
+                                d[1] = v[0].x - hl2.y;
+                                d[2] = v[0].y - v[0].x;
+                                d[3] = v[1].x - v[0].y;
+                                d[4] = v[1].y - v[1].x;
+                                d[5] = hr2.x - v[1].y;
+                            } else {
+                                d[0] = v[0].x - hl2.y;
+                                d[1] = v[0].y - v[0].x;
+                                d[2] = v[1].x - v[0].y;
+                                d[3] = v[1].y - v[1].x;
+                                d[4] = hr2.x - v[1].y;
+                                d[5] = hr2.y - hr2.x;
+                            }
+#pragma unroll
+                            for (int i = 0; i < 6; ++i) nn[i] = neg_part(d[i]);
+#pragma unroll
+                            for (int i = 0; i < 5; ++i) m[i] = minmod_n(d[i], d[i + 1], nn[i], nn[i + 1]);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) D[k] = fmaf(SX > 0 ? kx : -kx, m[k + 1] - m[k], d[k + 1]);
+                            c[0] = fma2(px.ncx2, make_float2(D[0], D[1]), c[0]);
+                            c[1] = fma2(px.ncx2, make_float2(D[2], D[3]), c[1]);
+                        }
+                        if (hy) {
+                            T y0[4], y1[4], y3[4];
+                            ldn<4>(at(src + w0), y0);
+                            ldn<4>(at(src + w1), y1);
+                            ldn<4>(at(src + w3), y3);
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                const float2 b0 = dec2(y0[2 * k], y0[2 * k + 1]), b1 = dec2(y1[2 * k], y1[2 * k + 1]);
+                                const float2 b3 = dec2(y3[2 * k], y3[2 * k + 1]);
+                                const float2 d0 = sub2(b1, b0), d1 = sub2(v[k], b1), d2 = sub2(b3, v[k]);
+                                float2 ma, mb;
+                                {
+                                    const float l = fminf(d1.x, 0.0f), u2 = fmaxf(d1.x, 0.0f);
+                                    ma.x = fminf(fmaxf(d0.x, l), u2);
+                                    mb.x = fminf(fmaxf(d2.x, l), u2);
+                                }
+                                {
+                                    const float l = fminf(d1.y, 0.0f), u2 = fmaxf(d1.y, 0.0f);
+                                    ma.y = fminf(fmaxf(d0.y, l), u2);
+                                    mb.y = fminf(fmaxf(d2.y, l), u2);
+                                }
+                                c[k] = fma2(nacy2, fma2(ky2, sub2(mb, ma), d1), c[k]);
+                            }
+                        }
+                        const float2 dn0 = add2(v[0], c[0]), dn1 = add2(v[1], c[1]);
+                        float2 e0 = dn0, e1 = dn1;
+                        if constexpr (ST == 1) {
+                            e0 = mul2(w2, add2(f2(rho0), dn0));
+                            e1 = mul2(w2, add2(f2(rho0), dn1));
+                        }
+                        const uint32_t dst = pw + (uint32_t)ix * pstride + oo;
+                        if (!special && !images) {
+                            pair_st<ST>(at(dst), e0, e1);
+                        } else {
+                            const T ev[4] = {from_r<T>(e0.x), from_r<T>(e0.y), from_r<T>(e1.x), from_r<T>(e1.y)};
+                            const R dn[4] = {dn0.x, dn0.y, dn1.x, dn1.y};
+                            finish(a0 + ix, dn, ev, dst);
+                        }
+                    };
+                    int ix = 0;
+#pragma unroll 1
+                    for (; ix < n / 2; ++ix) pop(ix, std::integral_constant<int, -1>{});
+                    if (n & 1) {
+                        pop(ix, std::integral_constant<int, 0>{});
+                        ++ix;
+                    }
+#pragma unroll 1
+                    for (; ix < n; ++ix) pop(ix, std::integral_constant<int, 1>{});
                 } else {
-                    ev[0] = from_r<T>(dn[0].x), ev[1] = from_r<T>(dn[0].y), ev[2] = from_r<T>(dn[1].x), ev[3] = from_r<T>(dn[1].y);
+                    const R ux = stt[0][0], uy = stt[1][0], om = stt[2][0], rho = stt[3][0], rhod = stt[4][0];
+                    const R usq = usq_of(ux, uy);
+                    R gu = R(0), dtr = R(0);
+                    if constexpr (FORCE) {
+                        gu = xi_dot(gx, gy, ux, uy);
+                        dtr = dtl * rho;
+                    }
+                    const R cry = ta->cry, ky = ta->ky;
+                    /* the window runs from upwind for either sign: for xi_y < 0 every difference,
+                     * and so the flux difference, is the printed one with its sign changed */
+                    const R nacry = up ? -cry : cry;
+                    const bool hy = cry != R(0);
+#pragma unroll 1
+                    for (int ix = 0; ix < n; ++ix) {
+                        const uint32_t src = pa + (uint32_t)ix * pstride;
+                        const Pop &px = tp[ix];
+                        const R w = ta[ix].w, winv = ta[ix].winv, cx = px.cx, crx = px.crx;
+                        const T *c0 = at(src + oo);
+                        const R v = dec(*c0, winv, rho0);
+                        const R eu = xi_dot(cx, cy, ux, uy);
+                        R inc = om * (deq(rhod, rho, eu, usq) - v);
+                        if (crx != R(0)) {
+                            R d0, d1, d2, kf;
+                            const R l1 = dec(c0[ox[1]], winv, rho0), q0 = dec(c0[ox[2]], winv, rho0);
+                            R far;
+                            if (crx > R(0)) {
+                                far = dec(c0[ox[0]], winv, rho0);
+                                d0 = l1 - far;
+                                d1 = v - l1;
+                                d2 = q0 - v;
+                                kf = px.kx;
+                            } else {
+                                far = dec(c0[ox[3]], winv, rho0);
+                                d0 = v - l1;
+                                d1 = q0 - v;
+                                d2 = far - q0;
+                                kf = -px.kx;
+                            }
+                            inc = fma(-crx, fma(kf, res_minmod(d1, d2) - res_minmod(d0, d1), d1), inc);
+                        }
+                        if (hy) {
+                            const R b0 = dec(*at(src + w0), winv, rho0), b1 = dec(*at(src + w1), winv, rho0);
+                            const R b3 = dec(*at(src + w3), winv, rho0);
+                            const R d0 = b1 - b0, d1 = v - b1, d2 = b3 - v;
+                            inc = fma(nacry, fma(ky, res_minmod(d1, d2) - res_minmod(d0, d1), d1), inc);
+                        }
+                        if constexpr (FORCE) inc = force_inc(dtr, xi_dot(cx, cy, gx, gy), eu, gu, inc);
+                        const R dn = v + inc;
+                        T ev[1];
+                        if (sr) ev[0] = encode_sr<ST>(dn, w, rho0, sr_bits(x0, (int)rr.j, W, a0 + ix, step_key));
+                        else ev[0] = encode<ST>(dn, w, rho0);
+                        const uint32_t dst = pw + (uint32_t)ix * pstride + oo;
+                        if (!special) {
+                            *at(dst) = ev[0];
+                        } else {
+                            const R dna[1] = {dn};
+                            finish(a0 + ix, dna, ev, dst);
+                        }
+                    }
                 }
-                put(plane(s, pn), rr.own, x0, ev);
-                if (rr.flags & (3 | RES_PUSH)) finish(s, a, pn, rr, rowi, x0, wsgn * cy, {dn[0].x, dn[0].y, dn[1].x, dn[1].y}, ev);
-                ph = ph + 1 == M ? 0 : ph + 1;
-                pn = pn + 1 == M ? 0 : pn + 1;
-            }
-        } else {
-            const R ux = stt[0][0], uy = stt[1][0], om = stt[2][0], rho = stt[3][0], rhod = stt[4][0];
-            const R usq = usq_of(ux, uy), gu = xi_dot(L.gx, L.gy, ux, uy);
-#pragma unroll 2
-            for (int a = a0; a < a1; ++a) {
-                const Pop &p = tp[a];
-                const T *pl = reinterpret_cast<const T *>(sm + h.off_plane[s] + (uint32_t)ph * pstride);
-                const R winv = p.winv, crx = p.crx, cry = p.cry;
-                const R v = dec(pl[oo], winv, rho0);
-                R Dx = R(0), Dy = R(0);
-                if (crx != R(0)) {
-                    const R l[2] = {dec(pl[ox[0]], winv, rho0), dec(pl[ox[1]], winv, rho0)};
-                    const R rr2[2] = {dec(pl[ox[2]], winv, rho0), dec(pl[ox[3]], winv, rho0)};
-                    const R vv[1] = {v};
-                    R D[1];
-                    x_flux_diff<1>(crx, p.kx, l, vv, rr2, D);
-                    Dx = D[0];
-                }
-                if (cry > R(0)) {
-                    const R ym2 = dec(pl[om2], winv, rho0), ym1 = dec(pl[om1], winv, rho0), yp1 = dec(pl[op1], winv, rho0);
-                    const R d0 = ym1 - ym2, d1 = v - ym1, d2 = yp1 - v, n1 = neg_part(d1);
-                    Dy = fma(p.ky, minmod_n(d1, d2, n1, neg_part(d2)) - minmod_n(d0, d1, neg_part(d0), n1), d1);
-                } else if (cry < R(0)) {
-                    const R ym1 = dec(pl[om1], winv, rho0), yp1 = dec(pl[op1], winv, rho0), yp2 = dec(pl[op2], winv, rho0);
-                    const R e0 = v - ym1, e1 = yp1 - v, e2 = yp2 - yp1, n1 = neg_part(e1);
-                    Dy = fma(-p.ky, minmod_n(e1, e2, n1, neg_part(e2)) - minmod_n(e0, e1, neg_part(e0), n1), e1);
-                }
-                const R eu = xi_dot(p.cx, p.cy, ux, uy);
-                R inc = om * (deq(rhod, rho, eu, usq) - v);
-                inc = fma(-crx, Dx, inc);
-                inc = fma(-cry, Dy, inc);
-                if constexpr (FORCE) inc = force_inc(L.dt * rho, xi_dot(p.cx, p.cy, L.gx, L.gy), eu, gu, inc);
-                const R dn = v + inc;
-                T ev[1];
-                if (sr) ev[0] = encode_sr<ST>(dn, p.w, rho0, sr_bits(x0, (int)rr.j, W, a, step_key));
-                else ev[0] = encode<ST>(dn, p.w, rho0);
-                put(plane(s, pn), rr.own, x0, ev);
-                if (rr.flags & (3 | RES_PUSH)) finish(s, a, pn, rr, rowi, x0, wsgn * p.cy, {dn}, ev);
-                ph = ph + 1 == M ? 0 : ph + 1;
-                pn = pn + 1 == M ? 0 : pn + 1;
             }
         }
-    }
-    /* wall rows keep the unrounded wall-bound values; rows next to another block's are
-     * stored there too */
-    __device__ __forceinline__ void finish(int s, int a, int pn, const ResRow &rr, int rowi, int x0, R xn, const R (&dn)[V],
-                                           const T (&ev)[V])
-    {
-        if (!EXACT && xn < R(0)) {
-            const int i = (rr.flags & 2) ? a - (h.q[s] - h.nh[s]) : a;
-            R *wb = reinterpret_cast<R *>(sm + h.off_wall) + (((size_t)rr.wallord * h.nhmax + i) * upr + x0 / V) * V;
-            res_st<V>(wb, dn);
-        }
-        if (CL && (rr.flags & RES_PUSH)) push(s, pn, pushes(rowi, 0), x0, ev);
     }
 };
 
@@ -553,8 +654,7 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
     using T = typename RT::T;
     using R = typename RT::R;
     namespace cg = cooperative_groups;
-    extern __shared__ __align__(16) unsigned char res_smem[];
-    ResHead &h = *reinterpret_cast<ResHead *>(res_smem);
+    const ResHead &h = res_head();
     __shared__ int part_sh;
     const int tid = threadIdx.x;
     for (;;) {
@@ -576,7 +676,6 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
             reinterpret_cast<uint4 *>(res_smem)[k] = reinterpret_cast<const uint4 *>(pp)[k];
         if constexpr (CL) cg::this_cluster().sync();   /* every block is running: its memory may be stored into */
         else __syncthreads();
-        RT rt(h, res_smem);
         const ResGRow *grow = reinterpret_cast<const ResGRow *>(pp + h.off_grow);
         const int nlat = h.nlat;
         /* level read: parameters [lat][base]; level written: that of an even or odd count */
@@ -605,13 +704,16 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
         }
         typename RT::Pop *pops = reinterpret_cast<typename RT::Pop *>(res_smem + h.off_pop);
         if constexpr (PAIR) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(&tabs[ids[0]]);
-            for (int k = tid; k < (int)(sizeof(RingTab) / 16); k += RES_THREADS) reinterpret_cast<uint4 *>(pops)[k] = src[k];
+            constexpr int NW = (int)(sizeof(RingPop) / 16);
+            for (int k = tid; k < (h.q[0] + h.q[1]) * NW; k += RES_THREADS) {
+                const int i = k / NW, s = i < h.q[0] ? 0 : 1;
+                reinterpret_cast<uint4 *>(pops)[k] = reinterpret_cast<const uint4 *>(&tabs[ids[0]].pop[s][s ? i - h.q[0] : i])[k - i * NW];
+            }
         } else {
             const StepParams<R> &p = par2[2 * (size_t)ids[0] + base];
-            for (int k = tid; k < 2 * LB_QMAX; k += RES_THREADS) {
-                const SetConst<R> &c = p.set[k / LB_QMAX];
-                const int a = k % LB_QMAX;
+            for (int k = tid; k < h.q[0] + h.q[1]; k += RES_THREADS) {
+                const SetConst<R> &c = p.set[k < h.q[0] ? 0 : 1];
+                const int a = k < h.q[0] ? k : k - h.q[0];
                 pops[k] = ResPop<R>{c.cx[a], c.cy[a], c.crx[a], c.cry[a], c.kx[a], c.ky[a], c.w[a], c.winv[a],
                                     c.wcx[a], c.wcy[a], c.wxx[a], c.wxy[a], c.wyy[a], c.hxx[a], c.hxy[a], c.hyy[a]};
             }
@@ -627,23 +729,24 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
                 const ResGRow g = grow[r0 + r];
                 const StepParams<R> &p = par2[2 * (size_t)g.lat + base];
                 const T v = static_cast<const T *>(p.fin[s])[(size_t)a * p.plane + (size_t)g.j * p.pitch + x + LB_GHOST];
-                T *row = rt.plane(s, a) + rt.rows[r0 + r].own * rt.pitch + rt.xoff;
+                const ResRow rr = RT::rows()[r0 + r];
+                T *row = RT::at(RT::place(h, s, a, rr.own));
                 row[x] = v;
-                if (rt.xoff != 0) {
+                if (h.xoff != 0) {
                     if (x < 2) row[x + W] = v;
                     if (x >= W - 2) row[x - W] = v;
                 }
                 if constexpr (CL) {
-                    if (rt.rows[r0 + r].flags & RES_PUSH) {
-                        const uint16_t *to = rt.pushes(r0 + r, 0);
+                    if (rr.flags & RES_PUSH) {
+                        const uint16_t *to = reinterpret_cast<const uint16_t *>(res_smem + h.off_push) + 8 * (r0 + r);
                         for (int t = 0; t < 2; ++t) {
                             const int rk = to[2 * t];
                             if (rk == RES_NONE) continue;
                             const ResRank &kk = h.rank[rk];
-                            T *local = reinterpret_cast<T *>(res_smem + kk.off_plane[s] + (uint32_t)a * kk.nslot[s] * rt.rowb);
-                            T *rrow = cg::this_cluster().map_shared_rank(local, rk) + to[2 * t + 1] * rt.pitch + rt.xoff;
+                            T *local = RT::at(kk.off_plane[s] + ((uint32_t)(a * kk.nslot[s] + to[2 * t + 1]) * (uint32_t)h.pitch + (uint32_t)h.xoff) * (uint32_t)sizeof(T));
+                            T *rrow = cg::this_cluster().map_shared_rank(local, rk);
                             rrow[x] = v;
-                            if (rt.xoff != 0) {
+                            if (h.xoff != 0) {
                                 if (x < 2) rrow[x + W] = v;
                                 if (x >= W - 2) rrow[x - W] = v;
                             }
@@ -654,26 +757,27 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
         }
         __syncthreads();
         const bool sr = !PAIR && h.sr != 0;
+        const int warp = tid / 32, nwall = h.nwall[0] + h.nwall[1], nsh = h.nsh[0] + h.nsh[1];
         for (int st = 0;; ++st) {
-            if (st == 0) rt.template moments<false>(phase);
-            else rt.template moments<true>(phase);
+            if (st > 0 && nwall > 0) {
+                RT::walls(phase);
+                __syncthreads();
+            }
+            RT::moments(phase);
             __syncthreads();
             if (st == nsteps) break;
-            rt.views(phase);
+            if (nsh > 0) RT::views(phase);
             if constexpr (CL) cg::this_cluster().sync();
-            else __syncthreads();
+            else if (nsh > 0) __syncthreads();
             for (int rd = 0; rd < h.rounds; ++rd) {
-                const int nc1 = (h.nunit[1] + 31) / 32, nc0 = (h.nunit[0] + 31) / 32;
-                const int u1 = nc1 * h.G[1], u0 = nc0 * h.G[0];
-                for (int u = rt.warp; u < u1 + u0; u += RES_WARPS) {
-                    const int s = u < u1 ? 1 : 0;
-                    const int k = s ? u : u - u1, nc = s ? nc1 : nc0;
-                    const int g = k / nc, chunk = k - g * nc;
-                    const int lo = rd * h.K[s], hi = min(h.q[s], lo + h.K[s]);
-                    const int per = (h.K[s] + h.G[s] - 1) / h.G[s];
-                    const int a0 = lo + g * per, a1 = min(hi, a0 + per);
-                    if (a0 < a1) rt.update(s, chunk, a0, a1, phase[s], step0 + (uint32_t)st + 1u, sr);
-                }
+                /* set 1 first: its items are the longer ones; the warps go on in set 0 where
+                 * set 1 left off */
+                const int kr1 = h.kr[1], kr0 = h.kr[0];
+                const int lo1 = min(h.n[1], rd * kr1), hi1 = min(h.n[1], lo1 + kr1);
+                const int lo0 = min(h.n[0], rd * kr0), hi0 = min(h.n[0], lo0 + kr0);
+                const int units1 = (h.nunit[1] * ((hi1 - lo1 + h.rpg[1] - 1) / h.rpg[1]) + 31) / 32;
+                RT::update(1, lo1, hi1, phase[1], warp, step0 + (uint32_t)st + 1u, sr);
+                RT::update(0, lo0, hi0, phase[0], (warp + RES_WARPS - units1 % RES_WARPS) % RES_WARPS, step0 + (uint32_t)st + 1u, sr);
                 if (rd + 1 < h.rounds) {
                     if constexpr (CL) cg::this_cluster().sync();
                     else __syncthreads();
@@ -704,17 +808,17 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
                     const int q = h.q[t], per = nr * W, total = q * per;
                     for (int k = tid; k < total; k += RES_THREADS) {
                         const int a = k / per, i = k - a * per, r = i / W, x = i - r * W;
-                        const ResRow rr = rt.rows[r0 + r];
+                        const ResRow rr = RT::rows()[r0 + r];
                         if (view && !(rr.flags & RES_SHADOW)) continue;
                         const ResGRow g = grow[r0 + r];
                         const StepParams<R> &p = par2[2 * (size_t)g.lat + sel];
                         T v;
                         if (!view) {
-                            v = rt.plane(t, rt.phys(t, a, phase[t]))[rr.own * rt.pitch + rt.xoff + x];
-                        } else {   /* as views() formed it */
+                            v = RT::at(RT::place(h, t, RT::phys(h, t, a, phase[t]), rr.own))[x];
+                        } else {   /* as views() forms it */
                             const R *hs = reinterpret_cast<const R *>(res_smem + h.off_herm) +
-                                          ((size_t)rr.shord * rt.upr + x / RT::V) * 6 * RT::V + x % RT::V;
-                            const typename RT::Pop &pc = pops[t * LB_QMAX + a];
+                                          (rr.shord * RT::upr_of(W) + x / RT::V) * 6 * RT::V + x % RT::V;
+                            const typename RT::Pop &pc = RT::pops(t)[a];
                             using PO = typename RT::PO;
                             R d = fma(hs[RT::V], PO::cx(pc), hs[0]);
                             d = fma(hs[2 * RT::V], PO::cy(pc), d);
@@ -738,11 +842,11 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
                     if (!aout) continue;
                     const R rho0 = p.rho0;
                     R rd = R(0), jx = R(0), jy = R(0);
-                    const int off = rt.rows[r0 + r].own * rt.pitch + rt.xoff + x;
+                    const int own = RT::rows()[r0 + r].own;
                     for (int a = 0; a < q; ++a) {
-                        const typename RT::Pop &pc = pops[s * LB_QMAX + a];
+                        const typename RT::Pop &pc = RT::pops(s)[a];
                         using PO = typename RT::PO;
-                        const R d = decode<ST>(rt.plane(s, rt.phys(s, a, phase[s]))[off], PO::winv(pc), rho0);
+                        const R d = decode<ST>(RT::at(RT::place(h, s, RT::phys(h, s, a, phase[s]), own))[x], PO::winv(pc), rho0);
                         rd = fma(PO::w(pc), d, rd);
                         jx = fma(PO::wcx(pc), d, jx);
                         jy = fma(PO::wcy(pc), d, jy);
