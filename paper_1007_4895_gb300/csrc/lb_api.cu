@@ -1063,7 +1063,7 @@ int ensure_learned_buffers(lb_ctx *c)
     const size_t N = (size_t)c->nx * c->ny;
     /* each buffer on its own, so a failed allocation is retried by the next call (what
      * did succeed stays owned by the context) */
-    if (!c->d_mom) c->d_mom = static_cast<float *>(own(c, 9 * N * sizeof(float)));
+    if (!c->d_mom) c->d_mom = static_cast<float *>(own(c, N * sizeof(float)));
     if (!c->d_feat) c->d_feat = static_cast<float *>(own(c, 8 * N * sizeof(float)));
     if (!c->d_p) c->d_p = static_cast<float *>(own(c, N * sizeof(float)));
     if (!c->d_tp) c->d_tp = static_cast<float *>(own(c, (size_t)c->ny * c->ntx * sizeof(float)));
@@ -1075,8 +1075,7 @@ template <typename R>
 int features_t(lb_ctx *c, float *dst)
 {
     StepParams<R> p = make_params<R>(c, c->cur, c->cur, c->t);
-    lbk::launch_moments<R>(c->store, p, LB_M_ALL, c->d_mom, 0, c->stream);
-    lbk::launch_features<R>(p, c->d_mom, dst, c->stream);
+    lbk::launch_features<R>(c->store, p, c->d_mom, dst, c->stream);
     return launch_check(c, "features");
 }
 

@@ -149,53 +149,159 @@ __global__ void get_pops_kernel(const __grid_constant__ StepParams<typename Stor
     }
 }
 
-/* Moment fields of every node from its own set: rho, u, P_xy = sum f (xi-u)_x (xi-u)_y,
- * Pi^neq = sum (f - f_eq) xi xi, q = (1/2) sum f |xi - u|^2 (xi - u). The rest-state
- * part w rho0 is summed in closed form (Gaussian moments up to third order, exact for
- * every set), so only deviations enter the sums. */
-template <int ST, typename OUT>
-__global__ void moments_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p, uint32_t mask,
-                               OUT *dst)
+/* Two neighbouring nodes' values of the arithmetic type: packed two-wide instructions for
+ * FP32 */
+template <typename R>
+struct Two {
+    R x, y;
+};
+template <typename R>
+__device__ __forceinline__ Two<R> two(R v) { return {v, v}; }
+__device__ __forceinline__ Two<float> fma_t(Two<float> a, Two<float> b, Two<float> c)
+{
+    const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
+    return {r.x, r.y};
+}
+__device__ __forceinline__ Two<float> mul_t(Two<float> a, Two<float> b)
+{
+    const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+    return {r.x, r.y};
+}
+/* a product that is added to: scalar, because a packed multiply and a packed add are fused
+ * into one rounding whatever the contraction setting */
+__device__ __forceinline__ Two<float> mul_s(Two<float> a, Two<float> b) { return {__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)}; }
+__device__ __forceinline__ Two<double> mul_s(Two<double> a, Two<double> b) { return {a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ Two<float> add_t(Two<float> a, Two<float> b)
+{
+    const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+    return {r.x, r.y};
+}
+__device__ __forceinline__ Two<double> fma_t(Two<double> a, Two<double> b, Two<double> c)
+{
+    return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+__device__ __forceinline__ Two<double> mul_t(Two<double> a, Two<double> b) { return {a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ Two<double> add_t(Two<double> a, Two<double> b) { return {a.x + b.x, a.y + b.y}; }
+template <typename R>
+__device__ __forceinline__ Two<R> neg_t(Two<R> a) { return {-a.x, -a.y}; }
+
+/* Moment fields of two neighbouring nodes of a set of Q populations: rho, u, P_xy = sum f
+ * (xi-u)_x (xi-u)_y, Pi^neq = sum (f - f_eq) xi xi, q = (1/2) sum f |xi - u|^2 (xi - u).
+ * The rest-state part w rho0 is summed in closed form (Gaussian moments up to third order,
+ * exact for every set), so only deviations enter the sums. The number of populations is a
+ * compile-time constant: all loads are in flight at once, the deviations stay in registers
+ * between the two passes and the set's constants come from the parameter block at fixed
+ * offsets (with a run-time count the deviations lived in local memory; one node per thread
+ * was bound by instruction issue, 45 a population). The operations of a node and their
+ * order are those of one node at a time. */
+template <int ST, int Q>
+__device__ __forceinline__ void node_fields(const StepParams<typename Store<ST>::R> &p,
+                                            const SetConst<typename Store<ST>::R> &c, const typename Store<ST>::T *f, int x,
+                                            Two<typename Store<ST>::R> (&vals)[9])
 {
     using T = typename Store<ST>::T;
     using R = typename Store<ST>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (x >= p.nx) return;
-    const int s = p.tmap[(size_t)j * p.ntx + x / LB_TILE_X] & LB_TILE_HIGH;
-    const SetConst<R> &c = p.set[s];
+    using W = Two<R>;
     const size_t plane = p.plane;
-    const T *f = static_cast<const T *>(p.fin[s]) + (size_t)j * p.pitch + x + LB_GHOST;
     const R rho0 = p.rho0;
-    R d[LB_QMAX];
-    R rd = R(0), jx = R(0), jy = R(0);
-    for (int a = 0; a < c.q; ++a) {
-        d[a] = dec_at<ST>(p, f[a * plane], c.winv[a], x + LB_GHOST);
-        rd = fma(c.w[a], d[a], rd);
-        jx = fma(c.wcx[a], d[a], jx);
-        jy = fma(c.wcy[a], d[a], jy);
+    W d[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        T raw[2];
+        ld2(f + a * plane, raw);
+        d[a] = W{dec_at<ST>(p, raw[0], c.winv[a], x + LB_GHOST), dec_at<ST>(p, raw[1], c.winv[a], x + 1 + LB_GHOST)};
     }
-    const R rho = rho0 + rd, ux = jx / rho, uy = jy / rho, usq = ux * ux + uy * uy;
+    W rd = two(R(0)), jx = rd, jy = rd;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        rd = fma_t(two(c.w[a]), d[a], rd);
+        jx = fma_t(two(c.wcx[a]), d[a], jx);
+        jy = fma_t(two(c.wcy[a]), d[a], jy);
+    }
+    const W rho = add_t(two(rho0), rd);
+    const W ux = {jx.x / rho.x, jx.y / rho.y}, uy = {jy.x / rho.x, jy.y / rho.y};
+    const W usq = add_t(mul_s(ux, ux), mul_s(uy, uy)), nusq = neg_t(usq);
     /* rest-state parts: sum w (xi-u)_x (xi-u)_y = ux uy; sum w |xi-u|^2 (xi-u)_x = -ux (4 + u^2) */
-    R pxy = rho0 * ux * uy, nxx = R(0), nxy = R(0), nyy = R(0);
-    R qx = R(-0.5) * rho0 * ux * (R(4) + usq), qy = R(-0.5) * rho0 * uy * (R(4) + usq);
-    for (int a = 0; a < c.q; ++a) {
-        const R cx = c.cx[a], cy = c.cy[a];
-        const R wd = c.w[a] * d[a];
-        const R dx = cx - ux, dy = cy - uy, dd = dx * dx + dy * dy;
-        const R eu = cx * ux + cy * uy;
-        const R wne = c.w[a] * (d[a] - deq(rd, rho, eu, usq));
-        pxy = fma(wd, dx * dy, pxy);
-        nxx = fma(wne, cx * cx, nxx);
-        nxy = fma(wne, cx * cy, nxy);
-        nyy = fma(wne, cy * cy, nyy);
-        qx = fma(R(0.5) * wd, dd * dx, qx);
-        qy = fma(R(0.5) * wd, dd * dy, qy);
+    W pxy = mul_t(mul_t(two(rho0), ux), uy), nxx = two(R(0)), nxy = nxx, nyy = nxx;
+    const W q4 = add_t(two(R(4)), usq);
+    W qx = mul_t(mul_t(two(R(-0.5) * rho0), ux), q4), qy = mul_t(mul_t(two(R(-0.5) * rho0), uy), q4);
+    const W nux = neg_t(ux), nuy = neg_t(uy);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const W cx = two(c.cx[a]), cy = two(c.cy[a]), w = two(c.w[a]);
+        const W wd = mul_t(w, d[a]);
+        const W dx = add_t(cx, nux), dy = add_t(cy, nuy), dd = add_t(mul_s(dx, dx), mul_s(dy, dy));
+        const W eu = add_t(mul_s(cx, ux), mul_s(cy, uy));
+        const W de = fma_t(rho, fma_t(two(R(0.5)), fma_t(eu, eu, nusq), eu), rd);   /* deq */
+        const W wne = mul_t(w, add_t(d[a], neg_t(de)));
+        const R xx = c.cx[a] * c.cx[a], xy = c.cx[a] * c.cy[a], yy = c.cy[a] * c.cy[a];
+        pxy = fma_t(wd, mul_t(dx, dy), pxy);
+        nxx = fma_t(wne, two(xx), nxx);
+        nxy = fma_t(wne, two(xy), nxy);
+        nyy = fma_t(wne, two(yy), nyy);
+        const W hw = mul_t(two(R(0.5)), wd);
+        qx = fma_t(hw, mul_t(dd, dx), qx);
+        qy = fma_t(hw, mul_t(dd, dy), qy);
     }
-    const R vals[9] = {rho, ux, uy, pxy, nxx, nxy, nyy, qx, qy};
+    vals[0] = rho;
+    vals[1] = ux;
+    vals[2] = uy;
+    vals[3] = pxy;
+    vals[4] = nxx;
+    vals[5] = nxy;
+    vals[6] = nyy;
+    vals[7] = qx;
+    vals[8] = qy;
+}
+
+/* node_fields by the set of the nodes x, x + 1 (a warp lies in one tile: no divergence; a
+ * pair never spans two) */
+template <int ST>
+__device__ __forceinline__ void node_fields_any(const StepParams<typename Store<ST>::R> &p, int x, int j,
+                                                Two<typename Store<ST>::R> (&vals)[9])
+{
+    using T = typename Store<ST>::T;
+    const int s = p.tmap[(size_t)j * p.ntx + x / LB_TILE_X] & LB_TILE_HIGH;
+    const T *f = static_cast<const T *>(p.fin[s]) + (size_t)j * p.pitch + x + LB_GHOST;
+    const int q = p.set[s].q;
+    /* the set index a constant too, so that its constants sit at fixed offsets */
+    if (s == 0) {
+        if (q == 9) node_fields<ST, 9>(p, p.set[0], f, x, vals);
+        else if (q == 16) node_fields<ST, 16>(p, p.set[0], f, x, vals);
+        else node_fields<ST, 36>(p, p.set[0], f, x, vals);
+    } else {
+        if (q == 9) node_fields<ST, 9>(p, p.set[1], f, x, vals);
+        else if (q == 16) node_fields<ST, 16>(p, p.set[1], f, x, vals);
+        else node_fields<ST, 36>(p, p.set[1], f, x, vals);
+    }
+}
+
+/* a block is one 128-column tile: 64 threads of two nodes */
+template <int ST, typename OUT>
+__global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) moments_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p,
+                                                     uint32_t mask, OUT *dst)
+{
+    using R = typename Store<ST>::R;
+    const int x = 2 * (blockIdx.x * 64 + threadIdx.x), j = blockIdx.y;
+    if (x >= p.nx) return;
+    Two<R> vals[9];
+    node_fields_any<ST>(p, x, j, vals);
     const size_t N = (size_t)p.nx * p.ny, n = (size_t)j * p.nx + x;
-    int k = 0;
+    const bool both = x + 1 < p.nx;
+    const bool vec = both && (p.nx & 1) == 0 && (reinterpret_cast<uintptr_t>(dst) & (2 * sizeof(OUT) - 1)) == 0;
+    OUT *o = dst + n;
+#pragma unroll
     for (int m = 0; m < 9; ++m)
-        if (mask & (1u << m)) dst[(size_t)(k++) * N + n] = OUT(vals[m]);
+        if (mask & (1u << m)) {
+            const OUT e[2] = {OUT(vals[m].x), OUT(vals[m].y)};
+            if (vec) {
+                st2(o, e);
+            } else {
+                o[0] = e[0];
+                if (both) o[1] = e[1];
+            }
+            o += N;
+        }
 }
 
 /* FP64 sums over every node: mass, |u - u_prev|^2, |u|^2, count of non-finite nodes.
@@ -284,12 +390,59 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Ste
     }
 }
 
-/* Features of the learned placement, from moment fields m [9][ny][nx] (rho, u,
- * P_xy, Pi^neq xx / xy / yy, q): Pi^neq / rho (3), q / rho (2), wall distance / H,
+/* Features of the learned placement: Pi^neq / rho (3), q / rho (2), wall distance / H,
  * local Kn = tau (Eq. (KN), without the dt / 2 shift) and Kn |grad rho| / rho with
- * central differences (one-sided at non-periodic edges). out [8][ny][nx]. */
+ * central differences (one-sided at non-periodic edges). out [8][ny][nx]. The first
+ * kernel forms the seven that a node's own populations give, and leaves its density in
+ * the FP32 scratch field rho; the second adds the gradient from the neighbours'
+ * densities (all nine moment fields went through memory before: 105 us -> 64 us on
+ * 2 097 152 nodes). */
+template <int ST>
+__global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) features_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p, float h,
+                                                      float *__restrict__ rho_out, float *__restrict__ out)
+{
+    using R = typename Store<ST>::R;
+    const int x = 2 * (blockIdx.x * 64 + threadIdx.x), j = blockIdx.y;
+    if (x >= p.nx) return;
+    Two<R> v[9];
+    node_fields_any<ST>(p, x, j, v);
+    const size_t N = (size_t)p.nx * p.ny, n = (size_t)j * p.nx + x;
+    float dw = 1.0f;
+    if (p.wall_diffuse[0] || p.wall_diffuse[1]) {
+        const int d0 = p.wall_diffuse[0] ? j : 1 << 30, d1 = p.wall_diffuse[1] ? p.ny - 1 - j : 1 << 30;
+        dw = (float)min(d0, d1) * h;
+    }
+    float e[8][2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        auto val = [&](int m) { return (float)(k ? v[m].y : v[m].x); };
+        const float rho = val(0), inv = 1.0f / rho;
+        e[0][k] = val(4) * inv;
+        e[1][k] = val(5) * inv;
+        e[2][k] = val(6) * inv;
+        e[3][k] = val(7) * inv;
+        e[4][k] = val(8) * inv;
+        e[5][k] = dw;
+        e[6][k] = p.tau_const ? (float)p.kn_rho : (float)p.kn_rho / rho;
+        e[7][k] = rho;
+    }
+    const bool both = x + 1 < p.nx;
+    const bool vec = both && (p.nx & 1) == 0 && ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(rho_out)) & 7) == 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        float *o = m < 7 ? out + m * N + n : rho_out + n;
+        if (vec) {
+            st2(o, e[m]);
+        } else {
+            o[0] = e[m][0];
+            if (both) o[1] = e[m][1];
+        }
+    }
+}
+
 template <typename R>
-__global__ void features_kernel(const StepParams<R> p, const float *m, float *out)
+__global__ void __launch_bounds__(128) gradient_feature_kernel(const __grid_constant__ StepParams<R> p, float h,
+                                                               const float *__restrict__ m, float *__restrict__ out)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (x >= p.nx) return;
@@ -300,7 +453,6 @@ __global__ void features_kernel(const StepParams<R> p, const float *m, float *ou
         if (p.periodic_y) jj = (jj + p.ny) % p.ny;
         return m[(size_t)jj * p.nx + xx];
     };
-    const float h = (float)p.h_grid;
     float gx, gy;
     {
         const bool lo = !p.periodic_x && x == 0, hi = !p.periodic_x && x == p.nx - 1;
@@ -313,19 +465,7 @@ __global__ void features_kernel(const StepParams<R> p, const float *m, float *ou
         gy = (rho_at(x, jb) - rho_at(x, ja)) / (h * (float)(jb - ja));
     }
     const float kn = p.tau_const ? (float)p.kn_rho : (float)p.kn_rho / rho;
-    float dw = 1.0f;
-    if (p.wall_diffuse[0] || p.wall_diffuse[1]) {
-        const int d0 = p.wall_diffuse[0] ? j : 1 << 30, d1 = p.wall_diffuse[1] ? p.ny - 1 - j : 1 << 30;
-        dw = (float)min(d0, d1) * h;
-    }
     const float inv = 1.0f / rho;
-    out[0 * N + n] = m[4 * N + n] * inv;
-    out[1 * N + n] = m[5 * N + n] * inv;
-    out[2 * N + n] = m[6 * N + n] * inv;
-    out[3 * N + n] = m[7 * N + n] * inv;
-    out[4 * N + n] = m[8 * N + n] * inv;
-    out[5 * N + n] = dw;
-    out[6 * N + n] = kn;
     out[7 * N + n] = kn * sqrtf(gx * gx + gy * gy) * inv;
 }
 
@@ -434,18 +574,20 @@ void launch_moments(int store, const StepParams<R> &p, uint32_t mask, void *dst,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (dst_f64) {
         LB_DISPATCH(store, if constexpr (store_matches<R, ST>())
-                               moments_kernel<ST, double><<<grid, 128, 0, st>>>(p, mask, static_cast<double *>(dst)));
+                               moments_kernel<ST, double><<<grid, 64, 0, st>>>(p, mask, static_cast<double *>(dst)));
     } else {
         LB_DISPATCH(store, if constexpr (store_matches<R, ST>())
-                               moments_kernel<ST, float><<<grid, 128, 0, st>>>(p, mask, static_cast<float *>(dst)));
+                               moments_kernel<ST, float><<<grid, 64, 0, st>>>(p, mask, static_cast<float *>(dst)));
     }
 }
 
 template <typename R>
-void launch_features(const StepParams<R> &p, const float *moments, float *out, void *stream)
+void launch_features(int store, const StepParams<R> &p, float *rho, float *out, void *stream)
 {
     dim3 grid((p.nx + 127) / 128, p.ny);
-    features_kernel<R><<<grid, 128, 0, static_cast<cudaStream_t>(stream)>>>(p, moments, out);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    LB_DISPATCH(store, if constexpr (store_matches<R, ST>()) features_kernel<ST><<<grid, 64, 0, st>>>(p, (float)p.h_grid, rho, out));
+    gradient_feature_kernel<R><<<grid, 128, 0, st>>>(p, (float)p.h_grid, rho, out);
 }
 
 template <typename R>
@@ -462,8 +604,8 @@ void launch_tile_max(const float *pr, int nx, int ny, int ntx, float *out, void 
     tile_max_kernel<<<grid, 64, 0, static_cast<cudaStream_t>(stream)>>>(pr, nx, ny, ntx, out);
 }
 
-template void launch_features<float>(const StepParams<float> &, const float *, float *, void *);
-template void launch_features<double>(const StepParams<double> &, const float *, float *, void *);
+template void launch_features<float>(int, const StepParams<float> &, float *, float *, void *);
+template void launch_features<double>(int, const StepParams<double> &, float *, float *, void *);
 template void launch_hermite_residual<float>(int, const StepParams<float> &, float *, void *);
 template void launch_hermite_residual<double>(int, const StepParams<double> &, float *, void *);
 

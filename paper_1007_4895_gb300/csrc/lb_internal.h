@@ -301,9 +301,9 @@ template <typename R>
 void launch_reduce(int store, const StepParams<R> &p, R *uprev, double *part, unsigned int *counter,
                    double *out, int nblocks, void *stream);
 int reduce_blocks(int nx, int ny, int nsm);
-/* learned placement: features [8][ny][nx] from moment fields [9][ny][nx] (float) */
+/* learned placement: features [8][ny][nx]; rho: scratch [ny][nx] */
 template <typename R>
-void launch_features(const StepParams<R> &p, const float *moments, float *out, void *stream);
+void launch_features(int store, const StepParams<R> &p, float *rho, float *out, void *stream);
 /* ||f - P2 f|| / rho per node (beyond-second-order Hermite content), [ny][nx] */
 template <typename R>
 void launch_hermite_residual(int store, const StepParams<R> &p, float *out, void *stream);
