@@ -441,13 +441,47 @@ __global__ void to_bf16_kernel(const float *th, __nv_bfloat16 *wb)
 }
 
 /* Inference on the tensor cores: mma.sync m16n8k16 with BF16 operands and FP32
- * accumulation. A warp takes 16 nodes at a time. Layer 1 is the 16 x 16 (8 features,
+ * accumulation. A warp takes 32 nodes at a time as two 16-node tiles (two independent
+ * chains, one read of the weight fragments). Layer 1 is the 16 x 16 (8 features,
  * zero-padded) by 16 x 64 product; its GELU outputs are rounded to BF16 and, because
  * the accumulator fragment of two neighbouring 8-column output tiles has exactly the
  * element layout of one 16-wide operand fragment, feed layer 2 from registers; layer 2's
  * GELU outputs meet W3 in FP32 (a dot product over the 64 hidden units, finished across
  * the four lanes that share a row). The weight fragments are built in shared memory
- * once per block. A node with a non-finite feature gets p = NaN. */
+ * once per block. A node with a non-finite feature gets p = NaN.
+ *
+ * What bounds it: the 128 GELUs of a node, on the FP32 and special-function units. They
+ * are evaluated in pairs as
+ *   gelu(a) = max(a, 0) - x E(x),   x = min(|a|, 5.75),   E(x) = erfc(x / sqrt 2) / 2,
+ * with log2 E a polynomial of degree 9 in packed FP32 arithmetic and one exp2 each: 8.5
+ * instructions a value against about 30 of the erf form. The coefficients are a weighted
+ * minimax fit (iteratively reweighted least squares on Chebyshev nodes) of log2 E on
+ * [0, 5.75] that bounds the error of x E by 1e-8; in FP32 the result is within 2.4e-7 of
+ * GELU on [-9, 9] (rms 5.0e-8; the erf form 4.5e-7, rms 6.4e-8), the cut at 5.75 included
+ * (x E = 2.6e-8 there). 2 097 152 nodes: 345 us -> 204 us. */
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 gelu2(float2 a)
+{
+    const float2 x = make_float2(fminf(fabsf(a.x), 5.75f), fminf(fabsf(a.y), 5.75f));
+    constexpr float C[10] = {-0.9999986886978149f,     -1.1511249542236328f,    -0.4591113328933716f,
+                             -0.052710652351379395f,   0.007307772058993578f,   -0.0002848419244401157f,
+                             -0.00014207529602572322f, 3.552617636159994e-05f,  -3.6852788980468176e-06f,
+                             1.509595932702723e-07f};
+    float2 p = make_float2(C[9], C[9]);
+#pragma unroll
+    for (int k = 8; k >= 0; --k) p = __ffma2_rn(p, x, make_float2(C[k], C[k]));
+    float2 e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(p.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(p.y));
+    const float2 r = make_float2(max_nan(a.x, 0.0f), max_nan(a.y, 0.0f));
+    return __ffma2_rn(make_float2(-x.x, -x.y), e, r);
+}
+
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
 {
     asm volatile(
@@ -471,102 +505,131 @@ __device__ __forceinline__ uint32_t pack_bf16_raw(__nv_bfloat16 lo, __nv_bfloat1
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
-__global__ void __launch_bounds__(128) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
-                                                        const float *__restrict__ norm,
-                                                        const float *__restrict__ X, long long n,
-                                                        float *__restrict__ p)
+/* (not inlined: rare, and 32 copies of it would not fit the instruction cache) */
+__device__ __noinline__ uint32_t gelu2_erf_bf16(float2 a) { return pack_bf16(gelu(a.x), gelu(a.y)); }
+
+/* A pair of GELUs rounded to BF16 as the erf form rounds them: a value that lies within 4
+ * FP32 units of a rounding boundary (one in 4096) is formed again in the erf form. (Below
+ * -1.5, where the erf form itself is off by more, the two may round apart; the values are
+ * below 0.1 there.) */
+__device__ __forceinline__ uint32_t gelu2_bf16(float2 a)
+{
+    constexpr float D = 4.76837158e-7f;   /* 2^-21 */
+    const float2 h = gelu2(a);
+    const float2 lo = __fmul2_rn(h, make_float2(1.0f - D, 1.0f - D)), hi = __fmul2_rn(h, make_float2(1.0f + D, 1.0f + D));
+    const uint32_t r = pack_bf16(lo.x, lo.y);
+    return r == pack_bf16(hi.x, hi.y) ? r : gelu2_erf_bf16(a);
+}
+
+__global__ void __launch_bounds__(128, 4) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
+                                                           const float *__restrict__ norm,
+                                                           const float *__restrict__ X, long long n,
+                                                           float *__restrict__ p)
 {
     /* operand fragments of the weights: B[k][n] of layer 1 is W1[n][k] (k < 8, zero
      * above), of layer 2 W2[n][k]; fragment register r of lane l holds the rows
      * 2 (l % 4) + {0, 1} (+ 8 for r = 1) of column l / 4 */
-    __shared__ uint32_t w1f[8][32][2];
-    __shared__ uint32_t w2f[4][8][32][2];
-    __shared__ float b1s[NH], b2s[NH], w3s[NH], nm[2 * NF], b3s;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
+    __shared__ uint32_t w1f[8][32];
+    __shared__ uint2 w2f[4][8][32];
+    __shared__ float2 b1s[NH / 2], b2s[NH / 2], w3s[NH / 2];
+    __shared__ float nm[2 * NF], b3s;
     for (int k = threadIdx.x; k < 8 * 32; k += blockDim.x) {
         const int nt = k / 32, l = k % 32, col = 8 * nt + l / 4, row = 2 * (l % 4);
-        w1f[nt][l][0] = pack_bf16_raw(wb[OFF_W1 + col * NF + row], wb[OFF_W1 + col * NF + row + 1]);
-        w1f[nt][l][1] = pack_bf16_raw(zero, zero);
+        w1f[nt][l] = pack_bf16_raw(wb[OFF_W1 + col * NF + row], wb[OFF_W1 + col * NF + row + 1]);
     }
     for (int k = threadIdx.x; k < 4 * 8 * 32; k += blockDim.x) {
         const int kt = k / 256, nt = (k / 32) % 8, l = k % 32;
         const int col = 8 * nt + l / 4, row = 16 * kt + 2 * (l % 4);
         const __nv_bfloat16 *w = wb + OFF_W2 + col * NH;
-        w2f[kt][nt][l][0] = pack_bf16_raw(w[row], w[row + 1]);
-        w2f[kt][nt][l][1] = pack_bf16_raw(w[row + 8], w[row + 9]);
+        w2f[kt][nt][l] = make_uint2(pack_bf16_raw(w[row], w[row + 1]), pack_bf16_raw(w[row + 8], w[row + 9]));
     }
-    for (int k = threadIdx.x; k < NH; k += blockDim.x) {
-        b1s[k] = __bfloat162float(wb[OFF_B1 + k]);
-        b2s[k] = __bfloat162float(wb[OFF_B2 + k]);
-        w3s[k] = __bfloat162float(wb[OFF_W3 + k]);
+    for (int k = threadIdx.x; k < NH / 2; k += blockDim.x) {
+        auto two = [&](int off) { return make_float2(__bfloat162float(wb[off + 2 * k]), __bfloat162float(wb[off + 2 * k + 1])); };
+        b1s[k] = two(OFF_B1);
+        b2s[k] = two(OFF_B2);
+        w3s[k] = two(OFF_W3);
     }
     if (threadIdx.x < 2 * NF) nm[threadIdx.x] = norm[threadIdx.x];
     if (threadIdx.x == 0) b3s = __bfloat162float(wb[OFF_B3]);
     __syncthreads();
 
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    const long long tiles = (n + 15) / 16;
+    const long long pairs = (n + 31) / 32;
     const long long stride = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < tiles; t += stride) {
-        const long long r0 = 16 * t + g, r1 = r0 + 8;   /* the two nodes (rows) of this lane */
-        /* layer-1 operand: normalised features 2q, 2q + 1 of both rows (columns 8..15 zero) */
-        float x[2][2];
-        bool ok0 = true, ok1 = true;
+    /* features 2q, 2q + 1 of this lane's four nodes (rows g, g + 8 of both tiles) */
+    float xr[4][2];
+    auto fetch = [&](long long t) {
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int f = 2 * q + e;
-            x[0][e] = r0 < n ? (X[(long long)f * n + r0] - nm[f]) / nm[NF + f] : 0.0f;
-            x[1][e] = r1 < n ? (X[(long long)f * n + r1] - nm[f]) / nm[NF + f] : 0.0f;
-            ok0 = ok0 && isfinite(x[0][e]);
-            ok1 = ok1 && isfinite(x[1][e]);
+        for (int k = 0; k < 4; ++k) {
+            const long long r = 32 * t + g + 8 * k;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) xr[k][e] = r < n ? X[(long long)(2 * q + e) * n + r] : nm[2 * q + e];
         }
-        /* a node is usable when all eight features are finite: the four lanes of a row
-         * hold two each */
-        const unsigned m0 = __ballot_sync(0xffffffffu, !ok0), m1 = __ballot_sync(0xffffffffu, !ok1);
-        const unsigned qm = 0xfu << (4 * g);
-        ok0 = !(m0 & qm);
-        ok1 = !(m1 & qm);
-        if (!ok0) x[0][0] = x[0][1] = 0.0f;
-        if (!ok1) x[1][0] = x[1][1] = 0.0f;
-        const uint32_t a1[4] = {pack_bf16(x[0][0], x[0][1]), pack_bf16(x[1][0], x[1][1]), 0u, 0u};
+    };
+    long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (t < pairs) fetch(t);
+    for (; t < pairs; t += stride) {
+        /* layer-1 operands: normalised features (columns 8..15 zero) */
+        uint32_t a1[2][2];
+        bool ok[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float x0 = (xr[k][0] - nm[2 * q]) / nm[NF + 2 * q], x1 = (xr[k][1] - nm[2 * q + 1]) / nm[NF + 2 * q + 1];
+            /* a node is usable when all eight features are finite: the four lanes of a row
+             * hold two each */
+            const unsigned bad = __ballot_sync(0xffffffffu, !(isfinite(x0) && isfinite(x1)));
+            ok[k] = !(bad & (0xfu << (4 * g)));
+            if (!ok[k]) x0 = x1 = 0.0f;
+            a1[k >> 1][k & 1] = pack_bf16(x0, x1);
+        }
+        if (t + stride < pairs) fetch(t + stride);
         /* layer 1 -> GELU -> BF16 operand fragments of layer 2 */
-        uint32_t a2[4][4];
+        uint32_t a2[2][4][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            const uint32_t b[2] = {w1f[nt][lane][0], w1f[nt][lane][1]};
-            mma_bf16(c, a1, b);
-            const int col = 8 * nt + 2 * q;
-            const float h00 = gelu(c[0] + b1s[col]), h01 = gelu(c[1] + b1s[col + 1]);
-            const float h10 = gelu(c[2] + b1s[col]), h11 = gelu(c[3] + b1s[col + 1]);
-            const int kt = nt >> 1, hi = (nt & 1) * 2;
-            a2[kt][hi] = pack_bf16(h00, h01);
-            a2[kt][hi + 1] = pack_bf16(h10, h11);
+            const uint32_t b[2] = {w1f[nt][lane], 0u};
+            const float2 bias = b1s[4 * nt + q];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                const uint32_t a[4] = {a1[m][0], a1[m][1], 0u, 0u};
+                mma_bf16(c, a, b);
+                const int kt = nt >> 1, hi = (nt & 1) * 2;
+                a2[m][kt][hi] = gelu2_bf16(__fadd2_rn(make_float2(c[0], c[1]), bias));
+                a2[m][kt][hi + 1] = gelu2_bf16(__fadd2_rn(make_float2(c[2], c[3]), bias));
+            }
         }
         /* layer 2 -> GELU -> W3 dot product */
-        float z0 = 0.0f, z1 = 0.0f;
-#pragma unroll
+        float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
         for (int nt = 0; nt < 8; ++nt) {
-            float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            float c[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
 #pragma unroll
             for (int kt = 0; kt < 4; ++kt) {
-                const uint32_t b[2] = {w2f[kt][nt][lane][0], w2f[kt][nt][lane][1]};
-                mma_bf16(c, a2[kt], b);
+                const uint2 w = w2f[kt][nt][lane];
+                const uint32_t b[2] = {w.x, w.y};
+#pragma unroll
+                for (int m = 0; m < 2; ++m) mma_bf16(c[m], a2[m][kt], b);
             }
-            const int col = 8 * nt + 2 * q;
-            z0 = fmaf(gelu(c[0] + b2s[col]), w3s[col], z0);
-            z0 = fmaf(gelu(c[1] + b2s[col + 1]), w3s[col + 1], z0);
-            z1 = fmaf(gelu(c[2] + b2s[col]), w3s[col], z1);
-            z1 = fmaf(gelu(c[3] + b2s[col + 1]), w3s[col + 1], z1);
+            const float2 bias = b2s[4 * nt + q], w3 = w3s[4 * nt + q];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const float2 h0 = gelu2(__fadd2_rn(make_float2(c[m][0], c[m][1]), bias));
+                const float2 h1 = gelu2(__fadd2_rn(make_float2(c[m][2], c[m][3]), bias));
+                z[2 * m] = fmaf(h0.y, w3.y, fmaf(h0.x, w3.x, z[2 * m]));
+                z[2 * m + 1] = fmaf(h1.y, w3.y, fmaf(h1.x, w3.x, z[2 * m + 1]));
+            }
         }
-        z0 += __shfl_xor_sync(0xffffffffu, z0, 1);
-        z0 += __shfl_xor_sync(0xffffffffu, z0, 2);
-        z1 += __shfl_xor_sync(0xffffffffu, z1, 1);
-        z1 += __shfl_xor_sync(0xffffffffu, z1, 2);
-        if (q == 0) {
-            if (r0 < n) p[r0] = ok0 ? 1.0f / (1.0f + expf(-(z0 + b3s))) : nanf("");
-            if (r1 < n) p[r1] = ok1 ? 1.0f / (1.0f + expf(-(z1 + b3s))) : nanf("");
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            z[k] += __shfl_xor_sync(0xffffffffu, z[k], 1);
+            z[k] += __shfl_xor_sync(0xffffffffu, z[k], 2);
         }
+        /* lane q of a row's four stores node k = q of its four */
+        const float zq = q == 0 ? z[0] : (q == 1 ? z[1] : (q == 2 ? z[2] : z[3]));
+        const bool okq = q == 0 ? ok[0] : (q == 1 ? ok[1] : (q == 2 ? ok[2] : ok[3]));
+        const long long r = 32 * t + g + 8 * q;
+        if (r < n) p[r] = okq ? 1.0f / (1.0f + expf(-(zq + b3s))) : nanf("");
     }
 }
 
@@ -683,10 +746,10 @@ namespace lbk {
 
 int mlp_infer_dev(lb_mlp *M, const float *x, int64_t n, float *p, void *stream)
 {
-    /* four warps per block, up to 8 blocks per SM resident (152 SMs): each warp walks
-     * its 16-node tiles with a grid stride */
-    const long long tiles = (n + 15) / 16;
-    const unsigned blocks = (unsigned)std::min<long long>((tiles + 3) / 4, 152LL * 8);
+    /* four warps per block, four blocks per SM resident (152 SMs): each warp walks its
+     * 32-node pairs of tiles with a grid stride */
+    const long long pairs = (n + 31) / 32;
+    const unsigned blocks = (unsigned)std::min<long long>((pairs + 3) / 4, 152LL * 4);
     lbm::infer_mma_kernel<<<blocks, 128, 0, static_cast<cudaStream_t>(stream)>>>(M->wb, M->norm, x, (long long)n, p);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LB_OK : mlp_err(LB_ERR_CUDA, std::string("lb_mlp_infer: ") + cudaGetErrorString(e));
