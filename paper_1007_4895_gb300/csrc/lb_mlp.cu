@@ -163,11 +163,11 @@ __global__ void adam_kernel(float *th, float *m, float *v, const float *g, int t
  * distributed shared memory, updates it and stores the new values into every block. Two
  * cluster barriers a batch; sums in a fixed order, so a run repeats bit for bit. The next
  * tile's samples (a gather over the shuffled order) are loaded while this one is computed.
- * Measured: 100 000 samples in batches of 256, one epoch 51.9 ms -> 4.8 ms. */
-constexpr int TR_NC = 8, TR_S = 32, TR_T = 512;
+ * Measured: 100 000 samples in batches of 256, one epoch 51.9 ms -> 4.8 ms with
+ * a cluster of 8 blocks, 4.0 ms with 16 (of which 1 ms is the host's shuffle). */
+constexpr int TR_S = 32, TR_T = 512;
 constexpr int TR_LD = NH + 4;   /* activation and W2 rows in shared memory: conflict-free 16-byte reads */
-constexpr int TR_SL = (NPARAM + TR_NC - 1) / TR_NC;
-static_assert(TR_T == 16 * TR_S && TR_SL <= 2 * TR_T && TR_T == 8 * NH, "thread mapping of the training kernel");
+static_assert(TR_T == 16 * TR_S && TR_T == 8 * NH, "thread mapping of the training kernel");
 
 struct TrainSmem {
     float w1[NH][NF + 4], w2[NH][TR_LD], b1[NH], b2[NH], w3[NH], b3, pad[3];
@@ -191,13 +191,16 @@ __device__ __forceinline__ float *train_param(TrainSmem &s, int k)
 /* Batches of `batch` samples (the last may be short) over samples idx[0 .. count): forward,
  * backward, Adam with step numbers t0 + 1, ...; p of sample idx[k] at its batch's weights
  * goes to pall[k] when pall is not NULL. th, m, v are read at the start and written at the
- * end. Launched as one cluster. */
-__global__ void __cluster_dims__(TR_NC, 1, 1) __launch_bounds__(TR_T, 1)
+ * end. Launched as one cluster of TR_NC blocks. */
+template <int TR_NC>
+__global__ void __launch_bounds__(TR_T, 1)
     train_kernel(float *__restrict__ th, float *__restrict__ m, float *__restrict__ v, const float *__restrict__ norm,
                  const float *__restrict__ X, long long n, const float *__restrict__ Y, const int *__restrict__ idx,
                  int count, int batch, int t0, float lr, float *__restrict__ pall)
 {
     namespace cg = cooperative_groups;
+    constexpr int TR_SL = (NPARAM + TR_NC - 1) / TR_NC;
+    static_assert(TR_SL <= 2 * TR_T, "two parameters of the slice per thread");
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char train_smem[];
     TrainSmem &s = *reinterpret_cast<TrainSmem *>(train_smem);
@@ -458,7 +461,7 @@ __global__ void to_bf16_kernel(const float *th, __nv_bfloat16 *wb)
  * minimax fit (iteratively reweighted least squares on Chebyshev nodes) of log2 E on
  * [0, 5.75] that bounds the error of x E by 1e-8; in FP32 the result is within 2.4e-7 of
  * GELU on [-9, 9] (rms 5.0e-8; the erf form 4.5e-7, rms 6.4e-8), the cut at 5.75 included
- * (x E = 2.6e-8 there). 2 097 152 nodes: 345 us -> 204 us. */
+ * (x E = 2.6e-8 there). 2 097 152 nodes: 345 us -> 201 us. */
 __device__ __forceinline__ float max_nan(float a, float b)
 {
     float r;
@@ -521,7 +524,7 @@ __device__ __forceinline__ uint32_t gelu2_bf16(float2 a)
     return r == pack_bf16(hi.x, hi.y) ? r : gelu2_erf_bf16(a);
 }
 
-__global__ void __launch_bounds__(128, 4) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
+__global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
                                                            const float *__restrict__ norm,
                                                            const float *__restrict__ X, long long n,
                                                            float *__restrict__ p)
@@ -648,7 +651,7 @@ struct lb_mlp {
     int *idx = nullptr;
     float *pall = nullptr;
     double *lpart = nullptr;
-    int idx_cap = 0;
+    int idx_cap = 0, train_blocks = 0;
     int t = 0;
     lb_opts opts{};
     cudaStream_t stream = nullptr;
@@ -705,14 +708,44 @@ int ensure_batch(lb_mlp *M, int B)
     return LB_OK;
 }
 
+cudaLaunchConfig_t train_config(int nc, cudaLaunchAttribute *at, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nc);
+    cfg.blockDim = dim3(lbm::TR_T);
+    cfg.dynamicSmemBytes = sizeof(lbm::TrainSmem);
+    cfg.stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = nc;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+/* blocks of the training cluster: 16 (beyond the portable size; a batch of 256 is then 16
+ * samples a block) where the device takes such a cluster, else 8 */
+int train_cluster()
+{
+    const int smem = (int)sizeof(lbm::TrainSmem);
+    cudaLaunchAttribute at;
+    int n = 0;
+    if (cudaFuncSetAttribute(lbm::train_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+        cudaFuncSetAttribute(lbm::train_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        const cudaLaunchConfig_t cfg = train_config(16, &at, nullptr);
+        if (cudaOccupancyMaxActiveClusters(&n, lbm::train_kernel<16>, &cfg) == cudaSuccess && n > 0) return 16;
+    }
+    cudaGetLastError();
+    if (cudaFuncSetAttribute(lbm::train_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) return 8;
+    cudaGetLastError();
+    return 0;
+}
+
 /* workspace of a training launch over `count` samples, and the kernel's shared memory */
 int ensure_train(lb_mlp *M, int count)
 {
-    if (cudaFuncSetAttribute(lbm::train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(lbm::TrainSmem)) != cudaSuccess) {
-        cudaGetLastError();
-        return mlp_err(LB_ERR_CUDA, "lb_mlp: the training kernel's shared memory was refused");
-    }
+    if (M->train_blocks == 0) M->train_blocks = train_cluster();
+    if (M->train_blocks == 0) return mlp_err(LB_ERR_CUDA, "lb_mlp: the training kernel cannot be resident");
     if (!M->lpart) M->lpart = (double *)mlp_alloc(M, sizeof(double) * lbm::LOSS_BLOCKS);
     if (count > M->idx_cap) {
         /* grow (old buffers stay owned until destroy) */
@@ -746,10 +779,10 @@ namespace lbk {
 
 int mlp_infer_dev(lb_mlp *M, const float *x, int64_t n, float *p, void *stream)
 {
-    /* four warps per block, four blocks per SM resident (152 SMs): each warp walks its
+    /* four warps per block, five blocks per SM resident (152 SMs): each warp walks its
      * 32-node pairs of tiles with a grid stride */
     const long long pairs = (n + 31) / 32;
-    const unsigned blocks = (unsigned)std::min<long long>((pairs + 3) / 4, 152LL * 4);
+    const unsigned blocks = (unsigned)std::min<long long>((pairs + 3) / 4, 152LL * 5);
     lbm::infer_mma_kernel<<<blocks, 128, 0, static_cast<cudaStream_t>(stream)>>>(M->wb, M->norm, x, (long long)n, p);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LB_OK : mlp_err(LB_ERR_CUDA, std::string("lb_mlp_infer: ") + cudaGetErrorString(e));
@@ -832,10 +865,13 @@ int lb_mlp_train(lb_mlp *M, const float *x, const float *y, int64_t n, int32_t e
             const int cnt = (int)std::min<int64_t>(chunk, n - s0);
             if (cudaMemcpyAsync(M->idx, perm.data() + s0, (size_t)cnt * 4, cudaMemcpyHostToDevice, M->stream) != cudaSuccess)
                 return mlp_err(LB_ERR_CUDA, "lb_mlp_train: copy failed");
-            lbm::train_kernel<<<lbm::TR_NC, lbm::TR_T, sizeof(lbm::TrainSmem), M->stream>>>(
-                M->th, M->m, M->v, M->norm, x, (long long)n, y, M->idx, cnt, batch, M->t, lr,
-                last_epoch ? M->pall : nullptr);
-            if (cudaGetLastError() != cudaSuccess) return mlp_err(LB_ERR_CUDA, "lb_mlp_train: launch failed");
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = train_config(M->train_blocks, &at, M->stream);
+            float *pall = last_epoch ? M->pall : nullptr;
+            const cudaError_t le = cudaLaunchKernelEx(
+                &cfg, M->train_blocks == 16 ? lbm::train_kernel<16> : lbm::train_kernel<8>, M->th, M->m, M->v,
+                (const float *)M->norm, x, (long long)n, y, (const int *)M->idx, cnt, (int)batch, M->t, lr, pall);
+            if (le != cudaSuccess) return mlp_err(LB_ERR_CUDA, std::string("lb_mlp_train: ") + cudaGetErrorString(le));
             M->t += (cnt + batch - 1) / batch;
             if (last_epoch) {
                 double part[lbm::LOSS_BLOCKS];
