@@ -143,9 +143,13 @@ typedef struct {
  *   9: 7's arithmetic on every row, the neighbour rows brought into a per-thread ring
  *      of shared-memory slots by asynchronous copies issued two nodes ahead, wall and
  *      shadow-row updates done by the same kernel (FP32 and 16-bit storage);
- *  10: 9's arithmetic in one persistent launch: warps take rows of 128 columns from
- *      per-SM queues (longest rows first), with the population loop unrolled over the
- *      velocity set (D2Q9 with D2Q16 or D2Q36; FP32 and 16-bit storage).
+ *  10: 9's arithmetic in one persistent launch (D2Q9 with D2Q16 or D2Q36; FP32 and 16-bit
+ *      storage): warps take rows of 128 columns from per-SM queues (longest rows first), or,
+ *      where both levels fit L2, blocks take tiles streamed by the tensor memory accelerator.
+ * With variant < 0 a small x-periodic lattice whose rows each use one set advances all the
+ * steps of an lb_step call in one launch with its state in shared memory (LB_IFACE_HERMITE,
+ * one reference density); lb_info then names the layout with the same bits, 9 (FP32 storage)
+ * or 0.
  * A layout this lattice cannot use falls back to 0. All layouts give the same result
  * (0, 2, 3 and 4 the same bits; 1, 5, 6 the same bits as 0 or differing in rounding;
  * 7, 8 and 9 differ from 0 in rounding; 10 the same bits as 9). */
@@ -357,8 +361,10 @@ typedef struct lb_batch lb_batch;
  * opts.rho0; every lattice needs opts.iface = LB_IFACE_HERMITE, reduce_every = 0, walls
  * without oscillation (omega = 0) and no pressure sides (else LB_ERR_INVALID, checked
  * before any device work). The kernel runs on opts[0].stream; device memory comes from
- * opts[0]'s allocator. Lattices start from rest (rho0, u = 0). lb_batch_create times
- * block sizes 128 / 256 / 512 on the batch and keeps the fastest. */
+ * opts[0]'s allocator. Lattices start from rest (rho0, u = 0). Lattices that fit a block's
+ * shared memory are bundled and stay there for all steps of a launch; else FP32 and 16-bit
+ * batches run on layout 10's rows, and for FP64 lb_batch_create times block sizes 128 / 256 /
+ * 512 on the batch and keeps the fastest. */
 int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps, const int32_t sets[2],
                     const lb_kn *kn, const lb_wall *walls, const lb_opts *opts, lb_batch **out);
 /* Every lattice nsteps steps: one persistent launch. Asynchronous. */

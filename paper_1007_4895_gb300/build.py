@@ -20,6 +20,8 @@ SOURCES = ["lb_api.cu", "lb_step.cu", "lb_step_st_f64.cu", "lb_step_st_f32.cu", 
            "lb_step_st_f16.cu", "lb_step_st_bf16.cu", "lb_pair_f32.cu", "lb_pair_f32dev.cu", "lb_pair_f16.cu",
            "lb_pair_bf16.cu", "lb_ring_f32.cu", "lb_ring_f32dev.cu", "lb_ring_f16.cu", "lb_ring_bf16.cu",
            "lb_ring2_f32_q16.cu", "lb_ring2_f32_q36.cu", "lb_ring2_f32dev_q16.cu", "lb_ring2_f32dev_q36.cu", "lb_ring2_f16_q16.cu", "lb_ring2_f16_q36.cu", "lb_ring2_bf16_q16.cu", "lb_ring2_bf16_q36.cu",
+           "lb_tile_f32_q16.cu", "lb_tile_f32_q36.cu", "lb_tile_f32dev_q16.cu", "lb_tile_f32dev_q36.cu",
+           "lb_tile_f16_q16.cu", "lb_tile_f16_q36.cu", "lb_tile_bf16_q16.cu", "lb_tile_bf16_q36.cu",
            "lb_resident.cu", "lb_resident_f64.cu", "lb_resident_f32.cu", "lb_resident_f32dev.cu",
            "lb_resident_f16_pair.cu", "lb_resident_bf16_pair.cu", "lb_resident_f16_node.cu", "lb_resident_bf16_node.cu",
            "lb_step3.cu", "lb_stream.cu", "lb_aux.cu", "lb_mlp.cu", "lb_noalloc.cu",
@@ -29,7 +31,7 @@ SOURCES = ["lb_api.cu", "lb_step.cu", "lb_step_st_f64.cu", "lb_step_st_f32.cu", 
 CONTRACT = {"lb_pair_f32.cu", "lb_pair_f32dev.cu", "lb_pair_f16.cu", "lb_pair_bf16.cu", "lb_ring_f32.cu",
             "lb_ring_f32dev.cu", "lb_ring_f16.cu", "lb_ring_bf16.cu", "lb_resident_f32.cu", "lb_resident_f32dev.cu",
             "lb_resident_f16_pair.cu", "lb_resident_bf16_pair.cu"} | {
-                f"lb_ring2_{f}_q{q}.cu" for f in ("f32", "f32dev", "f16", "bf16") for q in (16, 36)}
+                f"lb_{k}_{f}_q{q}.cu" for k in ("ring2", "tile") for f in ("f32", "f32dev", "f16", "bf16") for q in (16, 36)}
 
 
 def nvcc() -> str:

@@ -129,6 +129,13 @@ struct lb_ctx {
     int2 *d_rdesc = nullptr;
     uint32_t *d_rctr = nullptr;
     std::unique_ptr<lbk::RingTab> rtab;
+    /* layout 10 on tiles: units, those of set 1 first, and the tensor maps per level */
+    std::vector<int4> tunits_h;
+    int tunits_n1 = 0;
+    int4 *d_tunits = nullptr;
+    size_t tunits_cap = 0;
+    TileMaps tmaps[2];
+    bool tiles_ok = false;
     /* resident steps (lb_resident.cuh): several steps per launch, the state in shared memory */
     bool res_on = false, res_pair = false;
     lbk::ResPlan rplan;
@@ -577,6 +584,48 @@ int build_edge_lists(lb_ctx *c)
                                                   cudaMemcpyHostToDevice, c->stream), "row queue upload"))
             return e;
     }
+    /* units of layout 10 on tiles: runs of one set in a tile column without mode-A interface
+     * rows, cut into equal parts of at most TILE_ROWS rows; a bit for the node-by-node body (a
+     * tile that ends inside, periodic ghost columns of a width of no whole quads) */
+    {
+        std::vector<int4> part[2];
+        for (int tx = 0; tx < c->ntx; ++tx) {
+            const bool ragged = (tx + 1) * LB_TILE_X > c->nx;
+            const bool gcols = px && (tx == 0 || (tx + 1) * LB_TILE_X > c->nx - LB_GHOST);
+            auto flag = [&](int j) { return c->tmap[(size_t)j * c->ntx + tx]; };
+            for (int j = 0; j < c->ny;) {
+                if (flag(j) & LB_TILE_IFACE) {
+                    ++j;
+                    continue;
+                }
+                const int s = flag(j) & LB_TILE_HIGH;
+                int k = j;
+                while (k < c->ny && !(flag(k) & LB_TILE_IFACE) && (flag(k) & LB_TILE_HIGH) == s) ++k;
+                const int n = k - j, parts = (n + TILE_ROWS - 1) / TILE_ROWS;
+                for (int u = 0; u < parts; ++u) {
+                    const int a = j + (int)((long long)n * u / parts), b = j + (int)((long long)n * (u + 1) / parts);
+                    const int gen = ragged || (gcols && c->nx % 4 != 0);
+                    part[s].push_back(make_int4(tx, a, (b - a) | (gen << 8), s));
+                }
+                j = k;
+            }
+        }
+        c->tunits_n1 = (int)part[1].size();
+        c->tunits_h = part[1];
+        c->tunits_h.insert(c->tunits_h.end(), part[0].begin(), part[0].end());
+        if (!c->tunits_h.empty()) {
+            if (c->tunits_h.size() > c->tunits_cap) {
+                const size_t cap = std::max(c->tunits_h.size(), 2 * c->tunits_cap);
+                int4 *d = static_cast<int4 *>(own(c, cap * sizeof(int4)));
+                if (!d) return fail(LB_ERR_NOMEM, "device allocation failed");
+                c->d_tunits = d;
+                c->tunits_cap = cap;
+            }
+            if (int e = cuda_check(c, cudaMemcpyAsync(c->d_tunits, c->tunits_h.data(), c->tunits_h.size() * sizeof(int4),
+                                                      cudaMemcpyHostToDevice, c->stream), "tile unit upload"))
+                return e;
+        }
+    }
     /* compact-state segments */
     compact_segments(c, c->tmap, c->seg_h, c->nseg);
     if (!c->seg_h.empty()) {
@@ -673,6 +722,19 @@ int upload_tiles(lb_ctx *c)
  * that hold high-order rows; 7: layout 0's threads with paired FP32 arithmetic on the
  * rows without boundary work (lb_pair.cuh); 8: 7 with the block order of 5; 9: 7's
  * arithmetic fed by a per-thread ring of asynchronous copies (lb_ring.cuh). */
+/* Layout 10 has two forms with the same bits: rows through a per-thread ring (lb_ring2.cuh)
+ * and tiles streamed by the tensor memory accelerator (lb_tile.cuh). The tiles run ahead of
+ * the copies' latency, which is what a lattice in L2 is bound by; the rows need no warp to
+ * keep step with others, which wins once DRAM is. Us a step, rows / tiles: 1200 x 90 pressure
+ * channel 82 / 41 (16-bit 91 / 41), 1024 x 512 Poiseuille 46.8 / 41.9 (57.7 / 45.4), 16384 x
+ * 128 channel, whose two levels are larger than L2, 97 / 120 (92 / 134). */
+bool tiles_pay(const lb_ctx *c)
+{
+    size_t pops = 0;
+    for (size_t k = 0; k < c->tmap.size(); ++k) pops += (size_t)c->q[c->tmap[k] & LB_TILE_HIGH] * LB_TILE_X;
+    return 2 * pops * c->esize <= (size_t)100 << 20;
+}
+
 template <typename R>
 void launch_variant(lb_ctx *c, int variant, const StepParams<R> &p)
 {
@@ -712,6 +774,10 @@ void launch_variant(lb_ctx *c, int variant, const StepParams<R> &p)
             lbk::launch_ring(c->store, p, c->stream);
             return;
         }
+        if (variant == 10 && c->tiles_ok && tiles_pay(c) && !p.sr && !c->tunits_h.empty() &&
+            lbk::launch_tiles(c->store, p, *c->rtab, c->tmaps[c->cur], c->d_tunits, (int)c->tunits_h.size(), c->tunits_n1,
+                              c->d_rctr, c->d_err, c->stream) == 0)
+            return;
         if (variant == 10) {
             const lbk::RowQueues rq{c->d_rrows, c->d_rdesc, c->d_rctr, c->nsm};
             lbk::launch_ring_units(c->store, p, *c->rtab, rq, (int)((c->rrows_h.size() + 7) / 8), c->stream);
@@ -992,6 +1058,12 @@ int autotune_t(lb_ctx *c, float *step_ms)
                     (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV);
     for (int v = 0; v < LB_NUM_VARIANTS; ++v) {
         if (!variant_available(c, v) || (v == 10 && sr)) continue;
+        /* 16-bit storage and per-column references: layout 10 rounds unlike layouts 0 to 8, and
+         * on smaller lattices the runs so far have those layouts' values; it is offered from
+         * the size on where it has always been the fastest */
+        if (v == 10 && (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV || c->d_dcol) &&
+            (long long)c->nx * c->ny < 1250000LL)
+            continue;
         /* with the pressure pass, which layout 10 does inside its kernel when the lattice
          * has no body force */
         auto one = [&] {
@@ -1284,6 +1356,39 @@ bool make_maps(lb_ctx *c)
     return true;
 }
 
+/* Tensor maps of layout 10 on tiles: boxes of 136 columns of every set's planes
+ * and the carried moments of every level. */
+bool make_tile_maps(lb_ctx *c)
+{
+    if (c->store == LB_STORE_F64) return false;
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return false;
+    const CUtensorMapDataType dt = c->store == LB_STORE_F16_DEV    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                   : c->store == LB_STORE_BF16_DEV ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                                   : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const cuuint64_t rows = (cuuint64_t)c->ny + 2 * LB_GHOST_ROWS;
+    const cuuint32_t estr[3] = {1, 1, 1};
+    for (int lv = 0; lv < 2; ++lv) {
+        for (int s = 0; s < 2; ++s) {
+            const cuuint64_t dims[3] = {(cuuint64_t)c->pitch, rows, (cuuint64_t)c->q[s]};
+            const cuuint64_t strides[2] = {(cuuint64_t)c->pitch * c->esize, (cuuint64_t)c->pitch * rows * c->esize};
+            const cuuint32_t box[3] = {LB_TILE_X + 2 * LB_GHOST, (cuuint32_t)tile_box_rows((int)c->esize), 1};
+            if (enc(&c->tmaps[lv].box[s], dt, 3, c->planes[lv][s], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                return false;
+        }
+        const cuuint64_t dims[3] = {(cuuint64_t)c->pitch, (cuuint64_t)c->ny, 3};
+        const cuuint64_t strides[2] = {(cuuint64_t)c->pitch * 4, (cuuint64_t)c->pitch * c->ny * 4};
+        const cuuint32_t box[3] = {LB_TILE_X, TILE_ROWS, 3};
+        if (enc(&c->tmaps[lv].aux, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, c->aux[lv], dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
 /* A bounded wait inside a kernel ran out: the context is left in LB_ERR_TIMEOUT. */
 int check_device_error(lb_ctx *c)
 {
@@ -1503,6 +1608,7 @@ int lb_create(const lb_grid *grid, const uint8_t *region_map, const int32_t sets
         return fail(LB_ERR_CUDA, std::string("initial fill failed: ") + cudaGetErrorString(ce));
     }
     c->tma_ok = make_maps(c);
+    c->tiles_ok = make_tile_maps(c);
     if (!use_f64(c)) {
         /* constant tables of layouts 7 / 8 (without them those layouts are not offered) */
         c->d_ctab = own(c, lbk::pair_table_bytes());

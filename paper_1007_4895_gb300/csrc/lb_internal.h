@@ -140,7 +140,9 @@ void launch_aux(int store, const StepParams<R> &p, const int2 *list, int n, void
  * with its blocks launched in block_order, 9 layout 7's arithmetic fed by a per-thread
  * ring of asynchronous copies, boundary work in the same kernel (lb_ring.cuh), 10 layout
  * 9's arithmetic in a persistent kernel over row units, most expensive first, with the
- * rows without boundary work specialised on the velocity set (lb_ring2.cuh) */
+ * rows without boundary work specialised on the velocity set (lb_ring2.cuh), or over tiles
+ * fed by the tensor memory accelerator (lb_tile.cuh). Small lattices take several steps per
+ * launch instead (lb_resident.cuh). */
 #define LB_NUM_VARIANTS 11
 /* layout 7 / 8: p.block_order selects between them (FP32 and 16-bit storage); p.ctab
  * must hold the tables that launch_pair_table wrote for this lattice */

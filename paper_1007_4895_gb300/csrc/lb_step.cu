@@ -9,6 +9,7 @@
 
 #include "lb_common.cuh"
 #include "lb_pressure.cuh"
+#include "lb_tma.h"
 
 namespace lbk {
 
@@ -26,6 +27,9 @@ void launch_ring_store(const StepParams<float> &p, void *stream);
 template <int ST, int Q1>
 void launch_ring_units_store(const StepParams<float> &p, const RingTab &tab, const RowQueues &rq, int nblocks,
                              void *stream);
+template <int ST, int Q1>
+int launch_tiles_store(const StepParams<float> &p, const RingTab &tab, const TileMaps &maps, const int4 *units, int nunits,
+                       int n1, uint32_t *ctr, int *err, void *stream);
 template <int ST, int Q1>
 int launch_ring_batch_store(const StepParams<float> *params, const RingTab *tabs, const uint32_t *items,
                             const int2 *ranges, const int *order, int n, int nsteps, int base, int advance,
@@ -370,6 +374,21 @@ void launch_ring_units(int store, const StepParams<float> &p, const RingTab &tab
         case 4: (q36 ? launch_ring_units_store<4, 36> : launch_ring_units_store<4, 16>)(p, tab, rq, nblocks, stream); break;
         default: break;
     }
+}
+
+int launch_tiles(int store, const StepParams<float> &p, const RingTab &tab, const TileMaps &maps, const int4 *units,
+                 int nunits, int n1, uint32_t *ctr, int *err, void *stream)
+{
+    const bool q36 = p.set[1].q == 36;
+#define LB_TL(ST) (q36 ? launch_tiles_store<ST, 36> : launch_tiles_store<ST, 16>)(p, tab, maps, units, nunits, n1, ctr, err, stream)
+    switch (store) {
+        case 1: return LB_TL(1);
+        case 2: return LB_TL(2);
+        case 3: return LB_TL(3);
+        case 4: return LB_TL(4);
+        default: return -1;
+    }
+#undef LB_TL
 }
 
 int launch_ring_batch(int store, int q1, const StepParams<float> *params, const RingTab *tabs, const uint32_t *items,

@@ -16,7 +16,23 @@ struct TmaMaps {
     CUtensorMap box5[2];   /* per set: 136 columns x (stream rows + 4) rows x 1 plane (streamed layout) */
 };
 
+/* layout 10 on tiles: per set 136 columns x tile_box_rows(element size) rows x 1 plane of a
+ * level, and the level's carried moments, 128 columns x TILE_ROWS rows x 3 sums */
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int tile_box_rows(int esize) { return esize == 4 ? 4 : 8; }
+constexpr int TILE_ROWS = 7;   /* rows of a unit: one per consumer warp */
+struct TileMaps {
+    CUtensorMap box[2];
+    CUtensorMap aux;
+};
+
 namespace lbk {
+/* units [nunits] (tile, first row, rows | general << 8, set), the n1 of set 1 first; 0
+ * on launch, -1 if unavailable */
+int launch_tiles(int store, const StepParams<float> &p, const RingTab &tab, const TileMaps &maps, const int4 *units,
+                 int nunits, int n1, uint32_t *ctr, int *err, void *stream);
 int launch_step3(int store, const StepParams<float> &p, const TmaMaps &maps, int *err, void *stream);
 int step3_rows();
 int step3_cols();
