@@ -377,7 +377,7 @@ int finalize_level_t(lb_ctx *c, int level)
     /* carried moments of this level: read only by layouts 4 and 10 (and by the
      * autotuner, which runs while no layout is chosen yet) */
     if (c->variant < 0 || c->variant == 4 || c->variant == 10 || c->ring_batch)
-        lbk::launch_aux<R>(c->store, p, nullptr, 0, st);
+        lbk::launch_aux<R>(c->store, p, st);
     return launch_check(c, "finalize");
 }
 
@@ -2469,7 +2469,7 @@ int lb_batch_step_each(lb_batch *b, int64_t nsteps)
     /* layout 9 carries no moments: the ring batch's are summed again */
     if (b->ring && !b->resident && nsteps > 0)
         for (lb_ctx *c : b->inst) {
-            lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), nullptr, 0, c->stream);
+            lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), c->stream);
             if (int e = launch_check(c, "carried moments")) return e;
         }
     return LB_OK;

@@ -127,10 +127,10 @@ int launch_batch(int store, const void *params, const int *order, int n, int nst
                  unsigned int *queue, int threads, int grid, void *stream);
 /* resident blocks per SM of the batch kernel for a block size (0 on error) */
 int batch_blocks(int store, int threads);
-/* carried moments (streamed layout) of every node of the written level (list == NULL)
- * or of the listed quads (x0, j), from their stored populations */
+/* carried moments (layouts 4 and 10) of every node of the written level, from their
+ * stored populations */
 template <typename R>
-void launch_aux(int store, const StepParams<R> &p, const int2 *list, int n, void *stream);
+void launch_aux(int store, const StepParams<R> &p, void *stream);
 /* step-kernel layouts: 0 one node quad per thread, 1 TMA-fed producer / consumer,
  * 2 and 3 split plain / edge kernels with register blocks of 4 x 1 and 4 x 2 nodes,
  * 4 streamed (TMA, carried moments, boundary work at the end of each unit), 5 layout 0
