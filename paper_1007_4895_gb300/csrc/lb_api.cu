@@ -427,6 +427,19 @@ void launch_pack_t(lb_ctx *c, int unpack)
                         std::max(c->q[0], c->q[1]), c->d_stage, unpack, c->stream);
 }
 
+/* Layout 10 has two forms with the same bits: rows through a per-thread ring (lb_ring2.cuh)
+ * and tiles streamed by the tensor memory accelerator (lb_tile.cuh). The tiles run ahead of
+ * the copies' latency, which is what a lattice in L2 is bound by; the rows need no warp to
+ * keep step with others, which wins once DRAM is. Us a step, rows / tiles: 1200 x 90 pressure
+ * channel 82 / 41 (16-bit 91 / 41), 1024 x 512 Poiseuille 46.8 / 41.9 (57.7 / 45.4), 16384 x
+ * 128 channel, whose two levels are larger than L2, 97 / 120 (92 / 134). */
+bool tiles_pay(const lb_ctx *c)
+{
+    size_t pops = 0;
+    for (size_t k = 0; k < c->tmap.size(); ++k) pops += (size_t)c->q[c->tmap[k] & LB_TILE_HIGH] * LB_TILE_X;
+    return 2 * pops * c->esize <= (size_t)100 << 20;
+}
+
 /* Lists of the quads the plain kernels of the split step leave to the one-quad kernel:
  * every quad of a 4 x rb block that is not plain as a whole (plain_quad(), shared with
  * the device), except mode-A interface rows, which no step kernel updates. */
@@ -586,8 +599,10 @@ int build_edge_lists(lb_ctx *c)
     }
     /* units of layout 10 on tiles: runs of one set in a tile column without mode-A interface
      * rows, cut into equal parts of at most TILE_ROWS rows; a bit for the node-by-node body (a
-     * tile that ends inside, periodic ghost columns of a width of no whole quads) */
-    {
+     * tile that ends inside, periodic ghost columns of a width of no whole quads); none for
+     * lattices that take another layout, or whose levels call for the rows */
+    c->tunits_h.clear();
+    if (c->store != LB_STORE_F64 && (c->opts.variant < 0 || c->opts.variant == 10) && tiles_pay(c)) {
         std::vector<int4> part[2];
         for (int tx = 0; tx < c->ntx; ++tx) {
             const bool ragged = (tx + 1) * LB_TILE_X > c->nx;
@@ -722,18 +737,6 @@ int upload_tiles(lb_ctx *c)
  * that hold high-order rows; 7: layout 0's threads with paired FP32 arithmetic on the
  * rows without boundary work (lb_pair.cuh); 8: 7 with the block order of 5; 9: 7's
  * arithmetic fed by a per-thread ring of asynchronous copies (lb_ring.cuh). */
-/* Layout 10 has two forms with the same bits: rows through a per-thread ring (lb_ring2.cuh)
- * and tiles streamed by the tensor memory accelerator (lb_tile.cuh). The tiles run ahead of
- * the copies' latency, which is what a lattice in L2 is bound by; the rows need no warp to
- * keep step with others, which wins once DRAM is. Us a step, rows / tiles: 1200 x 90 pressure
- * channel 82 / 41 (16-bit 91 / 41), 1024 x 512 Poiseuille 46.8 / 41.9 (57.7 / 45.4), 16384 x
- * 128 channel, whose two levels are larger than L2, 97 / 120 (92 / 134). */
-bool tiles_pay(const lb_ctx *c)
-{
-    size_t pops = 0;
-    for (size_t k = 0; k < c->tmap.size(); ++k) pops += (size_t)c->q[c->tmap[k] & LB_TILE_HIGH] * LB_TILE_X;
-    return 2 * pops * c->esize <= (size_t)100 << 20;
-}
 
 template <typename R>
 void launch_variant(lb_ctx *c, int variant, const StepParams<R> &p)
@@ -774,7 +777,7 @@ void launch_variant(lb_ctx *c, int variant, const StepParams<R> &p)
             lbk::launch_ring(c->store, p, c->stream);
             return;
         }
-        if (variant == 10 && c->tiles_ok && tiles_pay(c) && !p.sr && !c->tunits_h.empty() &&
+        if (variant == 10 && c->tiles_ok && !p.sr && !c->tunits_h.empty() &&
             lbk::launch_tiles(c->store, p, *c->rtab, c->tmaps[c->cur], c->d_tunits, (int)c->tunits_h.size(), c->tunits_n1,
                               c->d_rctr, c->d_err, c->stream) == 0)
             return;
@@ -1360,7 +1363,7 @@ bool make_maps(lb_ctx *c)
  * and the carried moments of every level. */
 bool make_tile_maps(lb_ctx *c)
 {
-    if (c->store == LB_STORE_F64) return false;
+    if (c->store == LB_STORE_F64 || (c->opts.variant >= 0 && c->opts.variant != 10)) return false;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
     const CUtensorMapDataType dt = c->store == LB_STORE_F16_DEV    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16

@@ -5,7 +5,8 @@
  */
 #include <algorithm>
 #include <cstring>
-#include <map>
+#include <utility>
+#include <vector>
 
 #include "lb_internal.h"
 #include "lb_resident_host.h"
@@ -28,8 +29,8 @@ struct Part {
     std::vector<ResGRow> grow;
     std::vector<uint16_t> push, shlist;
     std::vector<int> ids;
-    /* per set: slot of row (lattice, j), and the halo rows among them */
-    std::map<std::pair<int, int>, int> slot[2], halo[2];
+    /* per set: the halo rows (j, slot) of a cluster's band */
+    std::vector<std::pair<int, int>> halo[2];
     int nwall = 0;
     size_t smem = 0;
     double cost = 0.0;
@@ -54,14 +55,19 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
     h.upr_magic = magic(upr);
     auto flag = [&](int lat, int j) { return L[lat].flags[(size_t)j * L[lat].ntx]; };
     auto set_of = [&](int lat, int j) { return (int)(flag(lat, j) & LB_TILE_HIGH); };
-    auto owned = [&](int lat, int j) {
-        for (const Piece &o : p.own)
-            if (o.lat == lat && j >= o.j0 && j < o.j1) return true;
-        return false;
-    };
     struct Own {
-        int lat, j, key;
+        int k, j, key;   /* piece, row */
     };
+    /* slot of row j of piece k in each set: flat tables (a bundle sweep looks up several
+     * hundred thousand rows; ordered maps made the plan of 512 channels 40 ms, these 9 ms) */
+    std::vector<size_t> base;
+    size_t nall = 0;
+    for (const Piece &o : p.own) {
+        base.push_back(nall);
+        nall += (size_t)L[o.lat].ny;
+    }
+    std::vector<int> slot[2] = {std::vector<int>(nall, -1), std::vector<int>(nall, -1)};
+    int nslot[2] = {0, 0};
     std::vector<Own> own[2];
     h.nwall[0] = h.nwall[1] = 0;
     for (size_t k = 0; k < p.own.size(); ++k) {
@@ -71,73 +77,66 @@ bool layout_part(const std::vector<ResLattice> &L, Part &p, const Sizes &z, bool
             const bool wall = (j == 0 && L[o.lat].wall[0]) || (j == L[o.lat].ny - 1 && L[o.lat].wall[1]);
             /* the rows with the longest chains first: walls, then shadow rows */
             h.nwall[set_of(o.lat, j)] += wall;
-            own[set_of(o.lat, j)].push_back({o.lat, j, wall ? 0 : ((flag(o.lat, j) & LB_TILE_SHADOW) ? 1 : 2)});
+            own[set_of(o.lat, j)].push_back({(int)k, j, wall ? 0 : ((flag(o.lat, j) & LB_TILE_SHADOW) ? 1 : 2)});
         }
     }
     for (int s = 0; s < 2; ++s) {
         std::stable_sort(own[s].begin(), own[s].end(), [](const Own &a, const Own &b) { return a.key < b.key; });
-        for (const Own &o : own[s]) {
-            const int n = (int)p.slot[s].size();
-            p.slot[s][{o.lat, o.j}] = n;
-        }
+        for (const Own &o : own[s]) slot[s][base[o.k] + o.j] = nslot[s]++;
         h.nrow[s] = (int)own[s].size();
         h.nunit[s] = h.nrow[s] * upr;
         h.unit_magic[s] = magic(h.nunit[s]);
         if (h.nunit[s] * 6 > 0xffff) return false;   /* items of a round */
     }
-    auto lat_index = [&](int lat) {
-        for (size_t k = 0; k < p.ids.size(); ++k)
-            if (p.ids[k] == lat) return (int)k;
-        return 0;
-    };
     int nshadow = 0;
     for (int s = 0; s < 2; ++s)
         for (const Own &o : own[s]) {
-            const ResLattice &l = L[o.lat];
+            const Piece &pc = p.own[o.k];
+            const ResLattice &l = L[pc.lat];
             ResRow r{};
             auto at = [&](int d) -> uint16_t {
                 int j = o.j + d;
                 if (l.periodic_y) j = (j + l.ny) % l.ny;
                 else j = std::max(0, std::min(l.ny - 1, j));
-                auto it = p.slot[s].find({o.lat, j});
-                if (it != p.slot[s].end()) return (uint16_t)it->second;
-                const int n = (int)p.slot[s].size();
-                p.slot[s][{o.lat, j}] = n;
-                if (!owned(o.lat, j)) p.halo[s][{o.lat, j}] = n;
+                int &n = slot[s][base[o.k] + j];
+                if (n < 0) {
+                    n = nslot[s]++;
+                    if (j < pc.j0 || j >= pc.j1) p.halo[s].push_back({j, n});
+                }
                 return (uint16_t)n;
             };
-            r.own = (uint16_t)p.slot[s][{o.lat, o.j}];
+            r.own = (uint16_t)slot[s][base[o.k] + o.j];
             r.m2 = at(-2);
             r.m1 = at(-1);
             r.p1 = at(1);
             r.p2 = at(2);
-            r.lat = (uint16_t)lat_index(o.lat);
+            r.lat = (uint16_t)o.k;
             r.view = RES_NONE;
             r.wallord = r.shord = RES_NONE;
             r.j = (uint16_t)o.j;
             if (o.j == 0 && l.wall[0]) r.flags |= 1;
             else if (o.j == l.ny - 1 && l.wall[1]) r.flags |= 2;
             if (r.flags & 3) r.wallord = (uint16_t)p.nwall++;
-            if (flag(o.lat, o.j) & LB_TILE_SHADOW) {
+            if (flag(pc.lat, o.j) & LB_TILE_SHADOW) {
                 r.flags |= RES_SHADOW;
                 r.shord = (uint16_t)nshadow++;
                 h.nsh[s] += 1;
                 p.shlist.push_back((uint16_t)p.rows.size());
             }
             p.rows.push_back(r);
-            p.grow.push_back({o.lat, o.j});
+            p.grow.push_back({pc.lat, o.j});
         }
     /* views live where this part's rows of the other set asked for a slot */
     for (int s = 0; s < 2; ++s)
         for (int k = 0; k < h.nrow[s]; ++k) {
             const int i = (s ? h.nrow[0] : 0) + k;
-            auto it = p.slot[1 - s].find({p.grow[i].lat, p.grow[i].j});
-            if (it == p.slot[1 - s].end()) continue;
+            const int v = slot[1 - s][base[own[s][k].k] + own[s][k].j];
+            if (v < 0) continue;
             if (!(p.rows[i].flags & RES_SHADOW)) return false;   /* a reader without a view */
-            p.rows[i].view = (uint16_t)it->second;
+            p.rows[i].view = (uint16_t)v;
         }
     for (int s = 0; s < 2; ++s) {
-        h.nslot[s] = (int)p.slot[s].size();
+        h.nslot[s] = nslot[s];
         if (h.nslot[s] > 60000) return false;
         h.q[s] = f.q[s];
         const int n1 = f.q[s] == 9 ? 3 : (f.q[s] == 16 ? 4 : 6);
@@ -316,7 +315,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
         for (size_t r = 0; r < parts.size(); ++r)
             for (int s = 0; s < 2; ++s)
                 for (const auto &hl : parts[r].halo[s]) {
-                    const int j = hl.first.second;
+                    const int j = hl.first;
                     for (size_t o = 0; o < parts.size(); ++o) {
                         Part &p = parts[o];
                         if (o == r || j < p.own[0].j0 || j >= p.own[0].j1) continue;
