@@ -441,13 +441,16 @@ __device__ __forceinline__ bool tile_row(const StepParams<float> &p, const RingT
     return alive;
 }
 
-/* a unit's stages passed over by a warp without a row in it */
+/* A unit's stages passed over by a warp without a row in it. Every lane has seen a stage full
+ * before lane 0 releases it: once all warps have, the producer refills the stage and its
+ * barrier moves on, and a lane still polling would wait on a parity that has gone by. */
 template <int ST>
 __device__ __forceinline__ bool tile_skip(TileRing &rg, int q)
 {
     bool alive = true;
     for (int a = 0; a < q && alive; ++a) {
         alive = tile_wait(&rg.full[rg.st], rg.parity);
+        __syncwarp();
         if ((threadIdx.x & 31) == 0) mbar_arrive(&rg.empty[rg.st]);
         if (++rg.st == (uint32_t)tile_stages<ST>()) {
             rg.st = 0;
@@ -582,6 +585,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
                 if (alive && u.x == p.ntx - 1 && p.pressure[1]) pressure_row<ST>(p, j, 1);
             }
         } else {
+            __syncwarp();   /* every lane has its copy of the unit: the slot may be refilled */
             if (lane == 0) mbar_arrive(&aempty[slot]);
             alive = tile_skip<ST>(rg, s ? Q1 : 9);
         }
