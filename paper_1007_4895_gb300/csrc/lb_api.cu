@@ -1067,11 +1067,10 @@ int autotune_t(lb_ctx *c, float *step_ms)
         if (v == 10 && (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV || c->d_dcol) &&
             (long long)c->nx * c->ny < 1250000LL)
             continue;
-        /* with the pressure pass, which layout 10 does inside its kernel when the lattice
-         * has no body force */
+        /* with the pressure pass, which layout 10 does inside its kernel where it can */
         auto one = [&] {
             launch_variant<R>(c, v, p);
-            if (v != 10 || p.has_force) lbk::launch_pressure<R>(c->store, p, c->stream);
+            if (v != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
         };
         for (int k = 0; k < 2; ++k) one();
         cudaEventRecord(e0, c->stream);
@@ -1248,7 +1247,7 @@ int step_t(lb_ctx *c, int64_t n)
         } else {
             launch_variant<R>(c, c->variant, p);
             lbk::launch_iface<R>(c->store, p, c->stream);
-            if (c->variant != 10 || p.has_force) lbk::launch_pressure<R>(c->store, p, c->stream);   /* else 10 does it */
+            if (c->variant != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
         }
         if (int e = launch_check(c, "step")) return e;
         c->cur ^= 1;

@@ -101,6 +101,20 @@ struct StepParams {
     SetConst<R> set[2];
 };
 
+/* Layout 10 sets the pressure columns inside its step kernel, at the end of the rows of the
+ * first and last tiles, from the node one step inwards. False where that is left to the
+ * pressure pass: with a body force (its registers would weigh on the force kernels), and
+ * where the last tile holds the boundary column alone (nx = 1 mod 128): the node inwards is
+ * then another warp's or block's, whose store this launch does not order before the read. */
+template <typename R>
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline bool pressure_in_step(const StepParams<R> &p)
+{
+    return !p.has_force && !(p.pressure[1] && p.nx % LB_TILE_X == 1);
+}
+
 /* storage codes match LB_STORE_* */
 namespace lbk {
 
