@@ -2232,7 +2232,7 @@ int batch_ring_setup(lb_batch *b)
     return LB_OK;
 }
 
-/* The resident steps for the whole batch: true when every lattice fits a block. */
+/* The resident steps for the whole batch, where every lattice fits a block. */
 int batch_resident_setup(lb_batch *b, int nsm)
 {
     std::vector<lbk::ResLattice> L;
@@ -2243,7 +2243,9 @@ int batch_resident_setup(lb_batch *b, int nsm)
         if (c->ny > 0xfff0 || c->nx > 0x7fff || (b->res_pair && !c->rtab)) return LB_OK;
         L.push_back(resident_lattice(c, resident_group(c, b->res_pair)));
     }
-    if (!lbk::res_plan_build(L, b->store, b->res_pair, 1, nsm, 0, b->plan)) return LB_OK;
+    if (!lbk::res_plan_build(L, b->store, b->res_pair, 1, nsm, 0, b->plan) ||
+        !lbk::resident_fits(b->store, b->res_pair, b->force, b->plan))
+        return LB_OK;
     b->d_plan = static_cast<unsigned char *>(batch_alloc(b, b->plan.blob.size()));
     b->d_off = static_cast<uint32_t *>(batch_alloc(b, b->plan.off.size() * sizeof(uint32_t)));
     if (!b->d_plan || !b->d_off) return fail(LB_ERR_NOMEM, "device allocation failed");

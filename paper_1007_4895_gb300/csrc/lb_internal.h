@@ -233,6 +233,10 @@ struct ResRank {
     int nslot[2];
 };
 constexpr int RES_MAX_CLUSTER = 16;
+/* What a plan may take of a block's 227 KB: the kernels of one-block parts hold one word of
+ * static shared memory (16 bytes with its alignment), and a launch whose static and dynamic
+ * parts together pass 227 KB is refused; those on a cluster hold none. */
+constexpr size_t res_smem_limit(bool cluster) { return 227 * 1024 - (cluster ? 0 : 16); }
 struct alignas(16) ResHead {
     int q[2], K[2], nh[2];          /* populations, spare planes, wall-bound populations per set */
     int nrow[2], nslot[2], nunit[2], nsh[2], nwall[2];   /* own rows, slots, units, shadow and wall rows */
@@ -272,6 +276,8 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
 int launch_resident(int store, bool pair, bool force, const ResPlan &plan, const void *d_plan, const uint32_t *d_off,
                     const void *params, const RingTab *tabs, int nsteps, int base, uint32_t step0, int advance,
                     unsigned int *queue, const void *osc, int blocks, void *stream);
+/* whether the device can hold a block (or a whole cluster) of the plan's kernel */
+bool resident_fits(int store, bool pair, bool force, const ResPlan &plan);
 
 /* The quad of nodes x0 .. x0+3 of row j needs none of the boundary work of the step
  * (wall overwrite, ghost-row or ghost-column copies, pressure column, mode-B shadow or

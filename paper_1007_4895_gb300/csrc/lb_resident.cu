@@ -15,8 +15,6 @@ namespace lbk {
 
 namespace {
 
-constexpr size_t RES_SMEM = 227 * 1024;   /* dynamic shared memory of one block */
-
 size_t up16(size_t v) { return (v + 15) / 16 * 16; }
 
 struct Piece {
@@ -219,7 +217,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
 {
     const Sizes z{pair ? 4 : 1, store == 0 ? 8 : (store <= 2 ? 4 : 2), store == 0 ? 8 : 4, store == 2, pair};
     const size_t pop_bytes = (L[0].q[0] + L[0].q[1]) * (pair ? sizeof(RingPop) : 16 * (size_t)z.rsize);
-    const size_t lat_bytes = 24 * (size_t)z.rsize;
+    const size_t lat_bytes = 24 * (size_t)z.rsize, limit = res_smem_limit(cluster > 1);
     std::vector<Part> parts;
     if (cluster > 1) {
         if (L.size() != 1 || cluster > RES_MAX_CLUSTER) return false;
@@ -257,7 +255,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
             if (!layout_part(L, p, z, false)) return false;
             bool fits = false;
             for (int r : {1, 2, 3, 6}) {
-                if (place_part(p, z, r, pop_bytes, lat_bytes) <= RES_SMEM) {
+                if (place_part(p, z, r, pop_bytes, lat_bytes) <= limit) {
                     fits = true;
                     break;
                 }
@@ -269,7 +267,7 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
             total += b;
         }
         std::stable_sort(cs.begin(), cs.end(), [](const Cost &a, const Cost &b) { return a.c > b.c; });
-        const size_t cap = RES_SMEM - up16(sizeof(ResHead)) - up16(pop_bytes);
+        const size_t cap = limit - up16(sizeof(ResHead)) - up16(pop_bytes);
         blocks = std::max(1, blocks);
         for (size_t nb = std::min<size_t>(L.size(), blocks * ((total + blocks * cap - 1) / (blocks * cap)));;
              nb = std::min<size_t>(L.size(), nb + blocks)) {
@@ -338,15 +336,15 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
     for (int r : {1, 2, 3, 6}) {
         bool all = true;
         for (Part &p : parts) {
-            if (cluster == 1 && p.h.rounds > 0 && p.smem <= RES_SMEM) continue;
-            all = place_part(p, z, r, pop_bytes, lat_bytes) <= RES_SMEM && all;
+            if (cluster == 1 && p.h.rounds > 0 && p.smem <= limit) continue;
+            all = place_part(p, z, r, pop_bytes, lat_bytes) <= limit && all;
         }
         if (all) break;
     }
     out = ResPlan();
     out.cluster = cluster;
     for (Part &p : parts) {
-        if (p.smem > RES_SMEM) return false;
+        if (p.smem > limit) return false;
         split_part(p);
         p.h.sr = sr;
         if (cluster > 1)
@@ -373,11 +371,9 @@ bool res_plan_build(const std::vector<ResLattice> &L, int store, bool pair, int 
     return true;
 }
 
-int launch_resident(int store, bool pair, bool force, const ResPlan &plan, const void *d_plan, const uint32_t *d_off,
-                    const void *params, const RingTab *tabs, int nsteps, int base, uint32_t step0, int advance,
-                    unsigned int *queue, const void *osc, int blocks, void *stream)
+namespace {
+int resident_store(int store, bool pair, const ResLaunch &a)
 {
-    const ResLaunch a{&plan, d_plan, d_off, params, tabs, nsteps, base, step0, advance, queue, osc, blocks, force, stream};
     switch (store) {
         case 0: return pair ? -1 : launch_resident_store<0, false>(a);
         case 1: return pair ? launch_resident_store<1, true>(a) : -1;
@@ -386,6 +382,24 @@ int launch_resident(int store, bool pair, bool force, const ResPlan &plan, const
         case 4: return pair ? launch_resident_store<4, true>(a) : launch_resident_store<4, false>(a);
         default: return -1;
     }
+}
+}  // namespace
+
+int launch_resident(int store, bool pair, bool force, const ResPlan &plan, const void *d_plan, const uint32_t *d_off,
+                    const void *params, const RingTab *tabs, int nsteps, int base, uint32_t step0, int advance,
+                    unsigned int *queue, const void *osc, int blocks, void *stream)
+{
+    return resident_store(store, pair, {&plan, d_plan, d_off, params, tabs, nsteps, base, step0, advance, queue, osc, blocks,
+                                        force, stream, false});
+}
+
+bool resident_fits(int store, bool pair, bool force, const ResPlan &plan)
+{
+    ResLaunch a{};
+    a.plan = &plan;
+    a.force = force;
+    a.query = true;
+    return resident_store(store, pair, a) == 0;
 }
 
 }  // namespace lbk

@@ -913,7 +913,16 @@ int resident_launch(const ResLaunch &a)
             cudaGetLastError();
             return -1;
         }
-    } else {
+    }
+    if (a.query) {
+        int n = 0;
+        cudaError_t e;
+        if constexpr (CL) e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+        else e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, RES_THREADS, a.plan->smem);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && n > 0 ? 0 : -1;
+    }
+    if constexpr (!CL) {
         cfg.gridDim = dim3(a.plan->parts < a.blocks ? a.plan->parts : a.blocks);
         if (cudaMemsetAsync(a.queue, 0, sizeof(unsigned int), cfg.stream) != cudaSuccess) return -1;
     }

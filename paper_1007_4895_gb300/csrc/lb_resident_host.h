@@ -20,6 +20,7 @@ struct ResLaunch {
     int blocks;
     bool force;
     void *stream;
+    bool query;   /* nothing is launched: 0 if a block (a cluster) of it can be resident */
 };
 template <int ST, bool PAIR>
 int launch_resident_store(const ResLaunch &a);
