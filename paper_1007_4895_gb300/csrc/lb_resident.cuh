@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "lb_pair.cuh"
@@ -890,11 +891,21 @@ int resident_launch(const ResLaunch &a)
     using R = typename Store<ST>::R;
     static_assert(sizeof(ResLat<R>) <= 24 * sizeof(R), "room of a lattice in the plan");
     auto kern = resident_kernel<ST, PAIR, FORCE, CL>;
-    /* raised on every launch: the limit is per function and device, and the call is cheap
-     * next to a launch of many steps */
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.plan->smem) != cudaSuccess) {
-        cudaGetLastError();
-        return -1;
+    /* The shared-memory limit (and leave for clusters beyond the portable size) is the
+     * kernel's, on a device, for every context and host thread: set once, to the most any plan
+     * takes. (Set to the plan's own size on each launch, one thread lowered it between
+     * another's call and launch.) */
+    static std::atomic<bool> ready[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    dev &= 63;
+    if (!ready[dev].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem_limit(CL)) != cudaSuccess ||
+            (CL && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+            cudaGetLastError();
+            return -1;
+        }
+        ready[dev].store(true, std::memory_order_release);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(RES_THREADS);
@@ -908,11 +919,6 @@ int resident_launch(const ResLaunch &a)
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        if (a.plan->cluster > 8 &&
-            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-            cudaGetLastError();
-            return -1;
-        }
     }
     if (a.query) {
         int n = 0;
