@@ -351,8 +351,10 @@ int lb_map_stats(lb_ctx *ctx, int64_t *updates, int64_t *fallbacks, double *high
  * Knudsen numbers and wall speeds) advanced together by ONE persistent kernel launch
  * per call instead of one launch per lattice and step. Each lattice is an ordinary
  * context (lb_batch_instance gives it back for lb_moments, lb_get_populations, ...) and
- * takes exactly the steps of lb_step: the batched kernel does the one-quad layout's
- * arithmetic in the same order, so the results are the same bits.
+ * takes exactly the steps of lb_step with layout 9 (FP32 and 16-bit storage, D2Q9 with D2Q16
+ * or D2Q36, lattices at most one tile wide) or layout 0: the same arithmetic in the same
+ * order, so the results are the same bits. A lattice's region map may change between calls
+ * (lb_set_region_map, lb_load, lb_learned_map_now); the next call of the batch plans anew.
  * ------------------------------------------------------------------------------- */
 typedef struct lb_batch lb_batch;
 

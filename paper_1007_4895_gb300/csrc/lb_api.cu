@@ -73,6 +73,7 @@ struct lb_ctx {
     int cur = 0;
     uint8_t *d_tmap = nullptr;
     std::vector<uint8_t> tmap;
+    uint64_t map_count = 0;         /* maps installed so far (a batch plans by its members' maps) */
     std::vector<int> iface_rows;
     double *d_part = nullptr, *d_out = nullptr;
     unsigned int *d_counter = nullptr;
@@ -726,6 +727,7 @@ int upload_tiles(lb_ctx *c)
     if (int e = cuda_check(c, cudaMemcpyAsync(c->d_tmap, c->tmap.data(), c->tmap.size(), cudaMemcpyHostToDevice,
                                               c->stream), "tile map upload"))
         return e;
+    c->map_count += 1;
     return build_edge_lists(c);
 }
 
@@ -2080,6 +2082,10 @@ struct lb_batch {
     lbk::ResPlan plan;
     unsigned char *d_plan = nullptr;
     uint32_t *d_off = nullptr;
+    size_t plan_cap = 0, off_cap = 0, items_cap = 0;
+    int nsm = 0;
+    int quad_threads = 0, quad_grid = 0;   /* block shape of the one-quad kernel, once timed */
+    uint64_t maps_seen = 0;         /* the members' map_count that the plan or the items are of */
     int status = LB_OK;
     std::vector<void *> owned;
 };
@@ -2097,6 +2103,19 @@ void *batch_alloc(lb_batch *b, size_t bytes)
     }
     if (p) b->owned.push_back(p);
     return p;
+}
+
+/* *p with room for `bytes`, grown as needed (an outgrown one stays owned until destroy) */
+template <typename T>
+bool batch_room(lb_batch *b, T **p, size_t *cap, size_t bytes)
+{
+    if (*p && bytes <= *cap) return true;
+    const size_t want = std::max(bytes, 2 * *cap);
+    void *d = batch_alloc(b, want);
+    if (!d) return false;
+    *p = static_cast<T *>(d);
+    *cap = want;
+    return true;
 }
 
 void batch_release(lb_batch *b)
@@ -2133,9 +2152,23 @@ int batch_upload_params(lb_batch *b)
     return LB_OK;
 }
 
+/* Every lattice's constants table (paired arithmetic), once: they do not depend on the maps. */
+int batch_tabs(lb_batch *b)
+{
+    if (b->d_tabs) return LB_OK;
+    std::vector<lbk::RingTab> tabs(b->n);
+    for (int i = 0; i < b->n; ++i) tabs[i] = *b->inst[i]->rtab;
+    lbk::RingTab *d = static_cast<lbk::RingTab *>(batch_alloc(b, sizeof(lbk::RingTab) * b->n));
+    if (!d) return fail(LB_ERR_NOMEM, "device allocation failed");
+    if (cudaMemcpyAsync(d, tabs.data(), sizeof(lbk::RingTab) * b->n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+        cudaStreamSynchronize(b->stream) != cudaSuccess)
+        return fail(LB_ERR_CUDA, "batch constants upload failed");
+    b->d_tabs = d;
+    return LB_OK;
+}
+
 /* Work items of the ring batch (see launch_ring_batch): per lattice, runs of consecutive
- * rows of one set and kind, at most 32 quads each, most work first; and every lattice's
- * constants table. */
+ * rows of one set and kind, at most 32 quads each, most work first. */
 int batch_ring_setup(lb_batch *b)
 {
     /* items (two words each, longest first per lattice), then the row lists they index */
@@ -2146,12 +2179,10 @@ int batch_ring_setup(lb_batch *b)
     };
     std::vector<std::vector<Item>> all(b->n);
     std::vector<int2> ranges(b->n);
-    std::vector<lbk::RingTab> tabs(b->n);
     size_t nitems = 0, nrows = 0;
     for (int i = 0; i < b->n; ++i) {
         const lb_ctx *c = b->inst[i];
         if (!c->rtab) return fail(LB_ERR_INVALID, "a batched lattice has no layout-10 constants");
-        tabs[i] = *c->rtab;
         const bool py = c->walls[0].kind == LB_WALL_PERIODIC;
         const int qpr = (c->nx + 3) / 4, per = 32 / qpr;
         /* set | kind << 1: 0 edge (stores node by node where not plain), 1 row (ghost-row
@@ -2212,13 +2243,11 @@ int batch_ring_setup(lb_batch *b)
             items.insert(items.end(), it.rows.begin(), it.rows.end());
             ++k;
         }
-    b->d_tabs = static_cast<lbk::RingTab *>(batch_alloc(b, sizeof(lbk::RingTab) * b->n));
-    b->d_items = static_cast<uint32_t *>(batch_alloc(b, sizeof(uint32_t) * items.size()));
-    b->d_ranges = static_cast<int2 *>(batch_alloc(b, sizeof(int2) * b->n));
-    if (!b->d_tabs || !b->d_items || !b->d_ranges) return fail(LB_ERR_NOMEM, "device allocation failed");
-    if (cudaMemcpyAsync(b->d_tabs, tabs.data(), sizeof(lbk::RingTab) * b->n, cudaMemcpyHostToDevice, b->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(b->d_items, items.data(), sizeof(uint32_t) * items.size(), cudaMemcpyHostToDevice, b->stream) !=
+    if (int e = batch_tabs(b)) return e;
+    if (!b->d_ranges) b->d_ranges = static_cast<int2 *>(batch_alloc(b, sizeof(int2) * b->n));
+    if (!b->d_ranges || !batch_room(b, &b->d_items, &b->items_cap, sizeof(uint32_t) * items.size()))
+        return fail(LB_ERR_NOMEM, "device allocation failed");
+    if (cudaMemcpyAsync(b->d_items, items.data(), sizeof(uint32_t) * items.size(), cudaMemcpyHostToDevice, b->stream) !=
             cudaSuccess ||
         cudaMemcpyAsync(b->d_ranges, ranges.data(), sizeof(int2) * b->n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
         cudaStreamSynchronize(b->stream) != cudaSuccess)
@@ -2233,8 +2262,9 @@ int batch_ring_setup(lb_batch *b)
 }
 
 /* The resident steps for the whole batch, where every lattice fits a block. */
-int batch_resident_setup(lb_batch *b, int nsm)
+int batch_resident_setup(lb_batch *b)
 {
+    b->resident = false;
     std::vector<lbk::ResLattice> L;
     for (const lb_ctx *c : b->inst) {
         for (int j = 0; j < c->ny; ++j)
@@ -2243,29 +2273,23 @@ int batch_resident_setup(lb_batch *b, int nsm)
         if (c->ny > 0xfff0 || c->nx > 0x7fff || (b->res_pair && !c->rtab)) return LB_OK;
         L.push_back(resident_lattice(c, resident_group(c, b->res_pair)));
     }
-    if (!lbk::res_plan_build(L, b->store, b->res_pair, 1, nsm, 0, b->plan) ||
-        !lbk::resident_fits(b->store, b->res_pair, b->force, b->plan))
+    lbk::ResPlan plan;
+    if (!lbk::res_plan_build(L, b->store, b->res_pair, 1, b->nsm, 0, plan) ||
+        !lbk::resident_fits(b->store, b->res_pair, b->force, plan))
         return LB_OK;
-    b->d_plan = static_cast<unsigned char *>(batch_alloc(b, b->plan.blob.size()));
-    b->d_off = static_cast<uint32_t *>(batch_alloc(b, b->plan.off.size() * sizeof(uint32_t)));
-    if (!b->d_plan || !b->d_off) return fail(LB_ERR_NOMEM, "device allocation failed");
-    cudaError_t e = cudaMemcpyAsync(b->d_plan, b->plan.blob.data(), b->plan.blob.size(), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->d_off, b->plan.off.data(), b->plan.off.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, b->stream);
-    std::vector<lbk::RingTab> tabs(b->res_pair ? b->n : 0);
-    if (b->res_pair) {
-        for (int i = 0; i < b->n; ++i) tabs[i] = *b->inst[i]->rtab;
-        b->d_tabs = static_cast<lbk::RingTab *>(batch_alloc(b, sizeof(lbk::RingTab) * b->n));
-        if (!b->d_tabs) return fail(LB_ERR_NOMEM, "device allocation failed");
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(b->d_tabs, tabs.data(), sizeof(lbk::RingTab) * b->n, cudaMemcpyHostToDevice, b->stream);
-    }
+    const size_t ob = plan.off.size() * sizeof(uint32_t);
+    if (!batch_room(b, &b->d_plan, &b->plan_cap, plan.blob.size()) || !batch_room(b, &b->d_off, &b->off_cap, ob))
+        return fail(LB_ERR_NOMEM, "device allocation failed");
+    cudaError_t e = cudaMemcpyAsync(b->d_plan, plan.blob.data(), plan.blob.size(), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_off, plan.off.data(), ob, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return fail(LB_ERR_CUDA, "batch plan upload failed");
+    if (b->res_pair)
+        if (int t = batch_tabs(b)) return t;
+    b->plan = std::move(plan);
     b->resident = true;
-    for (lb_ctx *c : b->inst) c->ring_batch = false;   /* no carried moments to keep */
     b->threads = 512;
-    b->grid = std::min(b->plan.parts, std::max(1, nsm));
+    b->grid = std::min(b->plan.parts, std::max(1, b->nsm));
     return LB_OK;
 }
 
@@ -2310,6 +2334,97 @@ void batch_advance(lb_batch *b, int64_t nsteps)
     b->phase ^= (int)(nsteps & 1);
 }
 
+/* Block shape of the one-quad kernel: every candidate timed once, without moving the state. */
+int batch_quad_setup(lb_batch *b)
+{
+    if (b->quad_threads == 0) {
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        cudaEventCreate(&e0);
+        cudaEventCreate(&e1);
+        int e = LB_OK;
+        float best = 1e30f;
+        for (int threads : {128, 256, 512}) {
+            const int per_sm = lbk::batch_blocks(b->store, threads);
+            if (per_sm < 1) continue;
+            b->threads = threads;
+            b->grid = std::min(b->n, b->nsm * per_sm);
+            float ms = 1e30f;
+            for (int rep = 0; rep < 2 && !e; ++rep) {
+                cudaEventRecord(e0, b->stream);
+                e = batch_launch(b, 4, 0, b->stream);
+                cudaEventRecord(e1, b->stream);
+                float t = 0.0f;
+                if (!e && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess)
+                    ms = std::min(ms, t);
+            }
+            if (!e && ms < best) {
+                best = ms;
+                b->quad_threads = b->threads;
+                b->quad_grid = b->grid;
+            }
+        }
+        if (e0) cudaEventDestroy(e0);
+        if (e1) cudaEventDestroy(e1);
+        if (e) return e;
+        if (b->quad_threads == 0) return fail(LB_ERR_CUDA, "no batch block size could be launched");
+    }
+    b->threads = b->quad_threads;
+    b->grid = b->quad_grid;
+    return LB_OK;
+}
+
+uint64_t batch_maps(const lb_batch *b)
+{
+    uint64_t k = 0;
+    for (const lb_ctx *c : b->inst) k += c->map_count;
+    return k;
+}
+
+/* What follows from the members' region maps: the queue order, and the kernel with its plan
+ * or items. The resident steps where every lattice fits a block's shared memory (the bits of
+ * the other two kernels): layout 9's arithmetic for the ring batch's lattices, layout 0's for
+ * FP64; else layout 10's bodies, or the one-quad kernel, which reads the maps itself. */
+int batch_plan(lb_batch *b)
+{
+    /* most work first */
+    std::vector<std::pair<double, int>> work(b->n);
+    for (int i = 0; i < b->n; ++i) {
+        const lb_ctx *c = b->inst[i];
+        double w = 0.0;
+        for (int j = 0; j < c->ny; ++j)
+            for (int tx = 0; tx < c->ntx; ++tx) {
+                const int cols = std::min(c->nx, (tx + 1) * LB_TILE_X) - tx * LB_TILE_X;
+                w += (double)cols * c->q[c->tmap[(size_t)j * c->ntx + tx] & LB_TILE_HIGH];
+            }
+        work[i] = {-w, i};
+    }
+    std::sort(work.begin(), work.end());
+    std::vector<int> order(b->n);
+    for (int i = 0; i < b->n; ++i) order[i] = work[i].second;
+    if (cudaMemcpyAsync(b->d_order, order.data(), sizeof(int) * b->n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+        cudaStreamSynchronize(b->stream) != cudaSuccess)
+        return fail(LB_ERR_CUDA, "batch order upload failed");
+    b->resident = false;
+    if (b->ring || b->store == LB_STORE_F64)
+        if (int e = batch_resident_setup(b)) return e;
+    if (b->ring && !b->resident)
+        if (int e = batch_ring_setup(b)) return e;
+    if (!b->ring && !b->resident)
+        if (int e = batch_quad_setup(b)) return e;
+    /* the ring batch reads carried moments: a batch that comes to it from the resident steps,
+     * which keep none, has them summed */
+    for (lb_ctx *c : b->inst) {
+        const bool carry = b->ring && !b->resident;
+        if (carry && !c->ring_batch) {
+            lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), c->stream);
+            if (int e = launch_check(c, "carried moments")) return e;
+        }
+        c->ring_batch = carry;
+    }
+    b->maps_seen = batch_maps(b);
+    return LB_OK;
+}
+
 int batch_ready(lb_batch *b)
 {
     if (!b) return fail(LB_ERR_INVALID, "null batch");
@@ -2318,7 +2433,7 @@ int batch_ready(lb_batch *b)
         if (c->status != LB_OK) return c->status;
         if (c->cur != b->phase) return fail(LB_ERR_INVALID, "a lattice of the batch was stepped on its own");
     }
-    return LB_OK;
+    return batch_maps(b) == b->maps_seen ? LB_OK : batch_plan(b);   /* a member has another map */
 }
 
 }  // namespace
@@ -2376,73 +2491,16 @@ int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps,
         c->ring_batch = b->ring;
         b->inst.push_back(c);
     }
-    /* most work first */
-    std::vector<std::pair<double, int>> work(n);
-    for (int i = 0; i < n; ++i) {
-        const lb_ctx *c = b->inst[i];
-        double w = 0.0;
-        for (int j = 0; j < c->ny; ++j)
-            for (int tx = 0; tx < c->ntx; ++tx) {
-                const int cols = std::min(c->nx, (tx + 1) * LB_TILE_X) - tx * LB_TILE_X;
-                w += (double)cols * c->q[c->tmap[(size_t)j * c->ntx + tx] & LB_TILE_HIGH];
-            }
-        work[i] = {-w, i};
-    }
-    std::sort(work.begin(), work.end());
-    std::vector<int> order(n);
-    for (int i = 0; i < n; ++i) order[i] = work[i].second;
     b->d_order = static_cast<int *>(batch_alloc(b, sizeof(int) * n));
     b->d_queue = static_cast<unsigned int *>(batch_alloc(b, 256));
     int e = (b->d_order && b->d_queue) ? LB_OK : fail(LB_ERR_NOMEM, "device allocation failed");
-    if (!e && cudaMemcpyAsync(b->d_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess)
-        e = fail(LB_ERR_CUDA, "batch order upload failed");
     if (!e) e = b->store == LB_STORE_F64 ? batch_upload_params<double>(b) : batch_upload_params<float>(b);
-    int dev = 0, nsm = 0;
+    int dev = 0;
     if (!e &&
-        (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
+        (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
         e = fail(LB_ERR_CUDA, "device query failed");
-    /* the resident steps where every lattice fits a block's shared memory (the bits of the
-     * other two kernels): layout 9's arithmetic for the ring batch's lattices, layout 0's
-     * for FP64 */
     b->res_pair = b->ring;
-    if (!e && (b->ring || b->store == LB_STORE_F64)) e = batch_resident_setup(b, nsm);
-    if (!e && b->ring && !b->resident) e = batch_ring_setup(b);
-    /* block size of the one-quad kernel: time each candidate without moving the state */
-    if (!e && !b->ring && !b->resident) {
-        cudaEvent_t e0 = nullptr, e1 = nullptr;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        float best = 1e30f;
-        int best_threads = 0, best_grid = 0;
-        for (int threads : {128, 256, 512}) {
-            const int per_sm = lbk::batch_blocks(b->store, threads);
-            if (per_sm < 1) continue;
-            b->threads = threads;
-            b->grid = std::min(n, nsm * per_sm);
-            float ms = 1e30f;
-            for (int rep = 0; rep < 2 && !e; ++rep) {
-                cudaEventRecord(e0, b->stream);
-                e = batch_launch(b, 4, 0, b->stream);
-                cudaEventRecord(e1, b->stream);
-                float t = 0.0f;
-                if (!e && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess)
-                    ms = std::min(ms, t);
-            }
-            if (!e && ms < best) {
-                best = ms;
-                best_threads = b->threads;
-                best_grid = b->grid;
-            }
-        }
-        if (e0) cudaEventDestroy(e0);
-        if (e1) cudaEventDestroy(e1);
-        if (!e && best_threads > 0) {
-            b->threads = best_threads;
-            b->grid = best_grid;
-        } else if (!e) {
-            e = fail(LB_ERR_CUDA, "no batch block size could be launched");
-        }
-    }
+    if (!e) e = batch_plan(b);
     if (e) {
         batch_release(b);
         delete b;
