@@ -146,6 +146,7 @@ struct lb_ctx {
     size_t rplan_cap = 0;
     std::tuple<int, int, int, int, int, uint64_t> res_key{};
     bool res_variant = false;       /* the layout in use stands in for the resident steps */
+    int res_cluster = 0;            /* the cluster size they were timed fastest with */
     uint32_t dcol_hash = 0;         /* FNV-1a of those deltas (0: one reference density) */
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     /* learned placement */
@@ -988,6 +989,7 @@ int setup_resident(lb_ctx *c, float *step_ms)
         if (!lbk::res_plan_build(one, c->store, c->res_pair, known, 1, sr, c->rplan)) return LB_OK;
         if (int e = resident_upload(c)) return e;
         c->res_on = true;
+        c->res_cluster = known;
         return LB_OK;
     }
     cudaEvent_t e0, e1;
@@ -1026,6 +1028,7 @@ int setup_resident(lb_ctx *c, float *step_ms)
         g_res_tune[key] = best_c;
     }
     c->res_on = true;
+    c->res_cluster = best_c;
     *step_ms = best / STEPS;
     return LB_OK;
 }
@@ -1812,32 +1815,29 @@ int lb_learned_map_now(lb_ctx *c)
 }  // extern "C"
 
 namespace {
-/* After a map change: the resident plan of the new map with the cluster size in use, or a
- * layout where the new map has none (timed on this map; every layout reads the level that
- * finalize_level completes next). */
+/* After a map change of a lattice on the resident steps: the plan of the new map, with the
+ * cluster size that was timed fastest where that fits. Where the new map has none, the steps go
+ * one launch each on the layout that lb_info names all along, which has the same bits; nothing
+ * is timed inside a run, and a later map may take the resident steps again. */
 int replan(lb_ctx *c)
 {
     if (!c->res_variant) return LB_OK;
     const int sr = (c->opts.rounding == LB_ROUND_STOCHASTIC &&
                     (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV)) ? 1 : 0;
+    const bool force = c->opts.gx != 0.0 || c->opts.gy != 0.0;
     c->res_on = false;
-    if (resident_candidate(c)) {
-        const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
-        const int now = c->rplan.cluster;
-        for (int cl : {now, 1, 2, 4, 8, 16})
-            if (lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, c->rplan)) {
-                if (int e = resident_upload(c)) return e;
-                c->res_on = true;
-                return LB_OK;
-            }
+    if (!resident_candidate(c)) return LB_OK;
+    const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
+    for (int cl : {c->res_cluster, 1, 2, 4, 8, 16}) {
+        lbk::ResPlan plan;
+        if (!lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, plan) ||
+            !lbk::resident_fits(c->store, c->res_pair, force, plan))
+            continue;
+        c->rplan = std::move(plan);
+        if (int e = resident_upload(c)) return e;
+        c->res_on = true;
+        return LB_OK;
     }
-    /* a later map may take the resident steps again: the flag stays */
-    float ms = 0.0f;
-    const int keep = c->variant;
-    c->variant = -1;   /* the level is completed for every layout */
-    if (int e = finalize_level(c, c->cur)) return e;
-    c->variant = choose_variant(c, &ms);
-    if (c->variant < 0) c->variant = keep;
     return LB_OK;
 }
 
