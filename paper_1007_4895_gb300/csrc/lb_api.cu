@@ -956,12 +956,18 @@ int resident_steps(lb_ctx *c, int n, int advance)
     return use_f64(c) ? resident_steps_t<double>(c, n, advance) : resident_steps_t<float>(c, n, advance);
 }
 
-std::mutex g_tune_mu;   /* the tuners' caches */
-std::map<std::tuple<int, int, int, int, int, uint64_t>, int> g_res_tune;   /* cluster size, 0: layouts */
+/* The tuners' caches: what was chosen, and the ms of a step with it, so that the resident
+ * steps and the layouts are compared by their times whichever of the two was known already */
+struct Tuned {
+    int choice;
+    float step_ms;
+};
+std::mutex g_tune_mu;
+std::map<std::tuple<int, int, int, int, int, uint64_t>, Tuned> g_res_tune;   /* cluster size, 0: layouts */
 
 /* Chooses the cluster size of the resident steps by timing (or takes the cached choice)
- * and leaves the plan on the device; res_on stays false when nothing fits. Returns the
- * time of a step in ms (0: taken from the cache). */
+ * and leaves the plan on the device; res_on stays false when nothing fits. *step_ms: the
+ * time of a step. */
 int setup_resident(lb_ctx *c, float *step_ms)
 {
     c->res_on = false;
@@ -981,7 +987,10 @@ int setup_resident(lb_ctx *c, float *step_ms)
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_res_tune.find(key);
-        if (it != g_res_tune.end()) known = it->second;
+        if (it != g_res_tune.end()) {
+            known = it->second.choice;
+            *step_ms = it->second.step_ms;
+        }
     }
     if (known == 0) return LB_OK;
     const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
@@ -1025,7 +1034,7 @@ int setup_resident(lb_ctx *c, float *step_ms)
     if (int e = resident_upload(c)) return e;
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
-        g_res_tune[key] = best_c;
+        g_res_tune[key] = {best_c, best / STEPS};
     }
     c->res_on = true;
     c->res_cluster = best_c;
@@ -1037,7 +1046,7 @@ int setup_resident(lb_ctx *c, float *step_ms)
  * writing the other one, which the next step overwrites) and keeps the fastest. Results
  * are cached per (storage, grid, sets, interface mode, map) for the process. */
 using TuneKey = std::tuple<int, int, int, int, int, int, uint64_t>;
-std::map<TuneKey, int> g_tune;
+std::map<TuneKey, Tuned> g_tune;
 
 template <typename R>
 int autotune_t(lb_ctx *c, float *step_ms)
@@ -1051,7 +1060,10 @@ int autotune_t(lb_ctx *c, float *step_ms)
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune.find(key);
-        if (it != g_tune.end()) return it->second;
+        if (it != g_tune.end()) {
+            *step_ms = it->second.step_ms;
+            return it->second.choice;
+        }
     }
     StepParams<R> p = make_params<R>(c, c->cur, c->cur ^ 1, c->t + c->dt);
     cudaEvent_t e0, e1;
@@ -1096,7 +1108,7 @@ int autotune_t(lb_ctx *c, float *step_ms)
     if (cudaGetLastError() != cudaSuccess) return 0;
     *step_ms = best_ms / 5.0f;
     std::lock_guard<std::mutex> g(g_tune_mu);
-    g_tune[key] = best;
+    g_tune[key] = {best, *step_ms};
     return best;
 }
 
@@ -1118,7 +1130,7 @@ int choose_steps(lb_ctx *c)
     float res_ms = 0.0f;
     c->res_variant = false;
     if (int e = setup_resident(c, &res_ms)) return e;
-    if (c->res_on && (res_ms == 0.0f || c->rplan.cost * c->rplan.cluster <= RES_ALWAYS)) {
+    if (c->res_on && c->rplan.cost * c->rplan.cluster <= RES_ALWAYS) {
         c->variant = c->res_pair ? 9 : 0;   /* the layout with the same bits */
         c->res_variant = true;
         return LB_OK;
@@ -1128,8 +1140,7 @@ int choose_steps(lb_ctx *c)
     if (c->res_on && lay_ms > 0.0f && lay_ms < res_ms) {
         c->res_on = false;
         std::lock_guard<std::mutex> g(g_tune_mu);
-        for (auto &kv : g_res_tune)   /* this lattice takes the layouts from now on */
-            if (kv.first == c->res_key) kv.second = 0;
+        g_res_tune[c->res_key] = {0, 0.0f};   /* its kind takes the layouts from now on */
     } else if (c->res_on) {
         c->variant = c->res_pair ? 9 : 0;
         c->res_variant = true;
