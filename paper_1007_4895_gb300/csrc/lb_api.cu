@@ -916,6 +916,14 @@ int resident_upload_t(lb_ctx *c)
     return cuda_check(c, cudaMemcpyAsync(d, h, off + ob, cudaMemcpyHostToDevice, c->stream), "resident plan upload");
 }
 int resident_upload(lb_ctx *c) { return use_f64(c) ? resident_upload_t<double>(c) : resident_upload_t<float>(c); }
+/* the plan in c->rplan on the device and the resident steps on; off where the allocator has no
+ * room for it: the lattice then runs on the layouts */
+int resident_start(lb_ctx *c)
+{
+    const int e = resident_upload(c);
+    c->res_on = e == LB_OK;
+    return e == LB_ERR_NOMEM ? LB_OK : e;
+}
 
 /* n <= RES_OSC steps with oscillating walls, any n with steady ones; advance = 0: the
  * level is left as it is */
@@ -994,10 +1002,8 @@ int setup_resident(lb_ctx *c, float *step_ms)
     const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
     if (known > 0) {
         if (!lbk::res_plan_build(one, c->store, c->res_pair, known, 1, sr, c->rplan)) return LB_OK;
-        if (int e = resident_upload(c)) return e;
-        c->res_on = true;
         c->res_cluster = known;
-        return LB_OK;
+        return resident_start(c);
     }
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
@@ -1036,15 +1042,13 @@ int setup_resident(lb_ctx *c, float *step_ms)
         g_res_tune[key] = {0, 0.0f};
     }
     if (best_c == 0 || !lbk::res_plan_build(one, c->store, c->res_pair, best_c, 1, sr, c->rplan)) return LB_OK;
-    if (int e = resident_upload(c)) return e;
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         g_res_tune[key] = {best_c, best / STEPS};
     }
-    c->res_on = true;
     c->res_cluster = best_c;
     *step_ms = best / STEPS;
-    return LB_OK;
+    return resident_start(c);
 }
 
 /* Autotuner: times every step-kernel layout on this lattice (reading the current level,
@@ -1850,9 +1854,7 @@ int replan(lb_ctx *c)
             !lbk::resident_fits(c->store, c->res_pair, force, plan))
             continue;
         c->rplan = std::move(plan);
-        if (int e = resident_upload(c)) return e;
-        c->res_on = true;
-        return LB_OK;
+        return resident_start(c);
     }
     return LB_OK;
 }
@@ -2295,7 +2297,7 @@ int batch_resident_setup(lb_batch *b)
         return LB_OK;
     const size_t ob = plan.off.size() * sizeof(uint32_t);
     if (!batch_room(b, &b->d_plan, &b->plan_cap, plan.blob.size()) || !batch_room(b, &b->d_off, &b->off_cap, ob))
-        return fail(LB_ERR_NOMEM, "device allocation failed");
+        return LB_OK;   /* no room for a plan: the other batch kernels */
     cudaError_t e = cudaMemcpyAsync(b->d_plan, plan.blob.data(), plan.blob.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_off, plan.off.data(), ob, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
