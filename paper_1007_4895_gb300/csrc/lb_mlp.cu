@@ -454,35 +454,35 @@ __global__ void to_bf16_kernel(const float *th, __nv_bfloat16 *wb)
  * once per block. A node with a non-finite feature gets p = NaN.
  *
  * What bounds it: the 128 GELUs of a node, on the FP32 and special-function units. They
- * are evaluated in pairs as
- *   gelu(a) = max(a, 0) - x E(x),   x = min(|a|, 5.75),   E(x) = erfc(x / sqrt 2) / 2,
- * with log2 E a polynomial of degree 9 in packed FP32 arithmetic and one exp2 each: 8.5
- * instructions a value against about 30 of the erf form. The coefficients are a weighted
- * minimax fit (iteratively reweighted least squares on Chebyshev nodes) of log2 E on
- * [0, 5.75] that bounds the error of x E by 1e-8; in FP32 the result is within 2.4e-7 of
- * GELU on [-9, 9] (rms 5.0e-8; the erf form 4.5e-7, rms 6.4e-8), the cut at 5.75 included
- * (x E = 2.6e-8 there). 2 097 152 nodes: 345 us -> 201 us. */
-__device__ __forceinline__ float max_nan(float a, float b)
+ * are evaluated in pairs, as twice the GELU (the weights behind it are halved, which is exact):
+ *   2 gelu(a) = (a + |a|) + y 2^P(y),   y = max(-|a|, -7),   2^P(-x) = erfc(x / sqrt 2),
+ * with P a polynomial of degree 9 without a constant term (so that near zero, where P is
+ * small, its rounding is too) in packed FP32 arithmetic, and one exp2 each: 8 instructions a
+ * value against about 30 of the erf form. The coefficients are a weighted minimax fit
+ * (iteratively reweighted least squares on Chebyshev nodes of [0, 7], each rounded to FP32 and
+ * the rest fitted again) of log2 erfc, off by at most 3.7e-9 of GELU. a + |a| keeps the erf
+ * form's values at NaN and the infinities (2 gelu(-inf) = NaN: the node has no p).
+ * Against FP64, largest error, the erf form in FP32 in brackets: relative 1.8e-7 (1.3e-7) for
+ * |a| < 0.25, 2.4e-7 (2.2e-7) to 1, 9.0e-8 (1.2e-7) for 1 < a < 9; absolute 4.4e-8 (6.5e-8) for
+ * -2 < a < -1, 2.2e-8 (1.2e-7) below, 1.2e-11 (0) below -7. Rms: up to 1.6 times the erf form's
+ * for -0.25 < a < 0, 1.1 times for 0 < a < 0.05 and -1 < a < -0.25, smaller elsewhere. (An earlier
+ * fit to log2 of half the erfc, cut off at 5.75, was off by 9.8e-7 of the value near zero and by
+ * 2.6e-8 below -5.75.)
+ * 2 097 152 nodes: 345 us in the erf form, 201 with the earlier fit, 207 with this one. */
+__device__ __forceinline__ float2 twice_gelu(float2 a)
 {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 gelu2(float2 a)
-{
-    const float2 x = make_float2(fminf(fabsf(a.x), 5.75f), fminf(fabsf(a.y), 5.75f));
-    constexpr float C[10] = {-0.9999986886978149f,     -1.1511249542236328f,    -0.4591113328933716f,
-                             -0.052710652351379395f,   0.007307772058993578f,   -0.0002848419244401157f,
-                             -0.00014207529602572322f, 3.552617636159994e-05f,  -3.6852788980468176e-06f,
-                             1.509595932702723e-07f};
-    float2 p = make_float2(C[9], C[9]);
+    const float2 y = make_float2(fmaxf(-fabsf(a.x), -7.0f), fmaxf(-fabsf(a.y), -7.0f));
+    constexpr float C[9] = {1.1511046886444092f,       -0.4592166244983673f,     0.05245400220155716f,
+                            0.006968232337385416f,     2.4232918804045767e-05f,  -0.00026060346863232553f,
+                            -6.681260128971189e-05f,   -8.086775778792799e-06f,  -4.048496009545488e-07f};
+    float2 p = make_float2(C[8], C[8]);
 #pragma unroll
-    for (int k = 8; k >= 0; --k) p = __ffma2_rn(p, x, make_float2(C[k], C[k]));
+    for (int k = 7; k >= 0; --k) p = __ffma2_rn(p, y, make_float2(C[k], C[k]));
+    p = __fmul2_rn(p, y);
     float2 e;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(p.x));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(p.y));
-    const float2 r = make_float2(max_nan(a.x, 0.0f), max_nan(a.y, 0.0f));
-    return __ffma2_rn(make_float2(-x.x, -x.y), e, r);
+    return __ffma2_rn(y, e, make_float2(a.x + fabsf(a.x), a.y + fabsf(a.y)));
 }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
@@ -509,19 +509,19 @@ __device__ __forceinline__ uint32_t pack_bf16_raw(__nv_bfloat16 lo, __nv_bfloat1
 }
 
 /* (not inlined: rare, and 32 copies of it would not fit the instruction cache) */
-__device__ __noinline__ uint32_t gelu2_erf_bf16(float2 a) { return pack_bf16(gelu(a.x), gelu(a.y)); }
+__device__ __noinline__ uint32_t twice_gelu_erf_bf16(float2 a) { return pack_bf16(2.0f * gelu(a.x), 2.0f * gelu(a.y)); }
 
-/* A pair of GELUs rounded to BF16 as the erf form rounds them: a value that lies within 4
- * FP32 units of a rounding boundary (one in 4096) is formed again in the erf form. (Below
- * -1.5, where the erf form itself is off by more, the two may round apart; the values are
- * below 0.1 there.) */
-__device__ __forceinline__ uint32_t gelu2_bf16(float2 a)
+/* A pair of them rounded to BF16: a value that lies within 4 FP32 units of a rounding boundary
+ * (one in 4096) is formed again in the erf form. For a > -1 the errors of the two forms add up
+ * to less than that distance, so every value is rounded as the erf form rounds it; below, where
+ * the erf form's own error is larger, the two may round apart. */
+__device__ __forceinline__ uint32_t twice_gelu_bf16(float2 a)
 {
     constexpr float D = 4.76837158e-7f;   /* 2^-21 */
-    const float2 h = gelu2(a);
+    const float2 h = twice_gelu(a);
     const float2 lo = __fmul2_rn(h, make_float2(1.0f - D, 1.0f - D)), hi = __fmul2_rn(h, make_float2(1.0f + D, 1.0f + D));
     const uint32_t r = pack_bf16(lo.x, lo.y);
-    return r == pack_bf16(hi.x, hi.y) ? r : gelu2_erf_bf16(a);
+    return r == pack_bf16(hi.x, hi.y) ? r : twice_gelu_erf_bf16(a);
 }
 
 __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
                                                            float *__restrict__ p)
 {
     /* operand fragments of the weights: B[k][n] of layer 1 is W1[n][k] (k < 8, zero
-     * above), of layer 2 W2[n][k]; fragment register r of lane l holds the rows
+     * above), of layer 2 W2[n][k] / 2; fragment register r of lane l holds the rows
      * 2 (l % 4) + {0, 1} (+ 8 for r = 1) of column l / 4 */
     __shared__ uint32_t w1f[8][32];
     __shared__ uint2 w2f[4][8][32];
@@ -544,13 +544,14 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
         const int kt = k / 256, nt = (k / 32) % 8, l = k % 32;
         const int col = 8 * nt + l / 4, row = 16 * kt + 2 * (l % 4);
         const __nv_bfloat16 *w = wb + OFF_W2 + col * NH;
-        w2f[kt][nt][l] = make_uint2(pack_bf16_raw(w[row], w[row + 1]), pack_bf16_raw(w[row + 8], w[row + 9]));
+        auto half = [&](int r) { return 0.5f * __bfloat162float(w[r]); };   /* activations come doubled */
+        w2f[kt][nt][l] = make_uint2(pack_bf16(half(row), half(row + 1)), pack_bf16(half(row + 8), half(row + 9)));
     }
     for (int k = threadIdx.x; k < NH / 2; k += blockDim.x) {
         auto two = [&](int off) { return make_float2(__bfloat162float(wb[off + 2 * k]), __bfloat162float(wb[off + 2 * k + 1])); };
         b1s[k] = two(OFF_B1);
         b2s[k] = two(OFF_B2);
-        w3s[k] = two(OFF_W3);
+        w3s[k] = __fmul2_rn(two(OFF_W3), make_float2(0.5f, 0.5f));
     }
     if (threadIdx.x < 2 * NF) nm[threadIdx.x] = norm[threadIdx.x];
     if (threadIdx.x == 0) b3s = __bfloat162float(wb[OFF_B3]);
@@ -598,8 +599,8 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
                 const uint32_t a[4] = {a1[m][0], a1[m][1], 0u, 0u};
                 mma_bf16(c, a, b);
                 const int kt = nt >> 1, hi = (nt & 1) * 2;
-                a2[m][kt][hi] = gelu2_bf16(__fadd2_rn(make_float2(c[0], c[1]), bias));
-                a2[m][kt][hi + 1] = gelu2_bf16(__fadd2_rn(make_float2(c[2], c[3]), bias));
+                a2[m][kt][hi] = twice_gelu_bf16(__fadd2_rn(make_float2(c[0], c[1]), bias));
+                a2[m][kt][hi + 1] = twice_gelu_bf16(__fadd2_rn(make_float2(c[2], c[3]), bias));
             }
         }
         /* layer 2 -> GELU -> W3 dot product */
@@ -617,8 +618,8 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
             const float2 bias = b2s[4 * nt + q], w3 = w3s[4 * nt + q];
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
-                const float2 h0 = gelu2(__fadd2_rn(make_float2(c[m][0], c[m][1]), bias));
-                const float2 h1 = gelu2(__fadd2_rn(make_float2(c[m][2], c[m][3]), bias));
+                const float2 h0 = twice_gelu(__fadd2_rn(make_float2(c[m][0], c[m][1]), bias));
+                const float2 h1 = twice_gelu(__fadd2_rn(make_float2(c[m][2], c[m][3]), bias));
                 z[2 * m] = fmaf(h0.y, w3.y, fmaf(h0.x, w3.x, z[2 * m]));
                 z[2 * m + 1] = fmaf(h1.y, w3.y, fmaf(h1.x, w3.x, z[2 * m + 1]));
             }
