@@ -1835,6 +1835,22 @@ int lb_learned_map_now(lb_ctx *c)
 }  // extern "C"
 
 namespace {
+/* the plan of the resident steps on `cluster` blocks into c->rplan; false (and c->rplan as it
+ * was) where the lattice has none */
+bool resident_plan(lb_ctx *c, int cluster)
+{
+    if (!resident_candidate(c) || (c->res_pair && !c->rtab)) return false;
+    const int sr = (c->opts.rounding == LB_ROUND_STOCHASTIC &&
+                    (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV)) ? 1 : 0;
+    const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
+    lbk::ResPlan plan;
+    if (!lbk::res_plan_build(one, c->store, c->res_pair, cluster, 1, sr, plan) ||
+        !lbk::resident_fits(c->store, c->res_pair, c->opts.gx != 0.0 || c->opts.gy != 0.0, plan))
+        return false;
+    c->rplan = std::move(plan);
+    return true;
+}
+
 /* After a map change of a lattice on the resident steps: the plan of the new map, with the
  * cluster size that was timed fastest where that fits. Where the new map has none, the steps go
  * one launch each on the layout that lb_info names all along, which has the same bits; nothing
@@ -1842,20 +1858,9 @@ namespace {
 int replan(lb_ctx *c)
 {
     if (!c->res_variant) return LB_OK;
-    const int sr = (c->opts.rounding == LB_ROUND_STOCHASTIC &&
-                    (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV)) ? 1 : 0;
-    const bool force = c->opts.gx != 0.0 || c->opts.gy != 0.0;
     c->res_on = false;
-    if (!resident_candidate(c)) return LB_OK;
-    const std::vector<lbk::ResLattice> one{resident_lattice(c, 1)};
-    for (int cl : {c->res_cluster, 1, 2, 4, 8, 16}) {
-        lbk::ResPlan plan;
-        if (!lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, plan) ||
-            !lbk::resident_fits(c->store, c->res_pair, force, plan))
-            continue;
-        c->rplan = std::move(plan);
-        return resident_start(c);
-    }
+    for (int cl : {c->res_cluster, 1, 2, 4, 8, 16})
+        if (resident_plan(c, cl)) return resident_start(c);
     return LB_OK;
 }
 
@@ -1890,6 +1895,21 @@ int set_region_map_impl(lb_ctx *c, const uint8_t *map)
 }  // namespace
 
 extern "C" {
+
+/* For the tests, not part of the ABI (include/lb.h): the number of blocks that the resident
+ * steps of this lattice run on, 0 where its steps go one launch each. cluster > 0 puts it on
+ * them with that many blocks first; -1 where it has no such plan. */
+int lbi_resident_cluster(lb_ctx *c, int cluster)
+{
+    if (!c || c->status != LB_OK) return -1;
+    if (cluster > 0) {
+        if (!resident_plan(c, cluster) || resident_start(c) != LB_OK || !c->res_on) return -1;
+        c->res_cluster = cluster;
+        c->res_variant = true;
+        c->variant = c->res_pair ? 9 : 0;
+    }
+    return c->res_on ? c->rplan.cluster : 0;
+}
 
 int lb_get_populations(lb_ctx *c, int32_t set, double *dst)
 {
