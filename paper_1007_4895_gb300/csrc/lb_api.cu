@@ -782,6 +782,13 @@ void launch_variant(lb_ctx *c, int variant, const StepParams<R> &p)
             lbk::launch_ring(c->store, p, c->stream);
             return;
         }
+        if (variant == 10 && !p.has_force && p.pressure[1] && !pressure_in_step(p)) {
+            /* the pressure pass follows: the kernel takes the columns' nodes for inner ones */
+            StepParams<R> q = p;
+            q.pressure[0] = q.pressure[1] = 0;
+            launch_variant<R>(c, variant, q);
+            return;
+        }
         if (variant == 10 && c->tiles_ok && !p.sr && !c->tunits_h.empty() &&
             lbk::launch_tiles(c->store, p, *c->rtab, c->tmaps[c->cur], c->d_tunits, (int)c->tunits_h.size(), c->tunits_n1,
                               c->d_rctr, c->d_err, c->stream) == 0)

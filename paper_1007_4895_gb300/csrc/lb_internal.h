@@ -105,11 +105,10 @@ struct StepParams {
  * first and last tiles, from the node one step inwards. False where that is left to the
  * pressure pass: with a body force (its registers would weigh on the force kernels), and
  * where the last tile holds the boundary column alone (nx = 1 mod 128): the node inwards is
- * then another warp's or block's, whose store this launch does not order before the read. */
+ * then another warp's or block's, whose store this launch does not order before the read. (The
+ * host decides, and clears p.pressure for the kernel: a test in the tile kernel itself cost it 8
+ * to 16 more spilled bytes.) */
 template <typename R>
-#ifdef __CUDACC__
-__host__ __device__
-#endif
 inline bool pressure_in_step(const StepParams<R> &p)
 {
     return !p.has_force && !(p.pressure[1] && p.nx % LB_TILE_X == 1);

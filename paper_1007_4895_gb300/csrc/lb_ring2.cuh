@@ -661,10 +661,11 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, ring10_blocks<ST>())
         __syncwarp();
         /* the pressure columns of this row: the pressure pass's work, done here once the
          * row's nodes are stored (the warp barrier above makes them visible to all lanes; the
-         * node inwards is in this row of this tile: see pressure_in_step) */
+         * node inwards is in this row of this tile: where it is not, the host leaves the columns
+         * to the pressure pass and clears p.pressure, see pressure_in_step) */
         if constexpr (!FORCE) {
-            if (tx == 0 && p.pressure[0] && pressure_in_step(p)) pressure_row<ST>(p, j, 0);
-            if (tx == p.ntx - 1 && p.pressure[1] && pressure_in_step(p)) pressure_row<ST>(p, j, 1);
+            if (tx == 0 && p.pressure[0]) pressure_row<ST>(p, j, 0);
+            if (tx == p.ntx - 1 && p.pressure[1]) pressure_row<ST>(p, j, 1);
         }
     }
     /* the last warp out zeroes the counters for the next launch */

@@ -581,8 +581,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
             __syncwarp();
             /* the pressure columns of this row, once its nodes are stored (see lb_ring2.cuh) */
             if constexpr (!FORCE) {
-                if (alive && u.x == 0 && p.pressure[0] && pressure_in_step(p)) pressure_row<ST>(p, j, 0);
-                if (alive && u.x == p.ntx - 1 && p.pressure[1] && pressure_in_step(p)) pressure_row<ST>(p, j, 1);
+                if (alive && u.x == 0 && p.pressure[0]) pressure_row<ST>(p, j, 0);
+                if (alive && u.x == p.ntx - 1 && p.pressure[1]) pressure_row<ST>(p, j, 1);
             }
         } else {
             __syncwarp();   /* every lane has its copy of the unit: the slot may be refilled */
