@@ -1094,10 +1094,14 @@ int autotune_t(lb_ctx *c, float *step_ms)
                     (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV);
     for (int v = 0; v < LB_NUM_VARIANTS; ++v) {
         if (!variant_available(c, v) || (v == 10 && sr)) continue;
-        /* 16-bit storage and per-column references: layout 10 rounds unlike layouts 0 to 8, and
-         * on smaller lattices the runs so far have those layouts' values; it is offered from
-         * the size on where it has always been the fastest */
-        if (v == 10 && (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV || c->d_dcol) &&
+        /* 16-bit storage under 1.25 M nodes: not offered. Layout 10 rounds unlike layouts 0 to 6,
+         * and in 16 bits a rounding that falls the other way moves the fields by 1e-4 to 5e-3
+         * within 20 steps; runs of these sizes have had layout 5's or 6's values, because on
+         * rows layout 10 is within 3 % of them or slower there (us a step, FP16, rows / best of
+         * the others: 1024 x 128 45.2 / 45.0, 4096 x 128 56.2 / 51.3, 4096 x 300 66.5 / 61.2) and
+         * wins from about there on (2048 x 700 69.2 / 79.7). Tiles would win below (1024 x 128
+         * 27.0), at the price of those values. */
+        if (v == 10 && (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV) &&
             (long long)c->nx * c->ny < 1250000LL)
             continue;
         /* with the pressure pass, which layout 10 does inside its kernel where it can */
