@@ -148,8 +148,9 @@ typedef struct {
  *      where both levels fit L2, blocks take tiles streamed by the tensor memory accelerator.
  * With variant < 0 a small x-periodic lattice whose rows each use one set advances all the
  * steps of an lb_step call in one launch with its state in shared memory (LB_IFACE_HERMITE,
- * one reference density); lb_info then names the layout with the same bits, 9 (FP32 storage)
- * or 0.
+ * one reference density), or, where that does not pay for the steps of the call, one launch a
+ * step on a layout of the same bits; lb_info then names 9 (FP32 storage) or 0, whose bits they
+ * are.
  * A layout this lattice cannot use falls back to 0. All layouts give the same result
  * (0, 2, 3 and 4 the same bits; 1, 5, 6 the same bits as 0 or differing in rounding;
  * 7, 8 and 9 differ from 0 in rounding; 10 the same bits as 9). */

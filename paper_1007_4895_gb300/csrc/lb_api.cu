@@ -149,6 +149,8 @@ struct lb_ctx {
     std::tuple<int, int, int, int, int, uint64_t> res_key{};
     bool res_variant = false;       /* the layout in use stands in for the resident steps */
     int res_cluster = 0;            /* the cluster size they were timed fastest with */
+    int64_t res_min = 1;            /* steps a launch of them must have to pay; fewer go on res_alt */
+    int res_alt = 0;                /* layout of the same bits, one launch a step */
     uint32_t dcol_hash = 0;         /* FNV-1a of those deltas (0: one reference density) */
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     /* learned placement */
@@ -380,7 +382,7 @@ int finalize_level_t(lb_ctx *c, int level)
     lbk::launch_pressure<R>(c->store, p, st);
     /* carried moments of this level: read only by layouts 4 and 10 (and by the
      * autotuner, which runs while no layout is chosen yet) */
-    if (c->variant < 0 || c->variant == 4 || c->variant == 10 || c->ring_batch)
+    if (c->variant < 0 || c->variant == 4 || c->variant == 10 || c->ring_batch || (c->res_variant && c->res_alt == 10))
         lbk::launch_aux<R>(c->store, p, st);
     return launch_check(c, "finalize");
 }
@@ -975,8 +977,90 @@ struct Tuned {
     int choice;
     float step_ms;
 };
+struct TunedRes {
+    int cluster;       /* 0: the layouts */
+    float step_ms;     /* in a launch of RES_TUNE_STEPS */
+    int64_t min_steps;
+    int alt;
+};
+constexpr int RES_TUNE_STEPS = 24;
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, uint64_t>, Tuned> g_res_tune;   /* cluster size, 0: layouts */
+std::map<std::tuple<int, int, int, int, int, uint64_t>, TunedRes> g_res_tune;
+
+/* ms of one step of layout v (reading the current level, writing the other one, which the next
+ * step overwrites), with the pressure pass, which layout 10 does inside its kernel where it can */
+template <typename R>
+float layout_ms(lb_ctx *c, int v, const StepParams<R> &p, cudaEvent_t e0, cudaEvent_t e1)
+{
+    auto one = [&] {
+        launch_variant<R>(c, v, p);
+        if (v != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
+    };
+    for (int k = 0; k < 2; ++k) one();
+    cudaEventRecord(e0, c->stream);
+    for (int k = 0; k < 5; ++k) one();
+    cudaEventRecord(e1, c->stream);
+    float ms = 0.0f;
+    return cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess ? ms / 5.0f : 1e30f;
+}
+
+/* ms of a launch of n resident steps; advance (n odd then): with the write-back, into the other
+ * level too */
+float resident_ms(lb_ctx *c, int n, int advance, cudaEvent_t e0, cudaEvent_t e1)
+{
+    float best = 1e30f;
+    for (int rep = 0; rep < 2; ++rep) {
+        cudaEventRecord(e0, c->stream);
+        if (resident_steps(c, n, advance) != LB_OK) {
+            c->status = LB_OK;   /* this size cannot be launched here */
+            break;
+        }
+        cudaEventRecord(e1, c->stream);
+        float t = 0.0f;
+        if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess) best = std::min(best, t);
+    }
+    return best;
+}
+
+/* the fewest steps for which a launch taking `one` ms with one step and `many` with n beats
+ * `once` ms and `step` ms a step; INT64_MAX: none */
+int64_t shortest_call(float one, float many, int n, float once, float step)
+{
+    const float a = (many - one) / (float)(n - 1), fixed = one - a;
+    if (!(a < step)) return INT64_MAX;
+    return std::max<int64_t>(1, (int64_t)std::ceil((fixed - once) / (step - a)));
+}
+
+/* How many steps a resident launch must have to pay, and the layout that takes fewer. A launch
+ * loads and writes back the whole level with a few blocks, which a step of the layouts does on
+ * the whole chip: 128 x 128 in FP32 deviations 90 us a call of one step, 25 a further step,
+ * against 30 on the layouts; 8 x 64 16 and 5 against 31. Layouts with the resident steps' bits
+ * are timed: 9 and 10 (FP32), 0, 5 and 6 (FP64 and 16-bit storage). Not where one resident step is
+ * below what any of them takes (a launch and a chain of 36 populations: 30 us, in FP64 220). */
+void tune_short_calls(lb_ctx *c, cudaEvent_t e0, cudaEvent_t e1)
+{
+    c->res_min = 1;
+    c->res_alt = c->res_pair ? 9 : 0;
+    const float one = resident_ms(c, 1, 1, e0, e1);
+    if (one <= (use_f64(c) ? 0.150f : 0.025f)) return;
+    float lay = 1e30f;
+    auto time = [&](auto r) {
+        using R = decltype(r);
+        const StepParams<R> p = make_params<R>(c, c->cur, c->cur ^ 1, c->t + c->dt);
+        for (int v : {9, 10, 0, 5, 6}) {
+            if ((v >= 9) != c->res_pair || !variant_available(c, v)) continue;
+            const float ms = layout_ms<R>(c, v, p, e0, e1);
+            if (ms < 0.97f * lay) {
+                lay = ms;
+                c->res_alt = v;
+            }
+        }
+    };
+    if (use_f64(c)) time(0.0);
+    else time(0.0f);
+    constexpr int MANY = 25;
+    c->res_min = shortest_call(one, resident_ms(c, MANY, 1, e0, e1), MANY, 0.0f, lay);
+}
 
 /* Chooses the cluster size of the resident steps by timing (or takes the cached choice)
  * and leaves the plan on the device; res_on stays false when nothing fits. *step_ms: the
@@ -1001,8 +1085,10 @@ int setup_resident(lb_ctx *c, float *step_ms)
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_res_tune.find(key);
         if (it != g_res_tune.end()) {
-            known = it->second.choice;
+            known = it->second.cluster;
             *step_ms = it->second.step_ms;
+            c->res_min = it->second.min_steps;
+            c->res_alt = it->second.alt;
         }
     }
     if (known == 0) return LB_OK;
@@ -1017,7 +1103,6 @@ int setup_resident(lb_ctx *c, float *step_ms)
         cudaGetLastError();
         return LB_OK;
     }
-    constexpr int STEPS = 24;
     float best = 1e30f;
     int best_c = 0;
     bool planned = false;
@@ -1025,37 +1110,29 @@ int setup_resident(lb_ctx *c, float *step_ms)
         if (!lbk::res_plan_build(one, c->store, c->res_pair, cl, 1, sr, c->rplan)) continue;
         planned = true;
         if (resident_upload(c) != LB_OK) continue;
-        float ms = 1e30f;
-        for (int rep = 0; rep < 2; ++rep) {
-            cudaEventRecord(e0, c->stream);
-            if (resident_steps(c, STEPS, 0) != LB_OK) {
-                c->status = LB_OK;   /* this size cannot be launched here */
-                break;
-            }
-            cudaEventRecord(e1, c->stream);
-            float t = 0.0f;
-            if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess) ms = std::min(ms, t);
-        }
+        const float ms = resident_ms(c, RES_TUNE_STEPS, 0, e0, e1);
         if (ms < 0.97f * best) {
             best = ms;
             best_c = cl;
         }
     }
+    /* its plan again, and what it takes in short calls */
+    int e = LB_OK;
+    if (best_c > 0 && lbk::res_plan_build(one, c->store, c->res_pair, best_c, 1, sr, c->rplan)) {
+        e = resident_start(c);
+        if (c->res_on) tune_short_calls(c, e0, e1);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (int e = launch_check(c, "resident tuning")) return e;
-    if (!planned) {   /* none of this shape fits: not tried again */
-        std::lock_guard<std::mutex> g(g_tune_mu);
-        g_res_tune[key] = {0, 0.0f};
-    }
-    if (best_c == 0 || !lbk::res_plan_build(one, c->store, c->res_pair, best_c, 1, sr, c->rplan)) return LB_OK;
-    {
-        std::lock_guard<std::mutex> g(g_tune_mu);
-        g_res_tune[key] = {best_c, best / STEPS};
-    }
+    if (e) return e;
+    if (int e2 = launch_check(c, "resident tuning")) return e2;
+    std::lock_guard<std::mutex> g(g_tune_mu);
+    if (!planned) g_res_tune[key] = {0, 0.0f, 1, 0};   /* none of this shape fits: not tried again */
+    if (!c->res_on) return LB_OK;
     c->res_cluster = best_c;
-    *step_ms = best / STEPS;
-    return resident_start(c);
+    *step_ms = best / RES_TUNE_STEPS;
+    g_res_tune[key] = {best_c, *step_ms, c->res_min, c->res_alt};
+    return LB_OK;
 }
 
 /* Autotuner: times every step-kernel layout on this lattice (reading the current level,
@@ -1104,21 +1181,11 @@ int autotune_t(lb_ctx *c, float *step_ms)
         if (v == 10 && (c->store == LB_STORE_F16_DEV || c->store == LB_STORE_BF16_DEV) &&
             (long long)c->nx * c->ny < 1250000LL)
             continue;
-        /* with the pressure pass, which layout 10 does inside its kernel where it can */
-        auto one = [&] {
-            launch_variant<R>(c, v, p);
-            if (v != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
-        };
-        for (int k = 0; k < 2; ++k) one();
-        cudaEventRecord(e0, c->stream);
-        for (int k = 0; k < 5; ++k) one();
-        cudaEventRecord(e1, c->stream);
-        float ms = 0.0f;
+        const float ms = layout_ms<R>(c, v, p, e0, e1);
         /* A later layout must win by more than 3 %: closer timings are within the noise of
          * five launches, and a layout that wins alone by that little can lose when several
          * lattices step concurrently. */
-        if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess &&
-            ms < 0.97f * best_ms) {
+        if (ms < 0.97f * best_ms) {
             best_ms = ms;
             best = v;
         }
@@ -1126,7 +1193,7 @@ int autotune_t(lb_ctx *c, float *step_ms)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (cudaGetLastError() != cudaSuccess) return 0;
-    *step_ms = best_ms / 5.0f;
+    *step_ms = best_ms;
     std::lock_guard<std::mutex> g(g_tune_mu);
     g_tune[key] = {best, *step_ms};
     return best;
@@ -1160,7 +1227,7 @@ int choose_steps(lb_ctx *c)
     if (c->res_on && lay_ms > 0.0f && lay_ms < res_ms) {
         c->res_on = false;
         std::lock_guard<std::mutex> g(g_tune_mu);
-        g_res_tune[c->res_key] = {0, 0.0f};   /* its kind takes the layouts from now on */
+        g_res_tune[c->res_key] = {0, 0.0f, 1, 0};   /* its kind takes the layouts from now on */
     } else if (c->res_on) {
         c->variant = c->res_pair ? 9 : 0;
         c->res_variant = true;
@@ -1268,22 +1335,25 @@ int step_t(lb_ctx *c, int64_t n)
             if (c->opts.reduce_every > 0) m = std::min<int64_t>(m, c->opts.reduce_every - c->step % c->opts.reduce_every);
             if (c->mlp && c->mlp_every > 0) m = std::min<int64_t>(m, c->mlp_every - c->step % c->mlp_every);
             if (c->walls[0].omega > 0.0 || c->walls[1].omega > 0.0) m = std::min<int64_t>(m, lbk::RES_OSC);
-            if (int e = resident_steps_t<R>(c, (int)m, 1)) return e;
-            c->cur ^= (int)(m & 1);
-            for (int64_t i = 0; i < m; ++i) c->t += c->dt;
-            c->step += m;
-            k += m - 1;
-            if (int e = after_step<R>(c)) return e;
-            continue;
+            if (m >= c->res_min) {
+                if (int e = resident_steps_t<R>(c, (int)m, 1)) return e;
+                c->cur ^= (int)(m & 1);
+                for (int64_t i = 0; i < m; ++i) c->t += c->dt;
+                c->step += m;
+                k += m - 1;
+                if (int e = after_step<R>(c)) return e;
+                continue;
+            }
         }
+        const int v = c->res_variant ? c->res_alt : c->variant;
         const double t_new = c->t + c->dt;
         StepParams<R> p = make_params<R>(c, c->cur, c->cur ^ 1, t_new);
         if (c->opts.scheme == LB_SCHEME_STREAM) {
             lbk::launch_exact_stream<R>(c->store, p, c->stream);
         } else {
-            launch_variant<R>(c, c->variant, p);
+            launch_variant<R>(c, v, p);
             lbk::launch_iface<R>(c->store, p, c->stream);
-            if (c->variant != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
+            if (v != 10 || !pressure_in_step(p)) lbk::launch_pressure<R>(c->store, p, c->stream);
         }
         if (int e = launch_check(c, "step")) return e;
         c->cur ^= 1;
@@ -1864,7 +1934,7 @@ bool resident_plan(lb_ctx *c, int cluster)
 
 /* After a map change of a lattice on the resident steps: the plan of the new map, with the
  * cluster size that was timed fastest where that fits. Where the new map has none, the steps go
- * one launch each on the layout that lb_info names all along, which has the same bits; nothing
+ * one launch each on the layout that short calls take (res_alt), which has the same bits; nothing
  * is timed inside a run, and a later map may take the resident steps again. */
 int replan(lb_ctx *c)
 {
@@ -1916,8 +1986,9 @@ int lbi_resident_cluster(lb_ctx *c, int cluster)
     if (cluster > 0) {
         if (!resident_plan(c, cluster) || resident_start(c) != LB_OK || !c->res_on) return -1;
         c->res_cluster = cluster;
+        c->res_min = 1;
+        c->res_alt = c->variant = c->res_pair ? 9 : 0;
         c->res_variant = true;
-        c->variant = c->res_pair ? 9 : 0;
     }
     return c->res_on ? c->rplan.cluster : 0;
 }

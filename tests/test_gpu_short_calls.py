@@ -1,0 +1,92 @@
+"""Calls of one or a few steps on lattices of the resident steps: where a resident launch does not
+pay, the steps go one launch each on a layout of the same bits, and cost what that costs. Long and
+short calls in any order, with in-step reductions, a reload and a map change between them, have the
+bits of one launch per step throughout."""
+import numpy as np
+import pytest
+
+from lbinputs import band_map, couette
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(128, 128, 12, "f32_dev"), (96, 90, 9, "f32"), (128, 300, 24, "bf16_dev"), (100, 100, 10, "f16_dev"), (64, 140, 14, "f64")]
+
+
+def _make(nx, ny, rows, store, **kw):
+    import paper_1007_4895_gb300 as lb
+    w = couette(nx=nx, ny=ny, rows=rows)
+    x, y = 2 * np.pi * np.arange(nx)[None, :] / nx, np.pi * np.arange(ny)[:, None] / ny
+    w.init = (1.0 + 0.02 * np.sin(x) * np.cos(y), 0.03 * np.cos(x) * np.sin(y), 0.02 * np.sin(x) * np.cos(2 * y))
+    w.cfl = 0.38
+    return lb.Lattice.from_workload(w, store=store, **kw)
+
+
+@pytest.mark.parametrize("rounding", ["nearest", "stochastic"])
+@pytest.mark.parametrize("nx,ny,rows,store", SIZES)
+def test_long_and_short_calls_have_the_same_bits(nx, ny, rows, store, rounding):
+    import paper_1007_4895_gb300 as lb
+    named = 9 if store in ("f32", "f32_dev") else 0
+    a = _make(nx, ny, rows, store, rounding=rounding)
+    b = _make(nx, ny, rows, store, rounding=rounding, variant=named)
+    if a.info()["variant"] != named:
+        pytest.skip("the layouts were faster here")
+
+    def same(what):
+        eff = b.effective_map()
+        for s in (0, 1):
+            assert np.array_equal(a.populations(s)[:, eff == s], b.populations(s)[:, eff == s]), (what, s)
+
+    def step(*calls):
+        for n in calls:
+            a.step(n)
+            b.step(n)
+    step(1, 1, 40, 2, 3, 30, 1, 7, 1)
+    same("calls")
+    n = a.state_bytes()
+    buf = np.zeros(n, np.uint8)
+    lb.lb_state_store(a.ctx, buf.ctypes.data, n)
+    for lat in (a, b):
+        lb.lb_state_load(lat.ctx, buf.ctypes.data, n)
+    step(1, 25, 1)
+    same("reload")
+    for lat in (a, b):
+        lat.set_region_map(band_map(nx, ny, rows + 2, rows - 1))
+    step(1, 1, 30, 2)
+    same("map")
+    assert a.info()["step"] == b.info()["step"] and a.reductions() == b.reductions()
+    a.close()
+    b.close()
+
+
+def test_in_step_reductions_at_every_step():
+    a = _make(128, 128, 12, "f32_dev", reduce_every=1)
+    b = _make(128, 128, 12, "f32_dev", reduce_every=1, variant=9)
+    a.step(13)
+    b.step(13)
+    assert a.reductions() == b.reductions()
+    for s in (0, 1):
+        assert np.array_equal(a.populations(s), b.populations(s))
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("nx,ny,rows,store", [(128, 128, 12, "f32_dev"), (128, 300, 24, "bf16_dev")])
+def test_single_steps_cost_no_more_than_on_the_layout_named(nx, ny, rows, store):
+    """A resident launch of one step took 90 and 154 us here, the layouts 30 and 43."""
+    import torch
+    took = []
+    for variant in (-1, 9 if store == "f32_dev" else 0):
+        lat = _make(nx, ny, rows, store, variant=variant)
+        best = 1e9
+        for _ in range(5):
+            lat.step(1)
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(50):
+                lat.step(1)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        took.append(best)
+        lat.close()
+    assert took[0] <= 1.25 * took[1], took
