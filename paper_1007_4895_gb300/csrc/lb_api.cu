@@ -2205,6 +2205,9 @@ struct lb_batch {
     size_t plan_cap = 0, off_cap = 0, items_cap = 0;
     int nsm = 0;
     int quad_threads = 0, quad_grid = 0;   /* block shape of the one-quad kernel, once timed */
+    int ring_grid = 1;
+    int64_t res_min = 1;            /* steps a launch on the resident steps must have to pay (ring
+                                     * batches: 4 until timed) */
     uint64_t maps_seen = 0;         /* the members' map_count that the plan or the items are of */
     int status = LB_OK;
     std::vector<void *> owned;
@@ -2376,8 +2379,11 @@ int batch_ring_setup(lb_batch *b)
     if (lbk::launch_ring_batch(b->store, b->q1, nullptr, nullptr, nullptr, nullptr, nullptr, b->n, 0, 0, 0, nullptr,
                                b->force, 0, &resident, b->stream) != 0 || resident < 1)
         return fail(LB_ERR_CUDA, "the batch kernel cannot be resident");
-    b->threads = 256;   /* the block the kernel is built for */
-    b->grid = std::min(b->n, resident);
+    b->ring_grid = std::min(b->n, resident);
+    if (!b->resident) {
+        b->threads = 256;   /* the block the kernel is built for */
+        b->grid = b->ring_grid;
+    }
     return LB_OK;
 }
 
@@ -2415,7 +2421,7 @@ int batch_resident_setup(lb_batch *b)
 
 int batch_launch(lb_batch *b, int64_t nsteps, int advance, cudaStream_t st)
 {
-    if (b->resident) {
+    if (b->resident && nsteps >= b->res_min) {
         const lbk::ResOsc<double> none{};   /* steady walls: only the count is read */
         static_assert(offsetof(lbk::ResOsc<double>, n) == 0 && offsetof(lbk::ResOsc<float>, n) == 0, "the count comes first");
         if (lbk::launch_resident(b->store, b->res_pair, b->force, b->plan, b->d_plan, b->d_off, b->d_params, b->d_tabs,
@@ -2430,7 +2436,7 @@ int batch_launch(lb_batch *b, int64_t nsteps, int advance, cudaStream_t st)
         return fail(LB_ERR_CUDA, "batch queue reset failed");
     const int r = b->ring ? lbk::launch_ring_batch(b->store, b->q1, static_cast<const StepParams<float> *>(b->d_params),
                                                    b->d_tabs, b->d_items, b->d_ranges, b->d_order, b->n, (int)nsteps,
-                                                   b->phase, advance, b->d_queue, b->force, b->grid, nullptr, st)
+                                                   b->phase, advance, b->d_queue, b->force, b->ring_grid, nullptr, st)
                           : lbk::launch_batch(b->store, b->d_params, b->d_order, b->n, (int)nsteps, b->phase, advance,
                                               b->d_queue, b->threads, b->grid, st);
     if (r != 0)
@@ -2493,6 +2499,44 @@ int batch_quad_setup(lb_batch *b)
     return LB_OK;
 }
 
+/* How many steps a launch on the resident steps must have to pay against layout 10's bodies,
+ * which load no more than a step needs (512 channels, FP32 deviations: 273 us a call of one step
+ * and 43 a further one, against 170 and 105; 64 channels 136 and 28, against 57 and 37): both
+ * timed without moving the state, a resident launch of an odd number of steps with its
+ * write-back into the other level. At creation only: a run times nothing. */
+int batch_time_calls(lb_batch *b)
+{
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
+        cudaGetLastError();
+        if (e0) cudaEventDestroy(e0);
+        return LB_OK;
+    }
+    int e = LB_OK;
+    auto ms = [&](int64_t from, int n, int advance) {
+        b->res_min = from;
+        float best = 1e30f;
+        for (int rep = 0; rep < 3 && !e; ++rep) {
+            cudaEventRecord(e0, b->stream);
+            e = batch_launch(b, n, advance, b->stream);
+            cudaEventRecord(e1, b->stream);
+            float t = 0.0f;
+            if (!e && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess)
+                best = std::min(best, t);
+        }
+        return best;
+    };
+    constexpr int MANY = 25, FEW = 5;
+    const float r1 = ms(INT64_MAX, 1, 0), rn = ms(INT64_MAX, FEW, 0), s1 = ms(1, 1, 1), sn = ms(1, MANY, 1);
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    b->res_min = 1;
+    if (e) return e;
+    const float step = (rn - r1) / (FEW - 1);
+    b->res_min = shortest_call(s1, sn, MANY, r1 - step, step);
+    return LB_OK;
+}
+
 uint64_t batch_maps(const lb_batch *b)
 {
     uint64_t k = 0;
@@ -2503,7 +2547,9 @@ uint64_t batch_maps(const lb_batch *b)
 /* What follows from the members' region maps: the queue order, and the kernel with its plan
  * or items. The resident steps where every lattice fits a block's shared memory (the bits of
  * the other two kernels): layout 9's arithmetic for the ring batch's lattices, layout 0's for
- * FP64; else layout 10's bodies, or the one-quad kernel, which reads the maps itself. */
+ * FP64; else, and for calls of a few steps, layout 10's bodies, or the one-quad kernel, which
+ * reads the maps itself (FP64 on the resident steps: in calls of every length, a chain of 36
+ * populations alone takes the one-quad kernel 220 us). */
 int batch_plan(lb_batch *b)
 {
     /* most work first */
@@ -2527,20 +2573,10 @@ int batch_plan(lb_batch *b)
     b->resident = false;
     if (b->ring || b->store == LB_STORE_F64)
         if (int e = batch_resident_setup(b)) return e;
-    if (b->ring && !b->resident)
+    if (b->ring)
         if (int e = batch_ring_setup(b)) return e;
     if (!b->ring && !b->resident)
         if (int e = batch_quad_setup(b)) return e;
-    /* the ring batch reads carried moments: a batch that comes to it from the resident steps,
-     * which keep none, has them summed */
-    for (lb_ctx *c : b->inst) {
-        const bool carry = b->ring && !b->resident;
-        if (carry && !c->ring_batch) {
-            lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), c->stream);
-            if (int e = launch_check(c, "carried moments")) return e;
-        }
-        c->ring_batch = carry;
-    }
     b->maps_seen = batch_maps(b);
     return LB_OK;
 }
@@ -2595,6 +2631,7 @@ int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps,
         b->force = b->force || opts[i].gx != 0.0 || opts[i].gy != 0.0;
     }
     b->q1 = sets[1];
+    b->res_min = b->ring ? 4 : 1;
     for (int i = 0; i < n; ++i) {
         lb_opts o = opts[i];
         /* no per-lattice timing: the batch kernel does the stepping, with the bits of
@@ -2621,6 +2658,7 @@ int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps,
         e = fail(LB_ERR_CUDA, "device query failed");
     b->res_pair = b->ring;
     if (!e) e = batch_plan(b);
+    if (!e && b->resident && b->ring) e = batch_time_calls(b);
     if (e) {
         batch_release(b);
         delete b;
@@ -2649,7 +2687,7 @@ int lb_batch_step_each(lb_batch *b, int64_t nsteps)
             if (int e = lb_step(c, 1)) return e;
     b->phase ^= (int)(nsteps & 1);
     /* layout 9 carries no moments: the ring batch's are summed again */
-    if (b->ring && !b->resident && nsteps > 0)
+    if (b->ring && nsteps > 0)
         for (lb_ctx *c : b->inst) {
             lbk::launch_aux<float>(c->store, make_params<float>(c, c->cur, c->cur, c->t), c->stream);
             if (int e = launch_check(c, "carried moments")) return e;

@@ -90,3 +90,48 @@ def test_single_steps_cost_no_more_than_on_the_layout_named(nx, ny, rows, store)
         took.append(best)
         lat.close()
     assert took[0] <= 1.25 * took[1], took
+
+
+@pytest.mark.parametrize("n,store", [(24, "f32_dev"), (24, "bf16_dev"), (9, "f32"), (9, "f64")])
+def test_batches_in_long_and_short_calls(n, store):
+    import paper_1007_4895_gb300 as lb
+    from lbinputs import batched_instances
+    b = lb.Batch(batched_instances(n=n, seed=11), store=store)
+    b.step_each(1)
+    for k in (1, 1, 30, 2, 1, 3, 26, 1):
+        b.step(k)
+    b.graph(2, replays=3)
+    b.step(1)
+    b.step_each(1)
+    b.step(20)
+    for i in (0, n // 2, n - 1):
+        alone = lb.Lattice.from_workload(batched_instances(n=n, seed=11)[i], store=store, variant=0 if store == "f64" else 9)
+        alone.step(1 + 65 + 6 + 1 + 1 + 20)
+        for s in (0, 1):
+            assert np.array_equal(b.lattice(i).populations(s), alone.populations(s)), (i, s)
+        alone.close()
+    b.close()
+
+
+def test_single_batch_steps_cost_about_a_step():
+    """64 channels: a launch of one resident step took 136 us and one of four 204; on layout 10's
+    bodies one step takes 57."""
+    import torch
+    import paper_1007_4895_gb300 as lb
+    from lbinputs import batched_instances
+    b = lb.Batch(batched_instances(n=64, seed=7), store="f32_dev")
+    took = {}
+    for k in (1, 4):
+        best = 1e9
+        for _ in range(5):
+            b.step(k)
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(30):
+                b.step(k)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        took[k] = best
+    b.close()
+    assert took[1] <= 0.45 * took[4], took
