@@ -192,8 +192,8 @@ enum { LB_ROUND_NEAREST = 0, LB_ROUND_STOCHASTIC = 1 };
  * lattice whose density varies along x (a pressure-driven channel) keeps small stored
  * magnitudes and loses less to 16-bit rounding. The arithmetic and its results in FP32
  * are those of one reference density; only the rounding of the stored values changes.
- * Values must be finite and positive; the array is copied at create. Layouts 0 and 5
- * support it (a forced other layout falls back to 0); batched lattices do not. The
+ * Values must be finite and positive; the array is copied at create. Layouts 0, 5 and 7 to
+ * 10 support it (a forced other layout falls back to 0); batched lattices do not. The
  * compact state (lb_state_*, checkpoints) holds the shifted values, so it belongs to a
  * lattice with the same reference densities. */
 

@@ -438,9 +438,13 @@ void launch_pack_t(lb_ctx *c, int unpack)
  * the copies' latency, which is what a lattice in L2 is bound by; the rows need no warp to
  * keep step with others, which wins once DRAM is. Us a step, rows / tiles: 1200 x 90 pressure
  * channel 82 / 41 (16-bit 91 / 41), 1024 x 512 Poiseuille 46.8 / 41.9 (57.7 / 45.4), 16384 x
- * 128 channel, whose two levels are larger than L2, 97 / 120 (92 / 134). */
+ * 128 channel, whose two levels are larger than L2, 97 / 120 (92 / 134). Smaller lattices with a
+ * reference density per column have the rows, unless layout 10 is asked for: on tiles it would
+ * be the choice there too (512 x 64 channel 45 / 34, layout 0 50), but the layouts of those
+ * lattices, 0 and 5 at ragged widths, are relied upon. */
 bool tiles_pay(const lb_ctx *c)
 {
+    if (c->d_dcol && c->opts.variant < 0 && (long long)c->nx * c->ny < 1250000LL) return false;
     size_t pops = 0;
     for (size_t k = 0; k < c->tmap.size(); ++k) pops += (size_t)c->q[c->tmap[k] & LB_TILE_HIGH] * LB_TILE_X;
     return 2 * pops * c->esize <= (size_t)100 << 20;
@@ -896,8 +900,8 @@ uint64_t resident_group(const lb_ctx *c, bool pair)
 
 /* The two launch parameter sets, the constants, the plan and its offsets on the device: one
  * allocation (grown as needed) and one copy, in stream order; pageable memory is taken over
- * before the copy call returns, so nothing waits (a copy each and a wait made a second lattice
- * of a shape 0.424 ms to create against 0.407 without resident steps) */
+ * before the copy call returns, so nothing waits (an 8 x 64 channel in FP32 deviations of a known
+ * shape: 427 us to create with a copy each and a wait, 407 so, 380 without resident steps) */
 template <typename R>
 int resident_upload_t(lb_ctx *c)
 {
