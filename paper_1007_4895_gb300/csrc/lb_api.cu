@@ -157,7 +157,7 @@ struct lb_ctx {
     lb_mlp *mlp = nullptr;
     int mlp_every = 0;
     float p_on = 0.5f, p_off = 0.3f;
-    float *d_mom = nullptr, *d_feat = nullptr, *d_p = nullptr, *d_tp = nullptr;
+    float *d_rho = nullptr, *d_feat = nullptr, *d_p = nullptr, *d_tp = nullptr;
     int64_t map_updates = 0, map_fallbacks = 0;
     std::vector<void *> owned;
 };
@@ -1244,11 +1244,11 @@ int ensure_learned_buffers(lb_ctx *c)
     const size_t N = (size_t)c->nx * c->ny;
     /* each buffer on its own, so a failed allocation is retried by the next call (what
      * did succeed stays owned by the context) */
-    if (!c->d_mom) c->d_mom = static_cast<float *>(own(c, N * sizeof(float)));
+    if (!c->d_rho) c->d_rho = static_cast<float *>(own(c, N * sizeof(float)));
     if (!c->d_feat) c->d_feat = static_cast<float *>(own(c, 8 * N * sizeof(float)));
     if (!c->d_p) c->d_p = static_cast<float *>(own(c, N * sizeof(float)));
     if (!c->d_tp) c->d_tp = static_cast<float *>(own(c, (size_t)c->ny * c->ntx * sizeof(float)));
-    if (!c->d_mom || !c->d_feat || !c->d_p || !c->d_tp) return fail(LB_ERR_NOMEM, "device allocation failed");
+    if (!c->d_rho || !c->d_feat || !c->d_p || !c->d_tp) return fail(LB_ERR_NOMEM, "device allocation failed");
     return LB_OK;
 }
 
@@ -1256,7 +1256,7 @@ template <typename R>
 int features_t(lb_ctx *c, float *dst)
 {
     StepParams<R> p = make_params<R>(c, c->cur, c->cur, c->t);
-    lbk::launch_features<R>(c->store, p, c->d_mom, dst, c->stream);
+    lbk::launch_features<R>(c->store, p, c->d_rho, dst, c->stream);
     return launch_check(c, "features");
 }
 

@@ -21,9 +21,10 @@
  * carried moments of a wall row are summed over its final values in order).
  *
  * The arithmetic is layout 9's, operation for operation: the same bits. Two blocks of 256
- * threads per SM, so that one block's epilogue does not leave the SM idle, at 128 registers:
- * with an eighth consumer warp (96 registers) the loop spilled, and with shared memory
- * taking all but 28 KB of L1 each reload went to L2 (1350 cycles a population). Measured
+ * threads per SM, so that one block's epilogue does not leave the SM idle, at 128 registers
+ * (FP32 and BF16 still spill 4 to 64 bytes, FP16 none): with an eighth consumer warp (96
+ * registers) the loop itself spilled, and with shared memory taking all but 28 KB of L1 each
+ * reload went to L2 (1350 cycles a population). Measured
  * (FP32 deviations, us a step, rows of lb_ring2.cuh / tiles): 1024 x 512 Poiseuille 46.8 /
  * 41.9, 1200 x 90 pressure channel 82 / 41; 16384 x 128, whose levels do not fit L2, 97 / 120:
  * the host picks by that (tiles_pay in lb_api.cu).
@@ -330,9 +331,10 @@ __device__ __forceinline__ bool tile_row(const StepParams<float> &p, const RingT
             copies(dst - col, e);
         }
     };
-    /* rolled, with one body per sign of xi_x (one in all for the few general rows): the code of
-     * every kind of row stays in the instruction cache (unrolled over the abscissae the kernel
-     * waited on instructions more than on memory), and the loop in its registers */
+    /* D2Q9: nine bodies, each of its abscissae; larger sets: the abscissae of xi_x unrolled (four
+     * or six bodies, signs and strides at compile time), rolled over those of xi_y; the few
+     * general rows one body, rolled. Instructions are what the kernel waits for most after its
+     * stages (2.5 cycles per issue on the 16384 x 128 channel). */
     if constexpr (GEN) {
 #pragma unroll 1
         for (int a = 0; a < Q; ++a) {
