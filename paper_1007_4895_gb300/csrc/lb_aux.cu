@@ -149,14 +149,23 @@ __global__ void get_pops_kernel(const __grid_constant__ StepParams<typename Stor
     }
 }
 
-/* Two neighbouring nodes' values of the arithmetic type: packed two-wide instructions for
- * FP32 */
+/* The nodes of a thread in the moment fields: two neighbours in FP32, in packed two-wide
+ * instructions; one in FP64, where a second only lengthens the chain on the FP64 units (4 x 32
+ * lattice 43 us with one node per thread, 74 with two; 1024 x 512 416 and 455) */
 template <typename R>
 struct Two {
     R x, y;
 };
+template <>
+struct Two<double> {
+    double x;
+};
 template <typename R>
-__device__ __forceinline__ Two<R> two(R v) { return {v, v}; }
+constexpr int nodes_of = sizeof(R) == 4 ? 2 : 1;
+__device__ __forceinline__ Two<float> two(float v) { return {v, v}; }
+__device__ __forceinline__ Two<double> two(double v) { return {v}; }
+__device__ __forceinline__ float node_of(const Two<float> &a, int k) { return k ? a.y : a.x; }
+__device__ __forceinline__ double node_of(const Two<double> &a, int) { return a.x; }
 __device__ __forceinline__ Two<float> fma_t(Two<float> a, Two<float> b, Two<float> c)
 {
     const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
@@ -170,7 +179,7 @@ __device__ __forceinline__ Two<float> mul_t(Two<float> a, Two<float> b)
 /* a product that is added to: scalar, because a packed multiply and a packed add are fused
  * into one rounding whatever the contraction setting */
 __device__ __forceinline__ Two<float> mul_s(Two<float> a, Two<float> b) { return {__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)}; }
-__device__ __forceinline__ Two<double> mul_s(Two<double> a, Two<double> b) { return {a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ Two<double> mul_s(Two<double> a, Two<double> b) { return {a.x * b.x}; }
 __device__ __forceinline__ Two<float> add_t(Two<float> a, Two<float> b)
 {
     const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
@@ -178,14 +187,16 @@ __device__ __forceinline__ Two<float> add_t(Two<float> a, Two<float> b)
 }
 __device__ __forceinline__ Two<double> fma_t(Two<double> a, Two<double> b, Two<double> c)
 {
-    return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+    return {fma(a.x, b.x, c.x)};
 }
-__device__ __forceinline__ Two<double> mul_t(Two<double> a, Two<double> b) { return {a.x * b.x, a.y * b.y}; }
-__device__ __forceinline__ Two<double> add_t(Two<double> a, Two<double> b) { return {a.x + b.x, a.y + b.y}; }
-template <typename R>
-__device__ __forceinline__ Two<R> neg_t(Two<R> a) { return {-a.x, -a.y}; }
+__device__ __forceinline__ Two<double> mul_t(Two<double> a, Two<double> b) { return {a.x * b.x}; }
+__device__ __forceinline__ Two<double> add_t(Two<double> a, Two<double> b) { return {a.x + b.x}; }
+__device__ __forceinline__ Two<float> neg_t(Two<float> a) { return {-a.x, -a.y}; }
+__device__ __forceinline__ Two<double> neg_t(Two<double> a) { return {-a.x}; }
+__device__ __forceinline__ Two<float> div_t(Two<float> a, Two<float> b) { return {a.x / b.x, a.y / b.y}; }
+__device__ __forceinline__ Two<double> div_t(Two<double> a, Two<double> b) { return {a.x / b.x}; }
 
-/* Moment fields of two neighbouring nodes of a set of Q populations: rho, u, P_xy = sum f
+/* Moment fields of a thread's nodes of a set of Q populations: rho, u, P_xy = sum f
  * (xi-u)_x (xi-u)_y, Pi^neq = sum (f - f_eq) xi xi, q = (1/2) sum f |xi - u|^2 (xi - u).
  * The rest-state part w rho0 is summed in closed form (Gaussian moments up to third order,
  * exact for every set), so only deviations enter the sums. The number of populations is a
@@ -207,9 +218,13 @@ __device__ __forceinline__ void node_fields(const StepParams<typename Store<ST>:
     W d[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
-        T raw[2];
-        ld2(f + a * plane, raw);
-        d[a] = W{dec_at<ST>(p, raw[0], c.winv[a], x + LB_GHOST), dec_at<ST>(p, raw[1], c.winv[a], x + 1 + LB_GHOST)};
+        if constexpr (nodes_of<R> == 2) {
+            T raw[2];
+            ld2(f + a * plane, raw);
+            d[a] = W{dec_at<ST>(p, raw[0], c.winv[a], x + LB_GHOST), dec_at<ST>(p, raw[1], c.winv[a], x + 1 + LB_GHOST)};
+        } else {
+            d[a] = W{dec_at<ST>(p, f[a * plane], c.winv[a], x + LB_GHOST)};
+        }
     }
     W rd = two(R(0)), jx = rd, jy = rd;
 #pragma unroll
@@ -219,7 +234,7 @@ __device__ __forceinline__ void node_fields(const StepParams<typename Store<ST>:
         jy = fma_t(two(c.wcy[a]), d[a], jy);
     }
     const W rho = add_t(two(rho0), rd);
-    const W ux = {jx.x / rho.x, jx.y / rho.y}, uy = {jy.x / rho.x, jy.y / rho.y};
+    const W ux = div_t(jx, rho), uy = div_t(jy, rho);
     const W usq = add_t(mul_s(ux, ux), mul_s(uy, uy)), nusq = neg_t(usq);
     /* rest-state parts: sum w (xi-u)_x (xi-u)_y = ux uy; sum w |xi-u|^2 (xi-u)_x = -ux (4 + u^2) */
     W pxy = mul_t(mul_t(two(rho0), ux), uy), nxx = two(R(0)), nxy = nxx, nyy = nxx;
@@ -254,8 +269,8 @@ __device__ __forceinline__ void node_fields(const StepParams<typename Store<ST>:
     vals[8] = qy;
 }
 
-/* node_fields by the set of the nodes x, x + 1 (a warp lies in one tile: no divergence; a
- * pair never spans two) */
+/* node_fields by the set of the node x (and x + 1: a warp lies in one tile, and a pair never
+ * spans two) */
 template <int ST>
 __device__ __forceinline__ void node_fields_any(const StepParams<typename Store<ST>::R> &p, int x, int j,
                                                 Two<typename Store<ST>::R> (&vals)[9])
@@ -276,24 +291,27 @@ __device__ __forceinline__ void node_fields_any(const StepParams<typename Store<
     }
 }
 
-/* a block is one 128-column tile: 64 threads of two nodes */
+/* a block is one 128-column tile: 64 threads of two nodes, or 128 of one */
+template <int ST>
+constexpr int field_threads = 128 / nodes_of<typename Store<ST>::R>;
 template <int ST, typename OUT>
-__global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) moments_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p,
+__global__ void __launch_bounds__(field_threads<ST>, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) moments_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p,
                                                      uint32_t mask, OUT *dst)
 {
     using R = typename Store<ST>::R;
-    const int x = 2 * (blockIdx.x * 64 + threadIdx.x), j = blockIdx.y;
+    constexpr int NV = nodes_of<R>;
+    const int x = NV * (blockIdx.x * field_threads<ST> + threadIdx.x), j = blockIdx.y;
     if (x >= p.nx) return;
     Two<R> vals[9];
     node_fields_any<ST>(p, x, j, vals);
     const size_t N = (size_t)p.nx * p.ny, n = (size_t)j * p.nx + x;
-    const bool both = x + 1 < p.nx;
+    const bool both = NV == 2 && x + 1 < p.nx;
     const bool vec = both && (p.nx & 1) == 0 && (reinterpret_cast<uintptr_t>(dst) & (2 * sizeof(OUT) - 1)) == 0;
     OUT *o = dst + n;
 #pragma unroll
     for (int m = 0; m < 9; ++m)
         if (mask & (1u << m)) {
-            const OUT e[2] = {OUT(vals[m].x), OUT(vals[m].y)};
+            const OUT e[2] = {OUT(node_of(vals[m], 0)), OUT(node_of(vals[m], 1))};
             if (vec) {
                 st2(o, e);
             } else {
@@ -398,11 +416,12 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Ste
  * densities (all nine moment fields went through memory before: 105 us -> 64 us on
  * 2 097 152 nodes). */
 template <int ST>
-__global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) features_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p, float h,
+__global__ void __launch_bounds__(field_threads<ST>, sizeof(typename Store<ST>::R) == 4 ? 8 : 1) features_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p, float h,
                                                       float *__restrict__ rho_out, float *__restrict__ out)
 {
     using R = typename Store<ST>::R;
-    const int x = 2 * (blockIdx.x * 64 + threadIdx.x), j = blockIdx.y;
+    constexpr int NV = nodes_of<R>;
+    const int x = NV * (blockIdx.x * field_threads<ST> + threadIdx.x), j = blockIdx.y;
     if (x >= p.nx) return;
     Two<R> v[9];
     node_fields_any<ST>(p, x, j, v);
@@ -414,8 +433,8 @@ __global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1
     }
     float e[8][2];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        auto val = [&](int m) { return (float)(k ? v[m].y : v[m].x); };
+    for (int k = 0; k < NV; ++k) {
+        auto val = [&](int m) { return (float)node_of(v[m], k); };
         const float rho = val(0), inv = 1.0f / rho;
         e[0][k] = val(4) * inv;
         e[1][k] = val(5) * inv;
@@ -426,7 +445,7 @@ __global__ void __launch_bounds__(64, sizeof(typename Store<ST>::R) == 4 ? 8 : 1
         e[6][k] = p.tau_const ? (float)p.kn_rho : (float)p.kn_rho / rho;
         e[7][k] = rho;
     }
-    const bool both = x + 1 < p.nx;
+    const bool both = NV == 2 && x + 1 < p.nx;
     const bool vec = both && (p.nx & 1) == 0 && ((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(rho_out)) & 7) == 0;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
@@ -574,10 +593,10 @@ void launch_moments(int store, const StepParams<R> &p, uint32_t mask, void *dst,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (dst_f64) {
         LB_DISPATCH(store, if constexpr (store_matches<R, ST>())
-                               moments_kernel<ST, double><<<grid, 64, 0, st>>>(p, mask, static_cast<double *>(dst)));
+                               moments_kernel<ST, double><<<grid, field_threads<ST>, 0, st>>>(p, mask, static_cast<double *>(dst)));
     } else {
         LB_DISPATCH(store, if constexpr (store_matches<R, ST>())
-                               moments_kernel<ST, float><<<grid, 64, 0, st>>>(p, mask, static_cast<float *>(dst)));
+                               moments_kernel<ST, float><<<grid, field_threads<ST>, 0, st>>>(p, mask, static_cast<float *>(dst)));
     }
 }
 
@@ -586,7 +605,7 @@ void launch_features(int store, const StepParams<R> &p, float *rho, float *out, 
 {
     dim3 grid((p.nx + 127) / 128, p.ny);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LB_DISPATCH(store, if constexpr (store_matches<R, ST>()) features_kernel<ST><<<grid, 64, 0, st>>>(p, (float)p.h_grid, rho, out));
+    LB_DISPATCH(store, if constexpr (store_matches<R, ST>()) features_kernel<ST><<<grid, field_threads<ST>, 0, st>>>(p, (float)p.h_grid, rho, out));
     gradient_feature_kernel<R><<<grid, 128, 0, st>>>(p, (float)p.h_grid, rho, out);
 }
 
