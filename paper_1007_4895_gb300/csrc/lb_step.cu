@@ -139,20 +139,21 @@ __global__ void shadows_kernel(const __grid_constant__ StepParams<typename Store
  *
  * Odd steps walk the rows from the top: the rows a step wrote last are still in L2 (129
  * MB) when the next step reads them first, which saves DRAM traffic once the two levels do
- * not fit. */
+ * not fit (the kernel of two nodes per thread; in FP64, bound by its units, it gained nothing:
+ * 2048 x 1024 758.4 and 757.7 us). */
 template <typename R>
 __device__ __forceinline__ int stream_row(const StepParams<R> &p)
 {
     return (p.step_key & 1u) ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y;
 }
 
-/* FP64: one thread per node. */
+/* One thread per node: FP64, and boxes of STREAM_ONE nodes at most. */
 template <int ST>
 __global__ void __launch_bounds__(128) exact_stream_kernel(const __grid_constant__ StepParams<typename Store<ST>::R> p)
 {
     using T = typename Store<ST>::T;
     using R = typename Store<ST>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, j = stream_row(p);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (x >= p.nx) return;
     /* the population loops are unrolled, so the set's constants are read from the
      * parameter block at fixed offsets; population a = 3 iy + ix over ascending
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(128) exact_stream_kernel(const __grid_constant
     }
 }
 
-/* FP32 and 16-bit storage: two neighbouring nodes per thread in packed two-wide FP32
+/* FP32 and 16-bit storage, larger boxes: two neighbouring nodes per thread in packed two-wide FP32
  * arithmetic, the same operations per node as above (the terms whose abscissa is zero
  * left out: they add exact zeros), so the same values. One node per thread was bound by
  * instruction issue (480 a node, 84 % of the issue slots: 64-bit addresses and scalar
@@ -450,12 +451,19 @@ void launch_pair(int store, const StepParams<float> &p, void *stream)
     }
 }
 
+/* One node per thread up to here: a small box is bound by the chain of one thread, which two
+ * nodes lengthen (us a step, FP32 deviations, two nodes / one: 64 x 16 6.2 / 4.2, 128 x 128 6.2 /
+ * 5.0, 513 x 257 6.8 / 6.2, 512 x 512 8.2 / 8.3, 1024 x 512 10.3 / 12.4); the same bits. */
+constexpr long long STREAM_ONE = 1 << 18;
 template <typename R>
 void launch_exact_stream(int store, const StepParams<R> &p, void *stream)
 {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const dim3 one((p.nx + 127) / 128, p.ny);
     if constexpr (std::is_same<R, double>::value) {
-        exact_stream_kernel<0><<<dim3((p.nx + 127) / 128, p.ny), 128, 0, st>>>(p);
+        exact_stream_kernel<0><<<one, 128, 0, st>>>(p);
+    } else if ((long long)p.nx * p.ny <= STREAM_ONE) {
+        LB_DISPATCH(store, if constexpr (store_matches<R, ST>()) exact_stream_kernel<ST><<<one, 128, 0, st>>>(p));
     } else {
         const dim3 grid((p.nx + 255) / 256, p.ny);
         LB_DISPATCH(store, if constexpr (store_matches<R, ST>()) {
