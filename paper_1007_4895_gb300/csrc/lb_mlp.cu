@@ -445,7 +445,7 @@ __global__ void to_bf16_kernel(const float *th, __nv_bfloat16 *wb)
 
 /* Inference on the tensor cores: mma.sync m16n8k16 with BF16 operands and FP32
  * accumulation. A warp takes 32 nodes at a time as two 16-node tiles (two independent
- * chains, one read of the weight fragments). Layer 1 is the 16 x 16 (8 features,
+ * chains, one read of the weight fragments), or, of few nodes, one tile. Layer 1 is the 16 x 16 (8 features,
  * zero-padded) by 16 x 64 product; its GELU outputs are rounded to BF16 and, because
  * the accumulator fragment of two neighbouring 8-column output tiles has exactly the
  * element layout of one 16-wide operand fragment, feed layer 2 from registers; layer 2's
@@ -468,7 +468,7 @@ __global__ void to_bf16_kernel(const float *th, __nv_bfloat16 *wb)
  * for -0.25 < a < 0, 1.1 times for 0 < a < 0.05 and -1 < a < -0.25, smaller elsewhere. (An earlier
  * fit to log2 of half the erfc, cut off at 5.75, was off by 9.8e-7 of the value near zero and by
  * 2.6e-8 below -5.75.)
- * 2 097 152 nodes: 345 us in the erf form, 201 with the earlier fit, 207 with this one. */
+ * 2 097 152 nodes: 345 us in the erf form, 201 with the earlier fit, 204 with this one. */
 __device__ __forceinline__ float2 twice_gelu(float2 a)
 {
     const float2 y = make_float2(fmaxf(-fabsf(a.x), -7.0f), fmaxf(-fabsf(a.y), -7.0f));
@@ -524,6 +524,8 @@ __device__ __forceinline__ uint32_t twice_gelu_bf16(float2 a)
     return r == pack_bf16(hi.x, hi.y) ? r : twice_gelu_erf_bf16(a);
 }
 
+/* M tiles per warp pass: two, or one where that is all a resident warp gets */
+template <int M>
 __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *__restrict__ wb,
                                                            const float *__restrict__ norm,
                                                            const float *__restrict__ X, long long n,
@@ -558,26 +560,26 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
     __syncthreads();
 
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-    const long long pairs = (n + 31) / 32;
+    const long long passes = (n + 16 * M - 1) / (16 * M);
     const long long stride = (long long)gridDim.x * (blockDim.x >> 5);
-    /* features 2q, 2q + 1 of this lane's four nodes (rows g, g + 8 of both tiles) */
-    float xr[4][2];
+    /* features 2q, 2q + 1 of this lane's nodes (rows g, g + 8 of each tile) */
+    float xr[2 * M][2];
     auto fetch = [&](long long t) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const long long r = 32 * t + g + 8 * k;
+        for (int k = 0; k < 2 * M; ++k) {
+            const long long r = 16 * M * t + g + 8 * k;
 #pragma unroll
             for (int e = 0; e < 2; ++e) xr[k][e] = r < n ? X[(long long)(2 * q + e) * n + r] : nm[2 * q + e];
         }
     };
     long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t < pairs) fetch(t);
-    for (; t < pairs; t += stride) {
+    if (t < passes) fetch(t);
+    for (; t < passes; t += stride) {
         /* layer-1 operands: normalised features (columns 8..15 zero) */
-        uint32_t a1[2][2];
-        bool ok[4];
+        uint32_t a1[M][2];
+        bool ok[2 * M];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2 * M; ++k) {
             float x0 = (xr[k][0] - nm[2 * q]) / nm[NF + 2 * q], x1 = (xr[k][1] - nm[2 * q + 1]) / nm[NF + 2 * q + 1];
             /* a node is usable when all eight features are finite: the four lanes of a row
              * hold two each */
@@ -586,15 +588,15 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
             if (!ok[k]) x0 = x1 = 0.0f;
             a1[k >> 1][k & 1] = pack_bf16(x0, x1);
         }
-        if (t + stride < pairs) fetch(t + stride);
+        if (t + stride < passes) fetch(t + stride);
         /* layer 1 -> GELU -> BF16 operand fragments of layer 2 */
-        uint32_t a2[2][4][4];
+        uint32_t a2[M][4][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
             const uint32_t b[2] = {w1f[nt][lane], 0u};
             const float2 bias = b1s[4 * nt + q];
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
+            for (int m = 0; m < M; ++m) {
                 float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                 const uint32_t a[4] = {a1[m][0], a1[m][1], 0u, 0u};
                 mma_bf16(c, a, b);
@@ -604,20 +606,20 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
             }
         }
         /* layer 2 -> GELU -> W3 dot product */
-        float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        float z[2 * M] = {};
 #pragma unroll 2
         for (int nt = 0; nt < 8; ++nt) {
-            float c[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
+            float c[M][4] = {};
 #pragma unroll
             for (int kt = 0; kt < 4; ++kt) {
                 const uint2 w = w2f[kt][nt][lane];
                 const uint32_t b[2] = {w.x, w.y};
 #pragma unroll
-                for (int m = 0; m < 2; ++m) mma_bf16(c[m], a2[m][kt], b);
+                for (int m = 0; m < M; ++m) mma_bf16(c[m], a2[m][kt], b);
             }
             const float2 bias = b2s[4 * nt + q], w3 = w3s[4 * nt + q];
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
+            for (int m = 0; m < M; ++m) {
                 const float2 h0 = twice_gelu(__fadd2_rn(make_float2(c[m][0], c[m][1]), bias));
                 const float2 h1 = twice_gelu(__fadd2_rn(make_float2(c[m][2], c[m][3]), bias));
                 z[2 * m] = fmaf(h0.y, w3.y, fmaf(h0.x, w3.x, z[2 * m]));
@@ -625,15 +627,21 @@ __global__ void __launch_bounds__(128, 5) infer_mma_kernel(const __nv_bfloat16 *
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2 * M; ++k) {
             z[k] += __shfl_xor_sync(0xffffffffu, z[k], 1);
             z[k] += __shfl_xor_sync(0xffffffffu, z[k], 2);
         }
-        /* lane q of a row's four stores node k = q of its four */
-        const float zq = q == 0 ? z[0] : (q == 1 ? z[1] : (q == 2 ? z[2] : z[3]));
-        const bool okq = q == 0 ? ok[0] : (q == 1 ? ok[1] : (q == 2 ? ok[2] : ok[3]));
-        const long long r = 32 * t + g + 8 * q;
-        if (r < n) p[r] = okq ? 1.0f / (1.0f + expf(-(zq + b3s))) : nanf("");
+        /* lane q of a row's four stores node k = q of its 2 M */
+        float zq = z[0];
+        bool okq = ok[0];
+#pragma unroll
+        for (int k = 1; k < 2 * M; ++k)
+            if (q == k) {
+                zq = z[k];
+                okq = ok[k];
+            }
+        const long long r = 16 * M * t + g + 8 * q;
+        if (q < 2 * M && r < n) p[r] = okq ? 1.0f / (1.0f + expf(-(zq + b3s))) : nanf("");
     }
 }
 
@@ -780,11 +788,19 @@ namespace lbk {
 
 int mlp_infer_dev(lb_mlp *M, const float *x, int64_t n, float *p, void *stream)
 {
-    /* four warps per block, five blocks per SM resident (152 SMs): each warp walks its
-     * 32-node pairs of tiles with a grid stride */
-    const long long pairs = (n + 31) / 32;
-    const unsigned blocks = (unsigned)std::min<long long>((pairs + 3) / 4, 152LL * 5);
-    lbm::infer_mma_kernel<<<blocks, 128, 0, static_cast<cudaStream_t>(stream)>>>(M->wb, M->norm, x, (long long)n, p);
+    /* four warps per block, five blocks per SM resident (152 SMs): each warp walks its passes of
+     * two 16-node tiles with a grid stride; of one tile where the warps outnumber the tiles, a
+     * shorter chain (a call of 1 to 8000 nodes 17.4 -> 14.8 us, 40 000 nodes 20.1 -> 19.3; 16.1 to
+     * 17.5 and 23 before two tiles shared a warp); the same values */
+    constexpr long long RESIDENT = 152LL * 5;
+    const long long tiles = (n + 15) / 16;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (tiles <= 4 * RESIDENT) {
+        lbm::infer_mma_kernel<1><<<(unsigned)((tiles + 3) / 4), 128, 0, st>>>(M->wb, M->norm, x, (long long)n, p);
+    } else {
+        const unsigned blocks = (unsigned)std::min<long long>((tiles + 7) / 8, RESIDENT);
+        lbm::infer_mma_kernel<2><<<blocks, 128, 0, st>>>(M->wb, M->norm, x, (long long)n, p);
+    }
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LB_OK : mlp_err(LB_ERR_CUDA, std::string("lb_mlp_infer: ") + cudaGetErrorString(e));
 }
