@@ -365,9 +365,10 @@ typedef struct lb_batch lb_batch;
  * without oscillation (omega = 0) and no pressure sides (else LB_ERR_INVALID, checked
  * before any device work). The kernel runs on opts[0].stream; device memory comes from
  * opts[0]'s allocator. Lattices start from rest (rho0, u = 0). Lattices that fit a block's
- * shared memory are bundled and stay there for all steps of a launch; else FP32 and 16-bit
- * batches run on layout 10's rows, and for FP64 lb_batch_create times block sizes 128 / 256 /
- * 512 on the batch and keeps the fastest. */
+ * shared memory are bundled and stay there for all steps of a launch; else, and in calls of a
+ * few steps where that is faster (timed at creation), FP32 and 16-bit batches run on layout
+ * 10's rows; for FP64 block sizes 128 / 256 / 512 are timed on the batch when it first needs
+ * one and the fastest kept. */
 int lb_batch_create(int32_t n, const lb_grid *grids, const uint8_t *const *maps, const int32_t sets[2],
                     const lb_kn *kn, const lb_wall *walls, const lb_opts *opts, lb_batch **out);
 /* Every lattice nsteps steps: one persistent launch. Asynchronous. */
